@@ -82,7 +82,7 @@ enum {
 
 /* arithmetic of the two big contractions (R = Phi^T L_g and M = R Theta) */
 enum {
-    AFQMC_PRECISION_FP64 = 0,  /* FP64 everywhere.  N <= 256, n_up <= 64, n_up^2 + n_dn^2 <= 4096, and
+    AFQMC_PRECISION_FP64 = 0,  /* FP64 everywhere, or exact integer products no less accurate.  N <= 256, n_up <= 64, n_up^2 + n_dn^2 <= 4096, and
                                   3 N n_up <= 25600 (e.g. N = 200 with 40 + 40 electrons) */
     AFQMC_PRECISION_BF16X3 = 1, /* the fused contraction on the tensor cores in split BF16 (hi*hi + hi*lo +
                                    lo*hi, FP32 accumulation, traces summed in FP64); trial orbitals, proposal
@@ -206,9 +206,10 @@ void afqmc_config_default(afqmc_config* cfg);
 
 /* Bytes of device workspace the configuration needs (0 if cfg is invalid).  Besides
  * the state and per-pair buffers it holds, for the walker-side contraction forms,
- * Y_g = L_g phi_w of every walker: (n_chol + 1) N 2 (n_up + n_dn) doubles per walker
- * in FP64 (4 MB per walker on the 50-orbital system), or the split-FP16 images
- * of it (6.2 MB per walker there). */
+ * Y_g = L_g phi_w: in FP64 (n_chol + 1) N 2 (n_up + n_dn) 64-bit integers per walker
+ * of a chunk and the digits of the chunk's pairs (about 4 GB at most) and of h and
+ * L_g (16 MB on the 50-orbital system, 1.1 GB at 200 orbitals), or the split-FP16 images
+ * of it (6.2 MB per walker on the 50-orbital system). */
 size_t afqmc_workspace_bytes(const afqmc_config* cfg);
 
 /* Create a context.
@@ -356,8 +357,16 @@ int64_t afqmc_launch_count(void);
  * 5 contract_tcw_kernel (tensor cores, general walker-side form B_p^T (X_g phi_w),
  * N <= 256, n_up <= 64: see tc_form), 6 contract_fp64c_kernel (precision FP64 with
  * complex trial samples: R_g = Phi^dagger X_g);
- * -1 if `cfg` is NULL or no kernel supports its sizes.  Host only. */
+ * -1 if `cfg` is NULL or no kernel supports its sizes.  Host only.  For precision
+ * FP64 with rcache = 0 the value names the FP64 arithmetic's kernel of these sizes
+ * (0, 3 or 6); where afqmc_fp64_digits says so, contract_fp64d_kernel runs in its
+ * place: the walker-side form B_p^T (X_g phi_w) on the tensor cores, every product
+ * as exact sums of integer digits, no less accurate than FP64 sums. */
 int afqmc_contract_kernel(const afqmc_config* cfg);
+/* 1 if the FP64 contraction of `cfg` runs on the tensor cores as integer digit
+ * products (N <= 224 and up to about 60 electrons per spin, 48 above 64 orbitals;
+ * precision FP64, rcache = 0), else 0.  Host only. */
+int afqmc_fp64_digits(const afqmc_config* cfg);
 
 /* Local energies, force-bias values and overlaps of a batch of (walker, trial
  * sample) pairs that allocates nothing.  The paper has no counterpart: this is

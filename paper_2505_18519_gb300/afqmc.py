@@ -52,7 +52,7 @@ EXPORTS = ("afqmc_config_default", "afqmc_workspace_bytes", "afqmc_init", "afqmc
            "afqmc_energy",
            "afqmc_energy_paths", "afqmc_observables", "afqmc_history", "afqmc_stats", "afqmc_state_save", "afqmc_state_load",
            "afqmc_destroy", "afqmc_last_error", "afqmc_philox_fill", "afqmc_profile", "afqmc_profile_read",
-           "afqmc_launch_count", "afqmc_contract_kernel", "afqmc_autotune", "afqmc_batch_create", "afqmc_batch_step", "afqmc_batch_sync",
+           "afqmc_launch_count", "afqmc_contract_kernel", "afqmc_fp64_digits", "afqmc_autotune", "afqmc_batch_create", "afqmc_batch_step", "afqmc_batch_sync",
            "afqmc_batch_destroy", "afqmc_mlp_n_params", "afqmc_mlp_params", "afqmc_mlp_eval", "afqmc_mlp_state",
            "afqmc_fp64_fma_rate", "afqmc_local_energy_noalloc", "afqmc_noalloc_scratch_bytes",
            "afqmc_noalloc_last_error", "afqmc_trial_orbitals", "afqmc_batch_shared_contractions")
@@ -112,6 +112,8 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.afqmc_launch_count.restype = ctypes.c_int64
     lib.afqmc_contract_kernel.argtypes = [ctypes.c_void_p]
     lib.afqmc_contract_kernel.restype = ctypes.c_int
+    lib.afqmc_fp64_digits.argtypes = [ctypes.c_void_p]
+    lib.afqmc_fp64_digits.restype = ctypes.c_int
     lib.afqmc_autotune.argtypes = [P, P]
     lib.afqmc_autotune.restype = I
     lib.afqmc_batch_create.argtypes = [I, P, P, ctypes.POINTER(P)]
@@ -422,6 +424,11 @@ def contract_kernel(cfg: AfqmcConfig) -> str:
     if k not in CONTRACT_KERNELS:
         raise AfqmcError(1, "no contraction kernel supports these sizes")
     return CONTRACT_KERNELS[k]
+
+
+def fp64_digits(cfg: AfqmcConfig) -> bool:
+    """Whether ``cfg``'s FP64 contraction runs on the tensor cores (exact integer digit products)."""
+    return bool(load_library().afqmc_fp64_digits(ctypes.byref(cfg)))
 
 
 def fp64_fma_rate(stream=None) -> float:

@@ -61,6 +61,11 @@ extern "C" int afqmc_contract_kernel(const afqmc_config* cfg) {
     return tc_kind(cfg);
 }
 
+extern "C" int afqmc_fp64_digits(const afqmc_config* cfg) {
+    return cfg && cfg->precision == AFQMC_PRECISION_FP64 && !cfg->rcache && cfg->n_paths >= 1 && cfg->n_walkers >= 1 &&
+           contract_fp64d_supported(cfg->N, cfg->n_up, cfg->n_dn, cfg->n_chol, cfg->n_walkers, cfg->n_paths);
+}
+
 // operand arithmetic of the walker-side tensor-core form: 0 bf16x3, 1 fp16x3, 2 fp16x6
 static int tc_mode(const afqmc_config* c) {
     return c->precision == AFQMC_PRECISION_FP16X6 ? 2 : (c->precision == AFQMC_PRECISION_FP16X3 ? 1 : 0);
@@ -342,9 +347,13 @@ static size_t layout(const afqmc_config* c, char* base, Workspace* ws) {
     w.Lt = (tck == 1 || tck == 2) ? take(contract_tc_image_bytes(d.N, d.nu, d.nd, d.G, f16c)) : nullptr;
     w.Yimg = tck == 2 ? take(contract_tcy_yimage_bytes(d.N, d.nu, d.nd, d.G, d.W, f16c)) : nullptr;
     w.tcw = tck == 5 ? take(contract_tcw_work_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P, tc_mode(c))) : nullptr;
-    const size_t ywalk = c->precision == AFQMC_PRECISION_FP64 ? contract_fp64_walker_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P)
-                                                              : 0;
-    w.ywalk = ywalk ? take(ywalk) : nullptr;
+    // FP64: the digit form's work space where it takes the sizes, else the walker-side form's
+    if (c->precision == AFQMC_PRECISION_FP64) {
+        const size_t fd = contract_fp64d_work_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P);
+        const size_t ywalk = fd ? 0 : contract_fp64_walker_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P);
+        w.fd = fd ? take(fd) : nullptr;
+        w.ywalk = ywalk ? take(ywalk) : nullptr;
+    }
     w.phi = (double2*)take(W * N * nt * 16);
     w.weight = (double*)take(W * 8);
     w.x = (double*)take(pairs * K * 8);
@@ -589,8 +598,10 @@ static afqmc_status measure(afqmc_ctx* ctx, int part = 0) {
     const bool f16 = ctx->cfg.precision == AFQMC_PRECISION_FP16X3;
     const bool fp64 = ctx->cfg.precision == AFQMC_PRECISION_FP64;
     const int tck = fp64 ? -1 : tc_kind(&ctx->cfg);
-    const int ovl = fp64 ? (!w.rc && !d.cphi && contract_fp64_walker_side(d.N, d.nu, d.nd, d.P) ? OVL_INVERSE : OVL_THETA)
-                         : (tck == 2 || tck == 5 ? OVL_TRIAL : OVL_THETA);
+    const bool digits = w.fd && !w.rc;
+    const int ovl = digits ? OVL_TRIAL
+                    : fp64 ? (!w.rc && !d.cphi && contract_fp64_walker_side(d.N, d.nu, d.nd, d.P) ? OVL_INVERSE : OVL_THETA)
+                           : (tck == 2 || tck == 5 ? OVL_TRIAL : OVL_THETA);
     if (part == 2) {
         CK(contract_tcw_finish(s, d, w.tcw, w.vpair, w.epair, tc_mode(&ctx->cfg)));
     } else {
@@ -614,6 +625,8 @@ static afqmc_status measure(afqmc_ctx* ctx, int part = 0) {
                             w.Phidf != nullptr));
         else
             CK(contract_tc(s, d, w.Lt, w.Phi, w.Theta, w.phi, w.Yimg, w.vpair, w.epair, w.status, f16));
+    } else if (digits) {
+        CK(contract_fp64d(s, d, w.fd, w.Theta, w.phi, w.vpair, w.epair, w.status));
     } else if (w.rc) {   // cached half-rotated matrices, refreshed for the paths that moved
         CK(rcache_refresh(s, d, w.h, w.Phi, w.rdirty, w.rlist, w.rcount, w.rc, w.counters));
         CK(contract_fp64r(s, d, w.rc, w.Theta, w.vpair, w.epair));
@@ -704,6 +717,10 @@ extern "C" afqmc_status afqmc_init_trial(const afqmc_config* cfg, const double* 
         if (e == cudaSuccess) e = cudaMemsetAsync(w.status, 0, 4, s);
         if (e != cudaSuccess) { st = fail(AFQMC_ERR_CUDA, "copying inputs: %s", cudaGetErrorString(e)); break; }
         StepParams p = params_of(cfg);
+        if (w.fd && (e = contract_fp64d_prepare(s, d, w.h, w.L, w.fd)) != cudaSuccess) {
+            st = fail(AFQMC_ERR_CUDA, "digits of h and L: %s", cudaGetErrorString(e));
+            break;
+        }
         if (w.tcw && (e = contract_tcw_prepare(s, d, w.h, w.L, w.tcw, tc_mode(cfg))) !=
                          cudaSuccess) {
             st = fail(AFQMC_ERR_CUDA, "tensor-core operand image: %s", cudaGetErrorString(e));

@@ -162,6 +162,7 @@ struct Workspace {
     void* Lt;           // split-BF16 image of (h, L_g) for the tensor-core contraction
     void* Yimg;         // split images of Y_g = X_g phi_w per walker (walker-side tensor-core form)
     void* tcw;          // work of the general walker-side tensor-core form (contract_tcw.cu)
+    void* fd;           // work of the FP64 digit form (contract_fp64d.cu)
     void* ywalk;        // Y_g = X_g phi_w of every walker, and the walkers' orbitals as columns (walker-side FP64 form)
     // composite walkers
     double2* phi;     // W*N*nt (nt = n_up + n_dn)

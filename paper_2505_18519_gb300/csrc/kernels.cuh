@@ -153,6 +153,17 @@ size_t contract_fp64_walker_bytes(int N, int nu, int nd, int G, long long W, int
 cudaError_t contract_fp64_walker(cudaStream_t s, const Dims& d, const double* h, const double* L, const double* Phi,
                                  const double2* Ainv, const double2* phi, void* work, double2* vpair, double2* epair);
 
+// contract_fp64d.cu: the FP64 contraction on the tensor cores (exact integer digit
+// products of FP64 accuracy): Z_{p,g} = B_p^T (X_g phi_w), B_p = Phi_p A_p^-T from
+// overlap_lu with OVL_TRIAL, real or complex trial samples.  N <= 224, n_up <= about
+// 60 (the digits of a column tile in shared memory).  work: contract_fp64d_work_bytes
+// bytes; contract_fp64d_prepare fills the digits of h and L once.
+bool contract_fp64d_supported(int N, int nu, int nd, int G, long long W, int P);
+size_t contract_fp64d_work_bytes(int N, int nu, int nd, int G, long long W, int P);
+cudaError_t contract_fp64d_prepare(cudaStream_t st, const Dims& d, const double* h, const double* L, void* work);
+cudaError_t contract_fp64d(cudaStream_t st, const Dims& d, void* work, const double2* Bm, const double2* phi,
+                           double2* vpair, double2* epair, int* status);
+
 // contract_tc.cu
 bool contract_tc_supported(int N, int nu, int nd, bool f16);
 size_t contract_tc_image_bytes(int N, int nu, int nd, int G, bool f16);
