@@ -878,7 +878,7 @@ __global__ void __launch_bounds__(TCY_THREADS, 1)
     __shared__ double2 eacc[2][TCY_MAXPG];
     __shared__ int sA[128];
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int quarter = warp & 3, half = (warp >> 2) & 1;
     const int bpw = (P + PG - 1) / PG;
     const long long w = blockIdx.x / bpw;
@@ -944,42 +944,46 @@ __global__ void __launch_bounds__(TCY_THREADS, 1)
     bool failed = false;
 
     if (warp == 8) {
-        // ---- producer (one thread)
-        if (lane == 0) {
-            int loaded = 0, consumed = 0;
-            auto load = [&](int st, int v) {
+        // ---- producer and MMA issue: one lane's copies and MMAs, the loop warp-uniform (waits agreed
+        // by a vote), so that the MMAs' operands come from uniform registers
+        int loaded = 0, consumed = 0;
+        auto wait = [&](uint64_t* bar, int phase) { return __all_sync(0xffffffffu, tc::mbar_wait(bar, (uint32_t)(phase & 1), lim)) != 0; };
+        auto load = [&](int st, int v) {
+            if (lane == 0) {
                 tc::mbar_arrive_expect_tx(&full_bar[st], unit_bytes);
                 tc::bulk_g2s(YR + (size_t)st * unit_bytes, ysrc + (size_t)v * unit_bytes, unit_bytes, &full_bar[st]);
-            };
-            for (; loaded < S && loaded < n_units; ++loaded) load(loaded, loaded);
-            for (int u = 0; u < n_units && !failed; ++u) {
-                const int b = u % nbuf, st = u % S;
-                // unit u not loaded yet (a one-stage ring): its stage frees when GEMM-M of unit u - S completes
-                while (loaded <= u) {
-                    const int v = loaded - S, sv = loaded % S;
-                    if (v >= 0 && !tc::mbar_wait(&empty_bar[sv], (uint32_t)((v / S) & 1), lim)) { failed = true; break; }
-                    load(sv, loaded);
-                    ++loaded;
-                }
-                if (failed) break;
-                // D_M buffer b is free once the epilogue of unit u - nbuf has read it
-                if (u >= nbuf && !tc::mbar_wait(&mempty[b], (uint32_t)((u / nbuf - 1) & 1), lim)) { failed = true; break; }
-                if (!tc::mbar_wait(&full_bar[st], (uint32_t)((u / S) & 1), lim)) { failed = true; break; }
-                tc::fence_after_sync();
-                ++consumed;
-                // both matrices of the unit in one operand of 2 NBY rows; D columns of buffer b:
-                // [matrix 0 | matrix 1] then (FP16) their corrections
-                const uint8_t* byh = YR + (size_t)st * unit_bytes;
-                const uint8_t* byl = byh + 2 * by_bytes;
-                const uint32_t d = taddr + (uint32_t)b * 2u * dms;
+            }
+            __syncwarp();
+        };
+        const uint64_t amh = tc::desc_sw128(tc::smem_u32(AMh)), aml = tc::desc_sw128(tc::smem_u32(AMl));
+        const uint64_t yr0 = tc::desc_sw128(tc::smem_u32(YR));
+        for (; loaded < S && loaded < n_units; ++loaded) load(loaded, loaded);
+        for (int u = 0; u < n_units && !failed; ++u) {
+            const int b = u % nbuf, st = u % S;
+            // unit u not loaded yet (a one-stage ring): its stage frees when GEMM-M of unit u - S completes
+            while (loaded <= u) {
+                const int v = loaded - S, sv = loaded % S;
+                if (v >= 0 && !wait(&empty_bar[sv], v / S)) { failed = true; break; }
+                load(sv, loaded);
+                ++loaded;
+            }
+            if (failed) break;
+            // D_M buffer b is free once the epilogue of unit u - nbuf has read it
+            if (u >= nbuf && !wait(&mempty[b], u / nbuf - 1)) { failed = true; break; }
+            if (!wait(&full_bar[st], u / S)) { failed = true; break; }
+            tc::fence_after_sync();
+            ++consumed;
+            // both matrices of the unit in one operand of 2 NBY rows; D columns of buffer b:
+            // [matrix 0 | matrix 1] then (FP16) their corrections
+            const uint64_t byh = yr0 + (uint64_t)((uint32_t)st * (unit_bytes >> 4)), byl = byh + (uint64_t)((2u * by_bytes) >> 4);
+            const uint32_t d = taddr + (uint32_t)b * 2u * dms;
+            __syncwarp();
+            if (tc::elect_one()) {
 #pragma unroll
                 for (int s = 0; s < 8; ++s) {
-                    const uint32_t ka = (uint32_t)((s >> 2) * 128 * 128 + (s & 3) * 32);
-                    const uint32_t kbo = (uint32_t)((s >> 2) * 2 * NBY * 128 + (s & 3) * 32);
-                    const uint64_t ah = tc::desc_sw128(tc::smem_u32(AMh) + ka),
-                                   al = tc::desc_sw128(tc::smem_u32(AMl) + ka);
-                    const uint64_t bh = tc::desc_sw128(tc::smem_u32(byh) + kbo),
-                                   bl = tc::desc_sw128(tc::smem_u32(byl) + kbo);
+                    const uint32_t ka = (uint32_t)((s >> 2) * 128 * 128 + (s & 3) * 32) >> 4;
+                    const uint32_t kbo = (uint32_t)((s >> 2) * 2 * NBY * 128 + (s & 3) * 32) >> 4;
+                    const uint64_t ah = amh + ka, al = aml + ka, bh = byh + kbo, bl = byl + kbo;
                     const uint32_t acc = s > 0 ? 1u : 0u;
                     tc::mma_f16(d, ah, bh, idd, acc);
                     if (F16) {
@@ -993,23 +997,24 @@ __global__ void __launch_bounds__(TCY_THREADS, 1)
                 }
                 tc::mma_commit(&empty_bar[st]);
                 tc::mma_commit(&mfull[b]);
-                // refill the stages whose MMAs (units up to u - 1) have completed
-                while (loaded < n_units && loaded - S <= u - 1) {
-                    const int v = loaded - S, sv = loaded % S;
-                    if (!tc::mbar_wait(&empty_bar[sv], (uint32_t)((v / S) & 1), lim)) { failed = true; break; }
-                    load(sv, loaded);
-                    ++loaded;
-                }
             }
-            if (failed) {
-                atomicOr(status, STATUS_TIMEOUT);
+            __syncwarp();
+            // refill the stages whose MMAs (units up to u - 1) have completed
+            while (loaded < n_units && loaded - S <= u - 1) {
+                const int v = loaded - S, sv = loaded % S;
+                if (!wait(&empty_bar[sv], v / S)) { failed = true; break; }
+                load(sv, loaded);
+                ++loaded;
             }
-            // drain: every issued copy and MMA completes before the block releases its memory
-            for (int v = max(consumed, loaded - S); v < loaded; ++v)
-                if (v >= 0) tc::mbar_wait(&full_bar[v % S], (uint32_t)((v / S) & 1), 1u << 22);
-            tc::mma_commit(&drain_bar);
-            tc::mbar_wait(&drain_bar, 0, 1u << 22);
         }
+        if (failed && lane == 0) atomicOr(status, STATUS_TIMEOUT);
+        // drain: every issued copy and MMA completes before the block releases its memory
+        for (int v = max(consumed, loaded - S); v < loaded; ++v)
+            if (v >= 0) tc::mbar_wait(&full_bar[v % S], (uint32_t)((v / S) & 1), 1u << 22);
+        __syncwarp();
+        if (tc::elect_one()) tc::mma_commit(&drain_bar);
+        __syncwarp();
+        tc::mbar_wait(&drain_bar, 0, 1u << 22);
         __syncwarp();
     } else {
         // ---- epilogue warps 0-7

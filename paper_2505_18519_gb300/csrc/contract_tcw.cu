@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(TCW_THREADS, 1)
     __shared__ volatile int fail;
     __shared__ int sPW[64];
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const long long wl0 = (long long)(blockIdx.x / n_gblk) * WPB;   // first walker of the block (in the chunk)
     const int nw = (int)min((long long)WPB, wb - wl0);              // walkers present
     const int gb = blockIdx.x % n_gblk;
@@ -311,14 +311,15 @@ __global__ void __launch_bounds__(TCW_THREADS, 1)
     if (warp == 0) {
         // ---- producer: unit v = (matrix g0 + v / (NP KCX), chunk (v / NP) % KCX, part v % NP)
         if (lane == 0) {
-            int issued = 0;
-            for (int v = 0; v < n_units; ++v) {
-                const int st = v % S;
-                if (v >= S && !wait_or_fail(&empty_bar[st], (uint32_t)(((v / S) - 1) & 1), lim, &fail)) { failed = true; break; }
-                const int g = g0 + v / (NP * KCX), c = (v / NP) % KCX, hh = v % NP;
+            int issued = 0, st = 0;
+            uint32_t ph = 1u;
+            const uint8_t* src = Ximg + (size_t)g0 * KCX * NP * RX;   // (matrix, chunk, part) follow one another
+            for (int v = 0; v < n_units; ++v, src += RX) {
+                if (v >= S && !wait_or_fail(&empty_bar[st], ph, lim, &fail)) { failed = true; break; }
                 tc::mbar_arrive_expect_tx(&full_bar[st], RX);
-                tc::bulk_g2s(ring + (size_t)st * RX, Ximg + (((size_t)g * KCX + c) * NP + hh) * RX, RX, &full_bar[st]);
+                tc::bulk_g2s(ring + (size_t)st * RX, src, RX, &full_bar[st]);
                 ++issued;
+                if (++st == S) { st = 0; ph ^= 1u; }
             }
             // every issued copy lands before the block leaves
             for (int v = max(0, issued - S); v < issued; ++v)
@@ -327,32 +328,35 @@ __global__ void __launch_bounds__(TCW_THREADS, 1)
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ---- MMA issue (one thread): D_Y = PW X_g^T, the part products of the header
-        if (lane == 0) {
-            const uint32_t idesc = F16 ? tc::idesc_f16_f32(128, N16) : tc::idesc_bf16_f32(128, N16);
-            int v = 0;
-            for (int gi = 0; gi < ng && !failed; ++gi) {
-                const int buf = gi % NBUF;
-                if (gi >= NBUF && !wait_or_fail(&dempty[buf], (uint32_t)(((gi / NBUF) - 1) & 1), lim, &fail)) {
-                    failed = true;
-                    break;
-                }
-                tc::fence_after_sync();
-                const uint32_t dh = taddr + (uint32_t)buf * tcols, dl = dh + (F16 ? (uint32_t)N16 : 0u);
-                for (int c = 0; c < KCX && !failed; ++c) {
-                    const int ks = min(4, (N16 - 64 * c) / 16);
-                    for (int hh = 0; hh < NP; ++hh, ++v) {
-                        const int st = v % S;
-                        if (!wait_or_fail(&full_bar[st], (uint32_t)((v / S) & 1), lim, &fail)) { failed = true; break; }
-                        tc::fence_after_sync();
-                        const uint32_t pa = tc::smem_u32(PW + (size_t)c * CS);
-                        const uint32_t pb = tc::smem_u32(ring + (size_t)st * RX);
-                        for (int s = 0; s < ks; ++s) {
-                            const uint64_t a0 = tc::desc_sw128(pa + s * 32), a1 = tc::desc_sw128(pa + PS + s * 32);
-                            const uint64_t bx = tc::desc_sw128(pb + s * 32);
+        // ---- MMA issue (one lane, the loop warp-uniform as in GEMM-Z): D_Y = PW X_g^T, the part
+        // products of the header
+        const uint32_t idesc = F16 ? tc::idesc_f16_f32(128, N16) : tc::idesc_bf16_f32(128, N16);
+        const uint64_t abase = tc::desc_sw128(tc::smem_u32(PW)), bbase = tc::desc_sw128(tc::smem_u32(ring));
+        bool ok = true;
+        int st = 0;
+        uint32_t ph = 0;
+        for (int gi = 0; gi < ng; ++gi) {
+            const int buf = NBUF == 2 ? (gi & 1) : 0, use = NBUF == 2 ? (gi >> 1) : gi;
+            if (use > 0) ok &= wait_or_fail(&dempty[buf], (uint32_t)((use - 1) & 1), lim, &fail);
+            tc::fence_after_sync();
+            const uint32_t dh = taddr + (uint32_t)buf * tcols, dl = dh + (F16 ? (uint32_t)N16 : 0u);
+            for (int c = 0; c < KCX; ++c) {
+                const int ks = min(4, (N16 - 64 * c) / 16);
+#pragma unroll
+                for (int hh = 0; hh < NP; ++hh) {
+                    ok &= wait_or_fail(&full_bar[st], ph, lim, &fail);
+                    tc::fence_after_sync();
+                    const uint64_t pa = abase + (uint64_t)((uint32_t)c * (CS >> 4));
+                    const uint64_t pb = bbase + (uint64_t)((uint32_t)st * (RX >> 4));
+                    __syncwarp();
+                    if (tc::elect_one()) {
+#pragma unroll
+                        for (int s = 0; s < 4; ++s) {
+                            if (s >= ks) break;
+                            const uint64_t a0 = pa + 2 * s, a1 = a0 + (PS >> 4), bx = pb + 2 * s;
                             const uint32_t first = (c == 0 && s == 0) ? 0u : 1u;
                             if constexpr (MODE == 2) {
-                                const uint64_t a2 = tc::desc_sw128(pa + 2 * PS + s * 32);
+                                const uint64_t a2 = a0 + 2 * (PS >> 4);
                                 if (hh == 0) {                 // X hi: hi*hi, mid*hi, lo*hi
                                     tc::mma_f16(dh, a0, bx, idesc, first);
                                     tc::mma_f16(dl, a1, bx, idesc, first);
@@ -372,15 +376,18 @@ __global__ void __launch_bounds__(TCW_THREADS, 1)
                             }
                         }
                         tc::mma_commit(&empty_bar[st]);
+                        if (c == KCX - 1 && hh == NP - 1) tc::mma_commit(&dfull[buf]);
                     }
+                    __syncwarp();
+                    if (++st == S) { st = 0; ph ^= 1u; }
                 }
-                if (!failed) tc::mma_commit(&dfull[buf]);
             }
-            if (failed) atomicOr(status, STATUS_TIMEOUT);
-            tc::mma_commit(&drain_bar);                 // every issued MMA completes before the block leaves
-            tc::mbar_wait(&drain_bar, 0, 1u << 22);
         }
+        if (!ok && lane == 0) atomicOr(status, STATUS_TIMEOUT);
+        failed = !ok;
+        if (tc::elect_one()) tc::mma_commit(&drain_bar);        // every issued MMA completes before the block leaves
         __syncwarp();
+        tc::mbar_wait(&drain_bar, 0, 1u << 22);
     } else {
         // ---- epilogue (warps 2-5): lane r = (v, b, ri) of D_Y holds Re/Im Y_g[:, b] of walker v
         const int quarter = warp & 3;
@@ -623,7 +630,7 @@ __device__ __forceinline__ void tcw_z_block(const TcwZArgs& A, long long bid, ui
     int* sA = sh.sA;
     float* scl = sh.scl;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     const long long wl = bid / MT;
     const int m = (int)(bid % MT);
     const int np = min(PB, P - m * PB);
@@ -677,16 +684,17 @@ __device__ __forceinline__ void tcw_z_block(const TcwZArgs& A, long long bid, ui
                 for (int c = 0; c < KC; ++c)
                     tc::bulk_g2s(Ares + (size_t)c * CH, Atile + (size_t)c * CH, CH, &a_bar);
             }
-            int issued = 0;
-            for (int v = 0; v < n_units; ++v) {
-                const int st = v % S;
-                if (v >= S && !wait_or_fail(&empty_bar[st], (uint32_t)(((v / S) - 1) & 1), lim, &fail)) { failed = true; break; }
-                const int t = v / KC, c = v % KC;
+            int issued = 0, st = 0, c = 0;
+            uint32_t ph = 1u;
+            for (int v = 0; v < n_units; ++v) {               // counters, no division: the loop sets the ring's pace
+                if (v >= S && !wait_or_fail(&empty_bar[st], ph, lim, &fail)) { failed = true; break; }
                 uint8_t* dst = ring + (size_t)st * stage_bytes;
                 tc::mbar_arrive_expect_tx(&full_bar[st], stage_bytes);
                 if (!a_res) tc::bulk_g2s(dst, Atile + (size_t)c * CH, CH, &full_bar[st]);
-                tc::bulk_g2s(dst + (a_res ? 0 : CH), Ywalk + ((size_t)t * KC + c) * bbytes, bbytes, &full_bar[st]);
+                tc::bulk_g2s(dst + (a_res ? 0 : CH), Ywalk + (size_t)v * bbytes, bbytes, &full_bar[st]);
                 ++issued;
+                if (++c == KC) c = 0;
+                if (++st == S) { st = 0; ph ^= 1u; }
             }
             for (int v = max(0, issued - S); v < issued; ++v)
                 tc::mbar_wait(&full_bar[v % S], (uint32_t)((v / S) & 1), 1u << 22);
@@ -695,33 +703,40 @@ __device__ __forceinline__ void tcw_z_block(const TcwZArgs& A, long long bid, ui
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ---- MMA issue (one thread)
-        if (lane == 0) {
-            const uint32_t idesc = F16 ? tc::idesc_f16_f32(128, NT) : tc::idesc_bf16_f32(128, NT);
-            if (a_res && !wait_or_fail(&a_bar, 0, lim, &fail)) failed = true;
-            int committed = 0;   // units whose ring stage was handed back by a commit
-            for (int t = 0; t < NTILES && !failed; ++t) {
-                const int b = t & 1;
-                if (t >= 2 && !wait_or_fail(&dempty[b], (uint32_t)(((t >> 1) - 1) & 1), lim, &fail)) { failed = true; break; }
+        // ---- MMA issue: one lane's instructions, but the whole warp runs the loop without a
+        // divergent exit, so that the operands stay in the uniform registers the MMA takes them
+        // from (in a branch of one lane each MMA's operands were moved there first).  After a
+        // timeout the waits return at once; the block's results are void then.
+        const uint32_t idesc = F16 ? tc::idesc_f16_f32(128, NT) : tc::idesc_bf16_f32(128, NT);
+        const uint64_t abase = tc::desc_sw128(tc::smem_u32(a_res ? Ares : ring));
+        const uint64_t bbase = tc::desc_sw128(tc::smem_u32(ring + (a_res ? 0 : CH)));
+        const uint32_t sstep = stage_bytes >> 4, bstep = bpart >> 4;   // descriptors count 16-byte units
+        bool ok = !a_res || wait_or_fail(&a_bar, 0, lim, &fail);
+        int st = 0;
+        uint32_t ph = 0;
+        for (int t = 0; t < NTILES; ++t) {
+            const int b = t & 1;
+            if (t >= 2) ok &= wait_or_fail(&dempty[b], (uint32_t)(((t >> 1) - 1) & 1), lim, &fail);
+            const uint32_t dh = taddr + (uint32_t)b * dcols, dl = dh + (F16 ? (uint32_t)NT : 0u);
+            for (int c = 0; c < KC; ++c) {
+                ok &= wait_or_fail(&full_bar[st], ph, lim, &fail);
                 tc::fence_after_sync();
-                const uint32_t dh = taddr + (uint32_t)b * dcols, dl = dh + (F16 ? (uint32_t)NT : 0u);
-                for (int c = 0; c < KC; ++c) {
-                    const int v = t * KC + c, st = v % S;
-                    if (!wait_or_fail(&full_bar[st], (uint32_t)((v / S) & 1), lim, &fail)) { failed = true; break; }
-                    tc::fence_after_sync();
-                    const int ks = min(4, (KZ - 64 * c) / 16);
-                    const uint8_t* sbase = ring + (size_t)st * stage_bytes;
-                    const uint32_t pa = tc::smem_u32(a_res ? Ares + (size_t)c * CH : sbase);
-                    const uint32_t pb = tc::smem_u32(sbase + (a_res ? 0 : CH));
-                    for (int s = 0; s < ks; ++s) {
-                        const uint64_t a0 = tc::desc_sw128(pa + s * 32), a1 = tc::desc_sw128(pa + TCW_PART + s * 32);
-                        const uint64_t b0 = tc::desc_sw128(pb + s * 32), b1 = tc::desc_sw128(pb + bpart + s * 32);
-                        const uint32_t first = (c == 0 && s == 0) ? 0u : 1u;
+                const int ks = min(4, (KZ - 64 * c) / 16);
+                const uint64_t pa = abase + (uint64_t)(a_res ? (uint32_t)c * (CH >> 4) : (uint32_t)st * sstep);
+                const uint64_t pb = bbase + (uint64_t)((uint32_t)st * sstep);
+                const uint32_t firstc = c == 0 ? 0u : 1u;
+                __syncwarp();
+                if (tc::elect_one()) {
+#pragma unroll
+                    for (int s = 0; s < 4; ++s) {
+                        if (s >= ks) break;
+                        const uint64_t a0 = pa + 2 * s, a1 = a0 + (TCW_PART >> 4);
+                        const uint64_t b0 = pb + 2 * s, b1 = b0 + bstep;
+                        const uint32_t first = s == 0 ? firstc : 1u;
                         // products grouped by their A part, which the collector buffer keeps
                         // between them (each part read from shared memory once per K step)
                         if constexpr (MODE == 2) {
-                            const uint64_t a2 = tc::desc_sw128(pa + 2 * TCW_PART + s * 32),
-                                           b2 = tc::desc_sw128(pb + 2 * bpart + s * 32);
+                            const uint64_t a2 = a0 + 2 * (TCW_PART >> 4), b2 = b0 + 2 * bstep;
                             tc::mma_f16_ca<1>(dh, a0, b0, idesc, first);
                             tc::mma_f16_ca<2>(dl, a0, b1, idesc, first);
                             tc::mma_f16_ca<3>(dl, a0, b2, idesc, 1u);
@@ -740,18 +755,21 @@ __device__ __forceinline__ void tcw_z_block(const TcwZArgs& A, long long bid, ui
                         }
                     }
                     tc::mma_commit(&empty_bar[st]);
-                    ++committed;
+                    if (c == KC - 1) tc::mma_commit(&dfull[b]);
                 }
-                if (!failed) tc::mma_commit(&dfull[b]);
+                __syncwarp();
+                if (++st == S) { st = 0; ph ^= 1u; }
             }
-            if (failed) atomicOr(status, STATUS_TIMEOUT);
-            tc::mma_commit(&drain_bar);
-            tc::mbar_wait(&drain_bar, 0, 1u << 22);
-            // the ring's last hand-backs, which no producer wait consumed, have arrived
-            // (the barriers may be initialised again for the block's next piece of work)
-            for (int v = max(0, committed - S); v < committed; ++v)
-                tc::mbar_wait(&empty_bar[v % S], (uint32_t)((v / S) & 1), 1u << 22);
         }
+        if (!ok && lane == 0) atomicOr(status, STATUS_TIMEOUT);
+        failed = !ok;
+        if (tc::elect_one()) tc::mma_commit(&drain_bar);
+        __syncwarp();
+        tc::mbar_wait(&drain_bar, 0, 1u << 22);
+        // the ring's last hand-backs, which no producer wait consumed, have arrived
+        // (the barriers may be initialised again for the block's next piece of work)
+        for (int v = max(0, n_units - S); v < n_units; ++v)
+            tc::mbar_wait(&empty_bar[v % S], (uint32_t)((v / S) & 1), 1u << 22);
         __syncwarp();
     } else {
         // ---- epilogue (warps 2-9, two per tensor-memory lane quadrant): lane r = (p_l, a)

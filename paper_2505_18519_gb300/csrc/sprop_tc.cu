@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
 
     const long long p0 = (long long)blockIdx.x * SP_NB;
     const int np = (int)min((long long)SP_NB, M - p0);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform
     if (warp == 1) {
         tc::tmem_alloc(&tslot, SP_TALLOC);
         tc::tmem_relinquish();
@@ -184,47 +184,49 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ---- MMA issue (one thread)
-        if (lane == 0) {
-            int v = 0, committed = 0;
-            const uint32_t bbase = tc::smem_u32(BD), rbase = tc::smem_u32(ring);
-            for (int t = 0; t < NTILE && !failed; ++t) {
-                const int b = t & 1;
-                if (t >= 2 && !sp_wait(&dempty[b], (uint32_t)(((t >> 1) - 1) & 1), lim, &fail)) {
-                    failed = true;
-                    break;
-                }
-                tc::fence_after_sync();
-                const uint32_t dbase = taddr + (uint32_t)b * SP_DCOLS;
-                for (int i = 0; i < DG_DIG && !failed; ++i) {
-                    // digit i of U against the proposals' digits 0 .. 4 - i, into accumulators i .. 4
-                    const uint32_t idesc = tc::idesc_f16_f32(128, (SP_ORD - i) * SP_NB);
-                    for (int kb = 0; kb < KBLK; ++kb, ++v) {
-                        const int st = v % SP_STAGES;
-                        if (!sp_wait(&full_bar[st], (uint32_t)((v / SP_STAGES) & 1), lim, &fail)) {
-                            failed = true;
-                            break;
-                        }
-                        tc::fence_after_sync();
-                        const uint32_t pa = rbase + (uint32_t)st * SP_TILE, pb = bbase + (uint32_t)kb * SP_BKB;
+        // ---- MMA issue: one lane's instructions, the loop warp-uniform without a divergent exit, so
+        // that the operands stay in uniform registers; after a timeout the waits return at once
+        // (the block's results are void then)
+        const uint64_t bbase = tc::desc_sw128(tc::smem_u32(BD)), rbase = tc::desc_sw128(tc::smem_u32(ring));
+        bool ok = true;
+        int st = 0;
+        uint32_t ph = 0;
+        for (int t = 0; t < NTILE; ++t) {
+            const int b = t & 1;
+            if (t >= 2) ok &= sp_wait(&dempty[b], (uint32_t)(((t >> 1) - 1) & 1), lim, &fail);
+            tc::fence_after_sync();
+            const uint32_t dbase = taddr + (uint32_t)b * SP_DCOLS;
 #pragma unroll
-                        for (int s = 0; s < 4; ++s) {
-                            const uint32_t acc = (i == 0 && kb == 0 && s == 0) ? 0u : 1u;
-                            tc::mma_f16(dbase + (uint32_t)(i * SP_NB), tc::desc_sw128(pa + 32u * s),
-                                        tc::desc_sw128(pb + 32u * s), idesc, acc);
-                        }
+            for (int i = 0; i < DG_DIG; ++i) {
+                // digit i of U against the proposals' digits 0 .. 4 - i, into accumulators i .. 4
+                const uint32_t idesc = tc::idesc_f16_f32(128, (SP_ORD - i) * SP_NB);
+                for (int kb = 0; kb < KBLK; ++kb) {
+                    ok &= sp_wait(&full_bar[st], ph, lim, &fail);
+                    tc::fence_after_sync();
+                    const uint64_t pa = rbase + (uint64_t)((uint32_t)st * (SP_TILE >> 4));
+                    const uint64_t pb = bbase + (uint64_t)((uint32_t)kb * (SP_BKB >> 4));
+                    __syncwarp();
+                    if (tc::elect_one()) {
+#pragma unroll
+                        for (int s = 0; s < 4; ++s)
+                            tc::mma_f16(dbase + (uint32_t)(i * SP_NB), pa + 2 * s, pb + 2 * s, idesc,
+                                        (i == 0 && kb == 0 && s == 0) ? 0u : 1u);
                         tc::mma_commit(&empty_bar[st]);
-                        ++committed;
+                        if (i == DG_DIG - 1 && kb == KBLK - 1) tc::mma_commit(&dfull[b]);
                     }
+                    __syncwarp();
+                    if (++st == SP_STAGES) { st = 0; ph ^= 1u; }
                 }
-                if (!failed) tc::mma_commit(&dfull[b]);
             }
-            if (failed) atomicOr(status, STATUS_TIMEOUT);
-            tc::mma_commit(&drain_bar);                  // every issued MMA completes before the block leaves
-            tc::mbar_wait(&drain_bar, 0, 1u << 22);
-            for (int u = max(0, committed - SP_STAGES); u < committed; ++u)
-                tc::mbar_wait(&empty_bar[u % SP_STAGES], (uint32_t)((u / SP_STAGES) & 1), 1u << 22);
         }
+        if (!ok && lane == 0) atomicOr(status, STATUS_TIMEOUT);
+        failed = !ok;
+        if (tc::elect_one()) tc::mma_commit(&drain_bar);         // every issued MMA completes before the block leaves
+        __syncwarp();
+        tc::mbar_wait(&drain_bar, 0, 1u << 22);
+        const int units = NTILE * DG_DIG * KBLK;
+        for (int u = max(0, units - SP_STAGES); u < units; ++u)
+            tc::mbar_wait(&empty_bar[u % SP_STAGES], (uint32_t)((u / SP_STAGES) & 1), 1u << 22);
         __syncwarp();
     } else {
         // ---- epilogue (warps 2-9): lane r = column e = 128 t + r of the tile; half h of the

@@ -79,12 +79,18 @@ __device__ __forceinline__ void mbar_fence_init() { asm volatile("fence.mbarrier
 __device__ __forceinline__ void mbar_inval(uint64_t* bar) {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// Wait for the phase with parity `parity` to complete, at most `limit` polls.
+// Wait for the phase with parity `parity` to complete, at most `limit` polls: the
+// first only looks, the others may suspend the thread for a while.
 // Returns false if it gave up (the caller records an error and stops).
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit = (1u << 26)) {
-    uint32_t addr = smem_u32(bar);
-    for (uint32_t it = 0; it < limit; ++it) {
-        uint32_t done;
+    uint32_t addr = smem_u32(bar), done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(addr), "r"(parity)
+        : "memory");
+    if (done) return true;
+    for (uint32_t it = 1; it < limit; ++it) {
         asm volatile(
             "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
             : "=r"(done)

@@ -280,6 +280,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
     const long long prob = blockIdx.x;
     if (alive && !alive[prob / P]) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int warp_u = __shfl_sync(0xffffffffu, warp, 0);   // the same, known to be uniform
     const int quad = warp & 3;
     const int row = 32 * quad + lane;                    // row i of S V owned by this thread
     const int col0 = (warp >> 2) * CPT;                  // its first column a
@@ -433,24 +434,30 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
     bool grew = false, failed = false;
     int k = 1;
     for (; k <= m; ++k) {
-        // 3a. the products S' V_{k-1}
-        if (tid == 0) {
+        // 3a. the products S' V_{k-1}: one lane issues them, chosen in a converged warp (warp_u),
+        // so that the operands come from uniform registers (a branch of one thread moved each
+        // MMA's operands there first, which took longer than the MMA)
+        if (warp_u == 0) {
             tc::fence_after_sync();
-            const uint32_t sbase = tc::smem_u32(SD), vbase = tc::smem_u32(VD);
+            const uint64_t sd0 = tc::desc_sw128(tc::smem_u32(SD)), vd0 = tc::desc_sw128(tc::smem_u32(VD));
+            __syncwarp();
+            if (tc::elect_one()) {
 #pragma unroll
-            for (int i = 0; i < TT_DIG; ++i) {
+                for (int i = 0; i < TT_DIG; ++i) {
 #pragma unroll
-                for (int kb = 0; kb < KB; ++kb) {
+                    for (int kb = 0; kb < KB; ++kb) {
 #pragma unroll
-                    for (int s = 0; s < 4; ++s) {
-                        const uint64_t ad = tc::desc_sw128(sbase + (uint32_t)i * TT_SDIG + (uint32_t)kb * TT_SKB + 32u * s);
-                        const uint64_t bd = tc::desc_sw128(vbase + (uint32_t)kb * VKB + 32u * s);
-                        const bool first = i == 0 && kb == 0 && s == 0;
-                        tc::mma_f16(taddr + (uint32_t)(i * NB), ad, bd, idesc[i], first ? 0u : 1u);
+                        for (int s = 0; s < 4; ++s) {
+                            const uint64_t ad = sd0 + (uint64_t)((uint32_t)i * (TT_SDIG >> 4) + (uint32_t)kb * (TT_SKB >> 4) + 2u * s);
+                            const uint64_t bd = vd0 + (uint64_t)((uint32_t)kb * (VKB >> 4) + 2u * s);
+                            const bool first = i == 0 && kb == 0 && s == 0;
+                            tc::mma_f16(taddr + (uint32_t)(i * NB), ad, bd, idesc[i], first ? 0u : 1u);
+                        }
                     }
                 }
+                tc::mma_commit(&mma_bar);
             }
-            tc::mma_commit(&mma_bar);
+            __syncwarp();
         }
         const bool ok = tc::mbar_wait(&mma_bar, (uint32_t)((k - 1) & 1), lim);
         if (__syncthreads_or(!ok)) {
