@@ -236,6 +236,18 @@ static bool refine_enabled(const afqmc_config* c) {
     return (k == 1 || k == 5) && contract_fp64_supported(c->N, c->n_up, c->n_dn);
 }
 
+// ... as integer digit products on the tensor cores above 128 orbitals.  There the double-float
+// kernel takes 2.4 ms per pair and as long for one pair as for nine (200 orbitals, 40 + 40 electrons:
+// 390 ms for the 165 of 512 pairs listed, the digits 75 ms, Y of their walkers included).  Below, lists are short, and the kernel's
+// runs of matrices fill the chip with a few pairs, where the digits start with Y of a whole
+// row tile of walkers: 18 of 4096 pairs at 120 orbitals 5.7 ms against 14.7 with the digits.  The context holds
+// the images of its own contraction besides, so a smaller chunk of walkers.
+static constexpr size_t REFINE_CHUNK = (size_t)1 << 30;
+static bool refine_digits(const afqmc_config* c) {
+    return refine_enabled(c) && c->N > 128 &&
+           contract_fp64d_supported(c->N, c->n_up, c->n_dn, c->n_chol, c->n_walkers, c->n_paths);
+}
+
 static const char* check_config(const afqmc_config* c) {
     if (!c) return "config is NULL";
     if (c->N < 1 || c->N > 256) return "N must be in [1, 256]";
@@ -337,8 +349,8 @@ static size_t layout(const afqmc_config* c, char* base, Workspace* ws) {
     w.expT = (double*)take(NN * 8);
     // the double-float propagation needs its work arrays in shared memory
     const bool prop_df = c->precision != AFQMC_PRECISION_FP64 && propagate_in_smem(d.N, d.nt);
-    w.Ldf = prop_df || refine_enabled(c) ? take(G * NN * 8) : nullptr;
-    w.hdf = refine_enabled(c) ? take(NN * 8) : nullptr;
+    w.Ldf = prop_df || (refine_enabled(c) && !refine_digits(c)) ? take(G * NN * 8) : nullptr;
+    w.hdf = refine_enabled(c) && !refine_digits(c) ? take(NN * 8) : nullptr;
     w.xdf = c->precision != AFQMC_PRECISION_FP64 ? take(std::max(pairs * K, 2 * W * G) * 8) : nullptr;
     w.expTdf = prop_df ? take(NN * 8) : nullptr;
     w.scratchNN = (double*)take(3 * NN * 8);
@@ -353,6 +365,8 @@ static size_t layout(const afqmc_config* c, char* base, Workspace* ws) {
         const size_t ywalk = fd ? 0 : contract_fp64_walker_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P);
         w.fd = fd ? take(fd) : nullptr;
         w.ywalk = ywalk ? take(ywalk) : nullptr;
+    } else if (refine_digits(c)) {
+        w.fd = take(contract_fp64d_work_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P, REFINE_CHUNK));
     }
     w.phi = (double2*)take(W * N * nt * 16);
     w.weight = (double*)take(W * 8);
@@ -374,6 +388,8 @@ static size_t layout(const afqmc_config* c, char* base, Workspace* ws) {
     w.refine_th2 = refine ? (double*)take(2 * pairs * 8) : nullptr;   // per pair (and spin)
     w.refine_items = refine ? (int*)take(pairs * 4) : nullptr;
     w.refine_n = refine ? (int*)take(4) : nullptr;
+    w.refine_base = refine ? (int*)take(W * 4) : nullptr;
+    w.refine_count = refine ? (int*)take(W * 4) : nullptr;
     w.refine_lam = refine ? (double*)take((G + 1) * 8) : nullptr;
     w.Aplanes = (double*)take(2 * W * NN * 8);
     w.phi_new = (double2*)take(W * N * nt * 16);
@@ -598,7 +614,7 @@ static afqmc_status measure(afqmc_ctx* ctx, int part = 0) {
     const bool f16 = ctx->cfg.precision == AFQMC_PRECISION_FP16X3;
     const bool fp64 = ctx->cfg.precision == AFQMC_PRECISION_FP64;
     const int tck = fp64 ? -1 : tc_kind(&ctx->cfg);
-    const bool digits = w.fd && !w.rc;
+    const bool digits = fp64 && w.fd && !w.rc;
     const int ovl = digits ? OVL_TRIAL
                     : fp64 ? (!w.rc && !d.cphi && contract_fp64_walker_side(d.N, d.nu, d.nd, d.P) ? OVL_INVERSE : OVL_THETA)
                            : (tck == 2 || tck == 5 ? OVL_TRIAL : OVL_THETA);
@@ -637,31 +653,35 @@ static afqmc_status measure(afqmc_ctx* ctx, int part = 0) {
                   : contract_fp64(s, d, w.h, w.L, w.Phi, w.Theta, w.vpair, w.epair, d.pairs));
     }
     if ((st = prof_mark(ctx, PH_CONTRACT)) != AFQMC_OK) return st;
-    if (w.refine_items && tck == 5) {
+    if (w.refine_items) {
         // the pairs whose error would put their walker above refine_tol, again: selected
-        // by ||A_p^-1||_F^2 from the overlap kernel with the per-pair form's error model
-        // (measured per-pair errors of this form sit at 0.3-0.5 of it for N = 120 and 200),
-        // their Theta formed in place of B, then the double-float per-pair contraction;
-        // the log-overlaps go to scratch
+        // by ||A_p^-1||_F^2 (the walker-side form: from the overlap kernel, the per-pair form from its
+        // Theta) with one error model (measured per-pair errors of the walker-side form sit at
+        // 0.3-0.5 of it for N = 120 and 200); the log-overlaps of the factors formed again go to scratch.
         // unit roundoff of the model: fp16x3 and bf16x3 operands about 20 bits; fp16x6 operands about
         // 31 bits, the entries reaching the traces as FP32 numbers (24 bits)
         const double u = tc_mode(&ctx->cfg) == 2 ? 0x1p-24 : 0x1p-20;
-        CK(refine_select(s, d, ctx->cfg.refine_tol, w.refine_lam + d.G, w.logdet, w.Theta, w.refine_th2, w.alive,
-                         w.refine_items, w.refine_n, w.counters, w.refine_th2, u));
-        for (int spin = 0; spin < 2; ++spin)
-            CK(overlap_lu(s, d, spin, w.Phi, phi_stride(d), w.phi, w.logdet_new, w.Theta, nullptr, w.status, d.pairs,
-                          d.P, OVL_THETA, nullptr, w.refine_items, w.refine_n));
-        if (d.cphi)   // complex trial samples: the listed pairs in FP64
+        if (tck == 5)
+            CK(refine_select(s, d, ctx->cfg.refine_tol, w.refine_lam + d.G, w.logdet, w.Theta, w.refine_th2, w.alive,
+                             w.refine_items, w.refine_n, w.refine_base, w.refine_count, w.counters, w.refine_th2, u));
+        else
+            CK(refine_select(s, d, ctx->cfg.refine_tol, w.refine_lam + d.G, w.logdet, w.Theta, w.refine_th2, w.alive,
+                             w.refine_items, w.refine_n, w.refine_base, w.refine_count, w.counters));
+        // the listed pairs' B = Phi A^-T (digit products) or Theta in FP64, in place of what the
+        // contraction read
+        if (w.fd || tck == 5)
+            for (int spin = 0; spin < 2; ++spin)
+                CK(overlap_lu(s, d, spin, w.Phi, phi_stride(d), w.phi, w.logdet_new, w.Theta, nullptr, w.status,
+                              d.pairs, d.P, w.fd ? OVL_TRIAL : OVL_THETA, nullptr, w.refine_items, w.refine_n));
+        if (w.fd)
+            CK(contract_fp64d(s, d, w.fd, w.Theta, w.phi, w.vpair, w.epair, w.status,
+                              PairList{w.refine_items, w.refine_base, w.refine_count}, REFINE_CHUNK));
+        else if (tck == 5 && d.cphi)   // complex trial samples: the listed pairs in FP64
             CK(contract_fp64c(s, d, w.h, w.L, reinterpret_cast<const double2*>(w.Phi), w.Theta, w.vpair, w.epair,
                               w.refine_items, w.refine_n));
         else
             CK(contract_fp64_listed(s, d, w.h, w.L, w.Phi, w.Theta, w.vpair, w.epair, w.refine_items, w.refine_n,
                                     d.pairs, w.hdf, w.Ldf, w.refine_th2, d.pairs));
-    } else if (w.refine_items) {   // per-pair form: Theta is at hand
-        CK(refine_select(s, d, ctx->cfg.refine_tol, w.refine_lam + d.G, w.logdet, w.Theta, w.refine_th2, w.alive,
-                         w.refine_items, w.refine_n, w.counters));
-        CK(contract_fp64_listed(s, d, w.h, w.L, w.Phi, w.Theta, w.vpair, w.epair, w.refine_items, w.refine_n, d.pairs,
-                                w.hdf, w.Ldf, w.refine_th2, d.pairs));
     }
     if ((st = prof_mark(ctx, PH_REFINE)) != AFQMC_OK) return st;
     CK(walker_average(s, d, w.logdet, w.vpair, w.epair, w.logov, w.sumS, w.vbar, w.ebar));
@@ -717,7 +737,8 @@ extern "C" afqmc_status afqmc_init_trial(const afqmc_config* cfg, const double* 
         if (e == cudaSuccess) e = cudaMemsetAsync(w.status, 0, 4, s);
         if (e != cudaSuccess) { st = fail(AFQMC_ERR_CUDA, "copying inputs: %s", cudaGetErrorString(e)); break; }
         StepParams p = params_of(cfg);
-        if (w.fd && (e = contract_fp64d_prepare(s, d, w.h, w.L, w.fd)) != cudaSuccess) {
+        if (w.fd && (e = contract_fp64d_prepare(s, d, w.h, w.L, w.fd, cfg->precision == AFQMC_PRECISION_FP64 ? FD_CHUNK : REFINE_CHUNK)) !=
+                        cudaSuccess) {
             st = fail(AFQMC_ERR_CUDA, "digits of h and L: %s", cudaGetErrorString(e));
             break;
         }

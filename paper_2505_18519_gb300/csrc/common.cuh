@@ -187,6 +187,8 @@ struct Workspace {
     double* refine_th2;   // W*P   ||Theta_p||_F^2
     int* refine_items;    // W*P   pairs to recompute in FP64
     int* refine_n;        // 1     their number
+    int* refine_base;     // W     first of each walker's in refine_items
+    int* refine_count;    // W     number of each walker's
     double* refine_lam;   // G+1   ||L_g||_2^2, then their sum at [G]
     int* cheb_redo;       // W*P+1 trial orbitals to redo in double-float (tensor-core kernel), count at [W*P]
     // double-float copies for the overlaps' products on the mixed path (null when not used):

@@ -35,7 +35,8 @@
 // 50 orbitals, 512 x 32 pairs 19.4 ms against 265 (contract_fp64z_kernel, 0.98 of the FP64
 // pipe); 120 orbitals, 8 x 64 pairs 18 ms against 458 (contract_fp64_kernel); 37 orbitals,
 // 24 x 9 pairs 0.18 ms against 1.07; 8 orbitals, 64 x 16 pairs 0.15 ms against 0.40: faster
-// at every size it takes, so it takes all of those (fd_shape).
+// at every size it takes, so it takes all of those (fd_shape).  With a list of pairs (the mixed path's
+// refinement, api.cu has the rule) blocks of walkers and tiles without listed pairs end at once.
 //
 // Accuracy: operands to 63 (62) bits of the largest entry of their group (a matrix
 // X_g; a walker; a pair's B; one walker's Y_g of one spin), products exact, Y rounded
@@ -349,8 +350,13 @@ __global__ void __launch_bounds__(FDY_THREADS, 1)
     fd_y_kernel(int N8, int nu, int nd, int G1, int KCX, int ksteps, int JT, int NTY, int nbuf, int S, int GPB, int n_gblk,
                 int a_res, long long wb, const uint8_t* __restrict__ Pimg, const uint8_t* __restrict__ Ximg,
                 long long* __restrict__ Y0, long long* __restrict__ Y1, unsigned int* __restrict__ ymax, int* status,
-                uint32_t lim) {
+                uint32_t lim, const int* __restrict__ listed) {
     constexpr int D = Dg64<BITS>::D;
+    if (listed) {                                      // no walker of the tile has a listed pair
+        const long long wt = (long long)(blockIdx.x / n_gblk) * 128 / (2 * (nu + nd)) + threadIdx.x;
+        const bool in = threadIdx.x < 65 && wt < wb && wt * 2 * (nu + nd) < ((long long)(blockIdx.x / n_gblk) + 1) * 128;
+        if (!__syncthreads_or(in && listed[wt] > 0)) return;
+    }
     extern __shared__ uint8_t smraw[];
     uint8_t* sm = (uint8_t*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
     const uint32_t bbytes = (uint32_t)D * (uint32_t)NTY * 128u;
@@ -467,23 +473,28 @@ __global__ void __launch_bounds__(FDY_THREADS, 1)
 // Block: walker w0 + blockIdx.x / MT, pairs m PB .. of the walker, one spin.  Row
 // r = 64 ri + p_l n + a: [Re B[:, a] | -Im B[:, a]] (ri = 0), [Im B[:, a] | Re B[:, a]]
 // (ri = 1), each half N8 elements of K; KC chunks of D digits.  bexp[pair]: the
-// pair's exponent; bsh[pair]: the right shift that brings its Z into 2^zbits.
+// pair's exponent; bsh[pair]: the right shift that brings its Z into 2^zbits.  With a list
+// the walker's pairs are its listed ones, in the order of the list.
 template <int BITS>
 __global__ void __launch_bounds__(256) fd_b_image_kernel(int N, int N8, int nt, int col0, int n, int P, int PB, int MT,
                                                          int KC, int zbits, long long w0,
                                                          const double2* __restrict__ Bm, uint8_t* __restrict__ out,
-                                                         int* __restrict__ bexp, int* __restrict__ bsh) {
+                                                         int* __restrict__ bexp, int* __restrict__ bsh, PairList list) {
     constexpr int D = Dg64<BITS>::D;
     __shared__ double smax[64], sl1[64];
     __shared__ int sbad[64], se[64];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long wl = blockIdx.x / MT;
     const int m = blockIdx.x % MT;
-    const int np = min(PB, P - m * PB);
+    const int np = min(PB, (list.count ? list.count[w0 + wl] : P) - m * PB);
+    if (np <= 0) return;
     const long long lp0 = wl * P + (long long)m * PB;                  // first pair, in the chunk
-    const double2* B0 = Bm + (w0 * P + lp0) * (long long)N * nt + col0;
+    __shared__ long long spair[64];
+    if (tid < np) spair[tid] = list.count ? (long long)list.items[list.base[w0 + wl] + m * PB + tid] : w0 * P + lp0 + tid;
+    __syncthreads();
+    const double2* B0 = Bm + col0;
     for (int q = warp; q < np * n; q += 8) {
-        const double2* Bq = B0 + (long long)(q / n) * N * nt + q % n;
+        const double2* Bq = B0 + spair[q / n] * N * nt + q % n;
         double mx = 0.0, l1 = 0.0;
         bool bad = false;
         for (int i = lane; i < N; i += 32) {
@@ -534,7 +545,7 @@ __global__ void __launch_bounds__(256) fd_b_image_kernel(int N, int N8, int nt, 
         const int kim = k8 >= h8;
         long long F[8];
         const bool ok = q < np * n && k8 < 2 * h8;
-        const double2* Bq = B0 + (long long)(ok ? q / n : 0) * N * nt + (ok ? q % n : 0);
+        const double2* Bq = B0 + spair[ok ? q / n : 0] * N * nt + (ok ? q % n : 0);
         const int be = ok ? se[q / n] : 0;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
@@ -562,6 +573,7 @@ struct FdZArgs {
     const unsigned int* ymax;               // of this spin: entry (wl 2) G1 + g
     double2 *vpart, *expart;                // [pair][g], [segment][pair]
     int* status;
+    const int* listed;                      // nullable: pairs of each walker (of the chunk), P at most
 };
 
 // Left shift that brings one walker's Y_g of a spin (largest |Y| >> 32 = m) to 0.99 2^(TOT - 1).
@@ -622,7 +634,8 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
     const long long wm = blockIdx.x / A.NRUN;          // (walker, tile)
     const long long wl = wm / A.MT;
     const int m = (int)(wm % A.MT);
-    const int np = min(A.PB, A.P - m * A.PB);
+    const int np = min(A.PB, (A.listed ? A.listed[wl] : A.P) - m * A.PB);
+    if (np <= 0) return;                               // uniform
     const long long lp0 = wl * A.P + (long long)m * A.PB;
     const int t0 = run * A.RUN, t1 = min(A.NCT, t0 + A.RUN);
     const int tiles = t1 - t0;
@@ -904,21 +917,29 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
 
 // ---------------------------------------------------------------- per pair: v_g and E_L
 // One warp per pair of the chunk (pair0 the first): v_g = sum_s Tr Z_s (g >= 1),
-// E_L = sum_s Tr Z_{s,0} + 1/2 sum_g [v_g^2 - sum_s Tr Z_{s,g}^2].
-__global__ void fd_finish_kernel(long long pair0, long long pairs, int G, int two_spins, int nseg0, int nseg1,
+// E_L = sum_s Tr Z_{s,0} + 1/2 sum_g [v_g^2 - sum_s Tr Z_{s,g}^2].  With a list (w0 the chunk's
+// first walker) pair i of a walker is its listed pair i.
+__global__ void fd_finish_kernel(long long pair0, long long pairs, int P, long long w0, PairList list, int G, int two_spins, int nseg0, int nseg1,
                                  const double2* __restrict__ vp0, const double2* __restrict__ vp1,
                                  const double2* __restrict__ ex0, const double2* __restrict__ ex1,
                                  double2* __restrict__ vpair, double2* __restrict__ epair) {
     const long long p = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (p >= pairs) return;
+    long long out = pair0 + p;
+    if (list.count) {
+        const long long w = w0 + p / P;
+        const int i = (int)(p % P);
+        if (i >= list.count[w]) return;
+        out = list.items[list.base[w] + i];
+    }
     const double2* a = vp0 + p * (G + 1);
     const double2* b = vp1 + p * (G + 1);
     double2 s = cmk(0.0, 0.0);
     for (int g = 1 + lane; g <= G; g += 32) {
         double2 v = a[g];
         if (two_spins) v = cadd(v, b[g]);
-        vpair[(pair0 + p) * G + (g - 1)] = v;
+        vpair[out * G + (g - 1)] = v;
         cfma(s, v, v);
     }
     for (int q = lane; q < nseg0 + nseg1; q += 32) {
@@ -934,7 +955,7 @@ __global__ void fd_finish_kernel(long long pair0, long long pairs, int G, int tw
     if (lane == 0) {
         double2 e = a[0];
         if (two_spins) e = cadd(e, b[0]);
-        epair[pair0 + p] = cmk(e.x + 0.5 * s.x, e.y + 0.5 * s.y);
+        epair[out] = cmk(e.x + 0.5 * s.x, e.y + 0.5 * s.y);
     }
 }
 
@@ -1010,7 +1031,7 @@ bool fd_spin(const FdShape& s, int n, int P, FdSpin& f) {
 }
 
 // Digits by the length of the products: K = 2 N8 of GEMM-Z (and N of GEMM-Y) terms at most.
-bool fd_shape(int N, int nu, int nd, int G, long long W, int P, FdShape& s) {
+bool fd_shape(int N, int nu, int nd, int G, long long W, int P, size_t chunk, FdShape& s) {
     if (N < 1 || nu < 1 || nd < 0 || nd > nu || W < 1 || P < 1) return false;
     s.N8 = fd_up(N, 8);
     // GEMM-Y: with one K chunk the A digits stay in shared memory and two accumulator
@@ -1034,13 +1055,13 @@ bool fd_shape(int N, int nu, int nd, int G, long long W, int P, FdShape& s) {
     }
     if (s.SY < (s.yres ? s.KCX * s.D : 2)) return false;
     s.ximg = (size_t)s.G1 * s.JT * s.KCX * s.D * s.NTY * 128;
-    // about 4 GB of Y and A digits per chunk of walkers
+    // Y and A digits of as many walkers as `chunk` bytes hold
     size_t per = 0;
     for (int q = 0; q < 2; ++q) {
         const size_t y = (size_t)s.G1 * s.sp[q].n * 2 * s.N8 * 8;
         per += y + s.sp[q].aimg + (size_t)P * 16 * (s.G1 + s.sp[q].NSEG);
     }
-    s.WB = std::max(1LL, std::min(W, (long long)(((size_t)4 << 30) / per)));
+    s.WB = std::max(1LL, std::min(W, (long long)(chunk / per)));
     for (int q = 0; q < 2; ++q) {
         s.y[q] = (size_t)s.WB * s.G1 * s.sp[q].n * 2 * s.N8 * 8;
         s.aimg[q] = (size_t)s.WB * s.sp[q].aimg;
@@ -1097,7 +1118,7 @@ int fd_sms() {
 
 template <int BITS>
 cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWork& w, const double2* Bm,
-                   const double2* phi, double2* vpair, double2* epair, int* status) {
+                   const double2* phi, double2* vpair, double2* epair, int* status, const PairList& list) {
     const long long W = d.pairs / d.P;
     const int sms = fd_sms();
     cudaError_t e = raise_smem_limit((const void*)fd_y_kernel<BITS>, s.smem_y);
@@ -1115,7 +1136,7 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
         const int gpb = (s.G1 + want - 1) / want, ngb = (s.G1 + gpb - 1) / gpb;
         fd_y_kernel<BITS><<<(unsigned)(rt * ngb), FDY_THREADS, s.smem_y, st>>>(
             s.N8, d.nu, d.nd, s.G1, s.KCX, s.ysteps, s.JT, s.NTY, s.ybuf, s.SY, gpb, ngb, s.yres, wb, w.pimg, w.ximg, w.y[0], w.y[1],
-            w.ymax, status, FD_POLLS);
+            w.ymax, status, FD_POLLS, list.count ? list.count + w0 : nullptr);
         count_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         for (int q = 0; q < 2; ++q) {
@@ -1123,7 +1144,7 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
             if (f.n == 0) continue;
             fd_b_image_kernel<BITS><<<(unsigned)(wb * f.MT), 256, 0, st>>>(d.N, s.N8, d.nt, q ? d.nu : 0, f.n, d.P, f.PB,
                                                                          f.MT, s.KC, s.zbits, w0, Bm, w.aimg[q],
-                                                                         w.bexp[q], w.bsh[q]);
+                                                                         w.bexp[q], w.bsh[q], list);
             FdZArgs a;
             a.n = f.n; a.G1 = s.G1; a.N8 = s.N8; a.KC = s.KC; a.ksteps = s.zsteps; a.NT = f.NT; a.nbuf = f.nbuf; a.ngrp = f.ngrp; a.GB = f.GB;
             a.NCT = f.NCT; a.P = d.P; a.PB = f.PB; a.MT = f.MT; a.S = f.S; a.T = f.T; a.NSEG = f.NSEG;
@@ -1137,13 +1158,14 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
             a.Bimg = w.aimg[q]; a.bexp = w.bexp[q]; a.bsh = w.bsh[q]; a.pexp = w.pexp; a.xexp = w.xexp;
             a.Y = w.y[q]; a.ymax = w.ymax + (size_t)q * s.G1;
             a.vpart = w.vpart[q]; a.expart = w.expart[q]; a.status = status;
+            a.listed = list.count ? list.count + w0 : nullptr;
             contract_fp64d_kernel<BITS><<<(unsigned)(wm * a.NRUN), FDZ_THREADS, f.smem, st>>>(a, FD_POLLS);
             count_launches(2);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
         const long long pairs = wb * d.P;
         fd_finish_kernel<<<(unsigned)((pairs * 32 + 255) / 256), 256, 0, st>>>(
-            w0 * d.P, pairs, d.G, d.nd > 0, s.sp[0].NSEG, d.nd > 0 ? s.sp[1].NSEG : 0, w.vpart[0],
+            w0 * d.P, pairs, d.P, w0, list, d.G, d.nd > 0, s.sp[0].NSEG, d.nd > 0 ? s.sp[1].NSEG : 0, w.vpart[0],
             d.nd > 0 ? w.vpart[1] : w.vpart[0], w.expart[0], d.nd > 0 ? w.expart[1] : w.expart[0], vpair, epair);
         count_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -1163,31 +1185,31 @@ cudaError_t fd_prepare(cudaStream_t st, int N, const FdShape& s, const FdWork& w
 
 bool contract_fp64d_supported(int N, int nu, int nd, int G, long long W, int P) {
     FdShape s;
-    return fd_shape(N, nu, nd, G, W, P, s);
+    return fd_shape(N, nu, nd, G, W, P, FD_CHUNK, s);
 }
 
-size_t contract_fp64d_work_bytes(int N, int nu, int nd, int G, long long W, int P) {
+size_t contract_fp64d_work_bytes(int N, int nu, int nd, int G, long long W, int P, size_t chunk) {
     FdShape s;
-    if (!fd_shape(N, nu, nd, G, W, P, s)) return 0;
+    if (!fd_shape(N, nu, nd, G, W, P, chunk, s)) return 0;
     return fd_carve(nullptr, s, P).total;
 }
 
-cudaError_t contract_fp64d_prepare(cudaStream_t st, const Dims& d, const double* h, const double* L, void* work) {
+cudaError_t contract_fp64d_prepare(cudaStream_t st, const Dims& d, const double* h, const double* L, void* work, size_t chunk) {
     FdShape s;
-    if (!work || !fd_shape(d.N, d.nu, d.nd, d.G, d.pairs / d.P, d.P, s)) return cudaErrorInvalidValue;
+    if (!work || !fd_shape(d.N, d.nu, d.nd, d.G, d.pairs / d.P, d.P, chunk, s)) return cudaErrorInvalidValue;
     const FdWork w = fd_carve(work, s, d.P);
     return s.bits == 8 ? fd_prepare<8>(st, d.N, s, w, h, L) : fd_prepare<7>(st, d.N, s, w, h, L);
 }
 
 cudaError_t contract_fp64d(cudaStream_t st, const Dims& d, void* work, const double2* Bm, const double2* phi,
-                           double2* vpair, double2* epair, int* status) {
+                           double2* vpair, double2* epair, int* status, const PairList& list, size_t chunk) {
     FdShape s;
     if (!work || d.P < 1 || d.pairs % d.P != 0) return cudaErrorInvalidValue;
     if (d.pairs == 0) return cudaSuccess;
-    if (!fd_shape(d.N, d.nu, d.nd, d.G, d.pairs / d.P, d.P, s)) return cudaErrorInvalidValue;
+    if (!fd_shape(d.N, d.nu, d.nd, d.G, d.pairs / d.P, d.P, chunk, s)) return cudaErrorInvalidValue;
     const FdWork w = fd_carve(work, s, d.P);
-    return s.bits == 8 ? fd_run<8>(st, d, s, w, Bm, phi, vpair, epair, status)
-                       : fd_run<7>(st, d, s, w, Bm, phi, vpair, epair, status);
+    return s.bits == 8 ? fd_run<8>(st, d, s, w, Bm, phi, vpair, epair, status, list)
+                       : fd_run<7>(st, d, s, w, Bm, phi, vpair, epair, status, list);
 }
 
 }  // namespace afq

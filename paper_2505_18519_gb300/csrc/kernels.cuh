@@ -119,18 +119,18 @@ cudaError_t one_body_propagator(cudaStream_t s, int N, int G, double dtau, const
 cudaError_t contract_fp64(cudaStream_t s, const Dims& d, const double* h, const double* L, const double* Phi,
                           const double2* Theta, double2* vpair, double2* epair, long long pairs);
 bool contract_fp64_supported(int N, int nu, int nd);
-// Error-controlled refinement of the tensor-core contraction (per-pair form):
+// Error-controlled refinement of the tensor-core contraction:
 // lam = sum_g ||L_g||_2^2 (lam_g: G scratch values), once at init; per
 // measurement, the pairs each walker must recompute in FP64 so that its
-// estimated error stays below tol, appended to items (count in *n_items,
-// cumulative count in counters[5]).
+// estimated error stays below tol, appended to items (count in *n_items, walker w's
+// from wbase[w] on, wcount[w] of them; cumulative count in counters[5]).
 cudaError_t refine_scale(cudaStream_t s, int N, int G, const double* L, double* lam_g, double* lam);
 // th2_spins (nullable): ||Theta_p||_F^2 per pair and spin from the overlap kernel,
 // used instead of forming ||Theta_p||_F^2 from Theta; u: the contraction's
 // resolution in the error model (2^-20 for the per-pair form).
 cudaError_t refine_select(cudaStream_t s, const Dims& d, double tol, const double* lam, const double2* logdet,
                           const double2* Theta, double* th2, const int* alive, int* items, int* n_items,
-                          unsigned long long* counters, const double* th2_spins = nullptr, double u = 0x1p-20);
+                          int* wbase, int* wcount, unsigned long long* counters, const double* th2_spins = nullptr, double u = 0x1p-20);
 // The same contraction for the pairs items[0 .. *n_items) only (a device list of
 // pair indices, *n_items <= max_items), the others' vpair/epair left as they are;
 // with hdf and Ldf (double-float copies of h and L from u_to_df) R and M run in
@@ -157,12 +157,22 @@ cudaError_t contract_fp64_walker(cudaStream_t s, const Dims& d, const double* h,
 // products of FP64 accuracy): Z_{p,g} = B_p^T (X_g phi_w), B_p = Phi_p A_p^-T from
 // overlap_lu with OVL_TRIAL, real or complex trial samples.  N <= 224, n_up <= about
 // 60 (the digits of a column tile in shared memory).  work: contract_fp64d_work_bytes
-// bytes; contract_fp64d_prepare fills the digits of h and L once.
+// bytes; contract_fp64d_prepare fills the digits of h and L once.  chunk (the same in
+// the three calls): bytes for what the walkers worked on together take; h and L come on
+// top, and one walker is always taken.  With a list only the listed pairs are formed and written.
+constexpr size_t FD_CHUNK = (size_t)4 << 30;
+struct PairList {                // device arrays, all null: every pair
+    const int* items = nullptr;  // pairs; those of walker w at base[w] .. base[w] + count[w] - 1
+    const int* base = nullptr;
+    const int* count = nullptr;  // at most P each
+};
 bool contract_fp64d_supported(int N, int nu, int nd, int G, long long W, int P);
-size_t contract_fp64d_work_bytes(int N, int nu, int nd, int G, long long W, int P);
-cudaError_t contract_fp64d_prepare(cudaStream_t st, const Dims& d, const double* h, const double* L, void* work);
+size_t contract_fp64d_work_bytes(int N, int nu, int nd, int G, long long W, int P, size_t chunk = FD_CHUNK);
+cudaError_t contract_fp64d_prepare(cudaStream_t st, const Dims& d, const double* h, const double* L, void* work,
+                                   size_t chunk = FD_CHUNK);
 cudaError_t contract_fp64d(cudaStream_t st, const Dims& d, void* work, const double2* Bm, const double2* phi,
-                           double2* vpair, double2* epair, int* status);
+                           double2* vpair, double2* epair, int* status, const PairList& list = PairList(),
+                           size_t chunk = FD_CHUNK);
 
 // contract_tc.cu
 bool contract_tc_supported(int N, int nu, int nd, bool f16);

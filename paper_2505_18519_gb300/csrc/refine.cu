@@ -1,8 +1,9 @@
-// Error-controlled refinement of the tensor-core contraction (mixed precision,
-// per-pair form): the pairs that would put their walker's energy outside the
-// tolerance are recomputed by the per-pair contraction kernel in double-float
-// arithmetic (FP32 pairs, about 44 significant bits: some 2^24 times below the
-// split-FP16 error, at FP32 instruction rates).
+// Error-controlled refinement of the tensor-core contraction (mixed precision):
+// the pairs that would put their walker's energy outside the tolerance are
+// recomputed by the per-pair contraction kernel in double-float arithmetic (FP32
+// pairs, about 44 significant bits: some 2^24 times below the split-FP16 error,
+// at FP32 instruction rates), or, above 128 orbitals, with FP64 accuracy as
+// integer digit products on the tensor cores (contract_fp64d).
 //
 // The split-FP16 contraction carries about 20 significant bits per operand.
 // Its local-energy error grows with the conditioning of the overlap: for pair p
@@ -116,18 +117,22 @@ __global__ void __launch_bounds__(RF_T) theta_norm_kernel(int nn, long long pair
 
 // One block per walker: sort the walker's pairs by ||Theta_p||_F^2 (bitonic,
 // decreasing, ties by index), find how many of the largest must be refined, and
-// append their indices to items (order of walkers in the list is arbitrary).
+// append their indices to items (order of walkers in the list is arbitrary): the
+// walker's are items[wbase[w]] .. items[wbase[w] + wcount[w] - 1].
 __global__ void __launch_bounds__(RF_T) refine_select_kernel(int N, int P, double tol, const double* __restrict__ lam,
                                                              const double2* __restrict__ logdet,
                                                              const double* __restrict__ th2, int spins, double u,
                                                              const int* __restrict__ alive, int* items, int* n_items,
-                                                             unsigned long long* counters) {
+                                                             int* wbase, int* wcount, unsigned long long* counters) {
     __shared__ double key[RF_MAXP];
     __shared__ int id[RF_MAXP];
     __shared__ double red[RF_T / 32 + 1];
     __shared__ int s_base, s_k;
     const long long w = blockIdx.x;
-    if (alive && !alive[w]) return;
+    if (alive && !alive[w]) {
+        if (threadIdx.x == 0) wcount[w] = 0;
+        return;
+    }
     int P2 = 1;
     while (P2 < P) P2 <<= 1;
     for (int i = threadIdx.x; i < P2; i += RF_T) {
@@ -184,6 +189,8 @@ __global__ void __launch_bounds__(RF_T) refine_select_kernel(int N, int P, doubl
         }
         s_k = k;
         s_base = k > 0 ? atomicAdd(n_items, k) : 0;
+        wbase[w] = s_base;
+        wcount[w] = k;
         if (k > 0) atomicAdd(&counters[5], (unsigned long long)k);
     }
     __syncthreads();
@@ -192,7 +199,7 @@ __global__ void __launch_bounds__(RF_T) refine_select_kernel(int N, int P, doubl
 
 cudaError_t refine_select(cudaStream_t s, const Dims& d, double tol, const double* lam, const double2* logdet,
                           const double2* Theta, double* th2, const int* alive, int* items, int* n_items,
-                          unsigned long long* counters, const double* th2_spins, double u) {
+                          int* wbase, int* wcount, unsigned long long* counters, const double* th2_spins, double u) {
     if (d.P > RF_MAXP) return cudaErrorInvalidValue;
     if (d.pairs <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(n_items, 0, sizeof(int), s);
@@ -203,7 +210,7 @@ cudaError_t refine_select(cudaStream_t s, const Dims& d, double tol, const doubl
         count_launches(1);
     }
     refine_select_kernel<<<d.W, RF_T, 0, s>>>(d.N, d.P, tol, lam, logdet, th2_spins ? th2_spins : th2, th2_spins ? 1 : 0,
-                                              u, alive, items, n_items, counters);
+                                              u, alive, items, n_items, wbase, wcount, counters);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -65,3 +65,42 @@ def test_digit_contraction_matches_the_general_form(N, nu, nd, G, W, P):
     fb = (S[:, :, None] * v).sum(1) / sumS[:, None]
     grow = np.max(1.0 / np.abs(sumS)) * P                  # path signs that cancel magnify rounding
     assert np.max(np.abs(got["force_bias"] - fb)) < RTOL * grow * max(1.0, np.max(np.abs(v)))
+
+
+@pytest.mark.parametrize("precision,N,nu,nd,G,W,P", [
+    ("fp16x6", 140, 9, 7, 20, 5, 17),      # three row tiles of pairs a walker, walkers with few and with many
+    ("fp16x3", 150, 24, 24, 12, 9, 6),     # two pairs to a row tile
+    ("fp16x3", 129, 1, 0, 9, 70, 3),       # one spin, more walkers than a row tile of Y holds
+    ("fp16x6", 200, 40, 33, 6, 4, 3),      # one pair to a row tile, the largest electron numbers
+])
+def test_refined_pairs_alone_are_replaced(precision, N, nu, nd, G, W, P):
+    """Refinement at tolerances that list some pairs of some walkers: each pair's
+    energy is the tensor cores' own, bit for bit, or that of the FP64 context, and
+    the latter at least as often as the refinement counted.
+
+    Tolerance of an FP64 energy: RTOL, as above."""
+    s = ai.make_system(ai.SystemSpec(N, nu, nd, G, 3, True, 5000 + N))
+
+    def energies(prec, tol, state, **kw):
+        cfg = lib.make_config(N, nu, nd, G, 3, W, P, 0.005, 19, n_burn=2, precision=prec, refine_tol=tol, **kw)
+        ctx = lib.Context(cfg, s.h, s.L, s.Phi0, s.U)
+        ctx.load_state_arrays(state) if state is not None else ctx.step(1)
+        ctx.energy()
+        before = ctx.stats()["refined_pairs"]
+        ctx.energy()                                       # the same state again: the same pairs
+        out = ctx.observables()["e_local"], int(ctx.stats()["refined_pairs"] - before), ctx.state_arrays()
+        ctx.close()
+        return out
+
+    e64, _, state = energies("fp64", 0.0, None)
+    raw, none, _ = energies(precision, 0.0, state)
+    assert none == 0
+    counts = set()
+    for tol in [1e-300] + [10.0 ** (-0.5 * k) for k in range(4, 25)]:
+        e, n, _ = energies(precision, tol, state)
+        changed = e != raw
+        counts.add(n)
+        assert np.count_nonzero(changed) <= n <= W * P
+        assert np.count_nonzero(np.abs(e - e64) < RTOL * max(1.0, np.max(np.abs(e64)))) >= n
+        assert np.all(np.abs(e - e64)[changed] < RTOL * max(1.0, np.max(np.abs(e64))))
+    assert W * P in counts and len(counts) > 2             # some tolerance listed part of the pairs
