@@ -374,8 +374,10 @@ int afqmc_fp64_digits(const afqmc_config* cfg);
  * inside another framework's operator hook whose device memory must come from
  * that framework's pool, or a loop where an allocation, which may synchronise the
  * device, is not allowed).  Its intermediate matrices live in one fixed device
- * array of afqmc_noalloc_scratch_bytes() bytes (32 MiB) that every GPU loading
- * the library holds until exit; the caller passes only inputs and outputs.
+ * array of afqmc_noalloc_scratch_bytes() bytes (32 MiB), and the digits of the
+ * tensor-core contraction (FP64 accuracy, see afqmc_fp64_digits; sizes whose digits
+ * do not fit run the FP64 kernel) in another of 512 MiB, which a GPU holds from the
+ * first call on it until exit; the caller passes only inputs and outputs.
  *   h           N*N                      one-body matrix                    device
  *   L           n_chol*N*N               Cholesky vectors                   device
  *   Phi         n_pairs*N*n_up           trial orbitals of each pair        device

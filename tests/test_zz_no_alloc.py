@@ -150,3 +150,28 @@ def test_noalloc_rejects_batches_beyond_its_scratch():
     with pytest.raises(lib.AfqmcError) as ei:
         lib.local_energy_noalloc(1, 1, 1, 1, 1 << 59, 1, one, one, one, one, one, one, one)
     assert ei.value.status == 1 and "maximum" in str(ei.value)
+
+
+@pytest.mark.parametrize("spec,W,P,last", [
+    (ai.SystemSpec(8, 1, 1, 16, 6, False, 80), 8, 16, 16),       # the FP64 kernel's last batch
+    (ai.SystemSpec(8, 1, 1, 17, 6, False, 81), 3, 7, 7),         # the first of the digit products
+    (ai.SystemSpec(37, 7, 5, 40, 9, True, 82), 4, 9, 5),         # a last walker with fewer pairs
+    (ai.SystemSpec(37, 7, 5, 40, 9, True, 83), 1, 9, 2),         # that walker alone
+    (ai.SystemSpec(70, 9, 2, 30, 9, True, 84), 130, 1, 1),       # one pair per walker
+])
+def test_noalloc_splits_match_oracle(spec, W, P, last):
+    """Whole walkers and a last one with `last` of its P pairs, on both contraction kernels."""
+    s, ham, st = _oracle_state(spec, W, P, 0.01, 615)
+    d = _as_dict(st)
+    whole = _noalloc_on(d, s, spec, P)
+    dev = torch.device("cuda")
+    n = (W - 1) * P + last
+    Phi = torch.from_numpy(np.ascontiguousarray(d["Phi"].reshape(W * P, spec.N, spec.n_up)[:n])).to(dev)
+    phi = np.ascontiguousarray(np.concatenate([d["phi_up"], d["phi_dn"]], axis=2)).view(np.float64)
+    h, L, phi = (torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in (s.h, s.L, phi))
+    out = [torch.empty(2 * k, dtype=torch.float64, device=dev) for k in (n, n, n * spec.n_chol)]
+    lib.local_energy_noalloc(spec.N, spec.n_up, spec.n_dn, spec.n_chol, n, P, h, L, Phi, phi, *out)
+    part = [o.cpu().numpy().view(np.complex128) for o in out]
+    _compare_pairs_with_oracle(ham, st, *whole)
+    for got, want in zip(part, whole):
+        assert np.max(np.abs(got - want.reshape(-1)[:got.size])) < E_TOL
