@@ -153,7 +153,9 @@ typedef struct {
                            workspace per pair (16.4 GB for 512 x 32 pairs of the 50-orbital system) and needs
                            4 warps' shares of Theta (N x (n_up + n_dn) complex) and one matrix (N x n_up) in
                            220 KB of shared memory, and the refresh N^2 + 8 N n_up doubles in 200 KB (with
-                           10 + 10 electrons N <= 124; not 120 orbitals with 24 + 24).  0 (default): off */
+                           10 + 10 electrons N <= 124; not 120 orbitals with 24 + 24).  Where the digit
+                           products are faster (all but the smallest systems, see afqmc_fp64_digits), the
+                           measurement runs those and the space stays unread.  0 (default): off */
     int64_t wait_polls; /* tensor-core kernels: polls of an mbarrier before a main wait (a copy landing,
                            MMAs completing, an epilogue freeing a buffer) gives up; the block then sets
                            bit 4 of the device status word, lets its own copies and MMAs complete (a
@@ -299,7 +301,8 @@ afqmc_status afqmc_history(afqmc_ctx* ctx, double* out, int n, int* n_out);
  *   8 pairs recomputed by the refinement (see refine_tol) since init,
  *   9 population-control combs applied since init (see pop_period),
  *   10 walkers those combs replaced by copies of others,
- *   11 pairs whose cached half-rotated matrices were formed since init (see rcache),
+ *   11 pairs whose cached half-rotated matrices were formed since init (see rcache; where
+ *      the digit products run instead, pairs measured after their path had moved or was loaded),
  *   12 Chebyshev terms summed by the tensor-core trial-orbital kernel since init (see
  *      trial_form), 13 trial samples it handed to the double-float kernel because
  *      the Lanczos interval missed part of the spectrum */
@@ -358,14 +361,14 @@ int64_t afqmc_launch_count(void);
  * N <= 256, n_up <= 64: see tc_form), 6 contract_fp64c_kernel (precision FP64 with
  * complex trial samples: R_g = Phi^dagger X_g);
  * -1 if `cfg` is NULL or no kernel supports its sizes.  Host only.  For precision
- * FP64 with rcache = 0 the value names the FP64 arithmetic's kernel of these sizes
- * (0, 3 or 6); where afqmc_fp64_digits says so, contract_fp64d_kernel runs in its
+ * FP64 the value names the FP64 arithmetic's kernel of these sizes
+ * (0, 3, 4 or 6); where afqmc_fp64_digits says so, contract_fp64d_kernel runs in its
  * place: the walker-side form B_p^T (X_g phi_w) on the tensor cores, every product
  * as exact sums of integer digits, no less accurate than FP64 sums. */
 int afqmc_contract_kernel(const afqmc_config* cfg);
 /* 1 if the FP64 contraction of `cfg` runs on the tensor cores as integer digit
  * products (N <= 224 and up to about 60 electrons per spin, 48 above 64 orbitals;
- * precision FP64, rcache = 0), else 0.  Host only. */
+ * precision FP64; with rcache = 1 where it is faster than the cache), else 0.  Host only. */
 int afqmc_fp64_digits(const afqmc_config* cfg);
 
 /* Local energies, force-bias values and overlaps of a batch of (walker, trial

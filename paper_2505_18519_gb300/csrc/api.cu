@@ -61,8 +61,10 @@ extern "C" int afqmc_contract_kernel(const afqmc_config* cfg) {
     return tc_kind(cfg);
 }
 
+static bool cache_read(const afqmc_config* c);
+
 extern "C" int afqmc_fp64_digits(const afqmc_config* cfg) {
-    return cfg && cfg->precision == AFQMC_PRECISION_FP64 && !cfg->rcache && cfg->n_paths >= 1 && cfg->n_walkers >= 1 &&
+    return cfg && cfg->precision == AFQMC_PRECISION_FP64 && !cache_read(cfg) && cfg->n_paths >= 1 && cfg->n_walkers >= 1 &&
            contract_fp64d_supported(cfg->N, cfg->n_up, cfg->n_dn, cfg->n_chol, cfg->n_walkers, cfg->n_paths);
 }
 
@@ -225,6 +227,17 @@ extern "C" void afqmc_config_default(afqmc_config* c) {
     c->trial_alpha_re = 1.0;
     c->trial_alpha_im = 0.0;
     c->trial_slices = 1;
+}
+
+// rcache = 1: whether the measurement reads cached half-rotated matrices.  The digit-product
+// contraction, which has nothing to cache, is faster than reading them: 50 orbitals, 128 x 32
+// pairs 5.2 ms against 54 with 10 + 10 electrons, 256 x 32 pairs 1.5 against 15 with 1 + 1; 120
+// orbitals, 64 x 32 pairs with 2 + 2 1.6 against 35; 16 orbitals, 512 x 16 pairs 0.70 against 1.96.  Only the
+// smallest contractions of the smallest systems are too short for its launches (8 orbitals, 64 x 16
+// pairs, 32 matrices: 0.156 ms against 0.136 with 4 + 4 electrons, 0.151 against 0.130 with 1 + 1).
+static bool cache_read(const afqmc_config* c) {
+    const double work = (double)c->n_walkers * c->n_paths * (c->n_chol + 1) * c->N * (c->n_up * c->n_up + c->n_dn * c->n_dn);
+    return c->rcache && ((c->N <= 8 && work < 1e7) || !contract_fp64d_supported(c->N, c->n_up, c->n_dn, c->n_chol, c->n_walkers, c->n_paths));
 }
 
 // The tensor-core contraction's pairs with the largest error get recomputed in
@@ -411,7 +424,8 @@ static size_t layout(const afqmc_config* c, char* base, Workspace* ws) {
     w.macc = (double2*)take(2 * W * 16);
     w.mout = (double2*)take((2 * W + 2) * 16);
     if (c->rcache) {
-        w.rc = (double*)take(rcache_bytes(c->N, c->n_up, c->n_chol, (long long)c->n_walkers * c->n_paths));
+        double* rc = (double*)take(rcache_bytes(c->N, c->n_up, c->n_chol, (long long)c->n_walkers * c->n_paths));
+        w.rc = cache_read(c) ? rc : nullptr;
         w.rdirty = (int*)take(pairs * 4);
         w.rlist = (int*)take(pairs * 4);
         w.rcount = (int*)take(4);
@@ -615,6 +629,7 @@ static afqmc_status measure(afqmc_ctx* ctx, int part = 0) {
     const bool fp64 = ctx->cfg.precision == AFQMC_PRECISION_FP64;
     const int tck = fp64 ? -1 : tc_kind(&ctx->cfg);
     const bool digits = fp64 && w.fd && !w.rc;
+    if (part != 2 && digits && w.rdirty) CK(rcache_count_moved(s, d, w.rdirty, w.rlist, w.rcount, w.counters));
     const int ovl = digits ? OVL_TRIAL
                     : fp64 ? (!w.rc && !d.cphi && contract_fp64_walker_side(d.N, d.nu, d.nd, d.P) ? OVL_INVERSE : OVL_THETA)
                            : (tck == 2 || tck == 5 ? OVL_TRIAL : OVL_THETA);
@@ -1018,7 +1033,7 @@ extern "C" afqmc_status afqmc_energy_paths(afqmc_ctx* ctx, int rounds, int sweep
                                            double* ratio) {
     if (!ctx || !e_mix) return fail(AFQMC_ERR_ARG, "ctx and e_mix must not be NULL");
     if (rounds < 1 || sweeps < 0) return fail(AFQMC_ERR_ARG, "rounds must be >= 1 and sweeps >= 0");
-    if (ctx->ws.rc) return fail(AFQMC_ERR_ARG, "measurement paths are not available with rcache = 1");
+    if (ctx->cfg.rcache) return fail(AFQMC_ERR_ARG, "measurement paths are not available with rcache = 1");
     const Dims& d = ctx->d;
     Workspace& w = ctx->ws;
     cudaStream_t s = ctx->stream;

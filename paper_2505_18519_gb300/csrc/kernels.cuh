@@ -303,6 +303,9 @@ cudaError_t meas_finish(cudaStream_t s, const Dims& d, int rounds, const double*
 // pairs flagged dirty, and the FP64 contraction that reads them.
 bool contract_fp64r_supported(int N, int nu, int nd);
 size_t rcache_bytes(int N, int nu, int G, long long pairs);
+// rcache_count_moved: counts the dirty pairs and clears their flags, for a measurement that reads no cache.
+cudaError_t rcache_count_moved(cudaStream_t s, const Dims& d, int* dirty, int* list, int* count,
+                               unsigned long long* counters);
 cudaError_t rcache_refresh(cudaStream_t s, const Dims& d, const double* X, const double* Phi, int* dirty, int* list,
                            int* count, double* Rc, unsigned long long* counters);
 cudaError_t contract_fp64r(cudaStream_t s, const Dims& d, const double* Rc, const double2* Theta, double2* vpair,

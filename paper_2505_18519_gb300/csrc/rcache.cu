@@ -12,6 +12,10 @@
 // walker-side form; each measurement first refreshes the pairs whose path
 // moved since the last one (n_up N^2 multiply-adds per matrix and pair).
 //
+// The measurement reads them where that is faster than the digit-product contraction, which
+// keeps nothing from step to step (the rule and both sides' times: cache_read in api.cu);
+// elsewhere only the count of the moved pairs is kept.
+//
 // Storage: Rc[pair][g1][k][a] = (X_g1 Phi_p)[k, a] = R_g1,p[a, k] (X symmetric),
 // (G + 1) N n_up doubles per pair.  dirty[pair] = 1 marks a pair to refresh.
 #include "kernels.cuh"
@@ -178,12 +182,28 @@ __global__ void rcache_count_kernel(const int* count, unsigned long long* counte
     counters[8] += (unsigned long long)*count;
 }
 
+static cudaError_t rcache_collect(cudaStream_t s, const Dims& d, int* dirty, int* list, int* count) {
+    const cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    rcache_collect_kernel<<<(unsigned)((d.pairs + 255) / 256), 256, 0, s>>>(d.pairs, dirty, list, count);
+    return cudaSuccess;
+}
+
+cudaError_t rcache_count_moved(cudaStream_t s, const Dims& d, int* dirty, int* list, int* count,
+                               unsigned long long* counters) {
+    if (d.pairs <= 0) return cudaSuccess;
+    const cudaError_t e = rcache_collect(s, d, dirty, list, count);
+    if (e != cudaSuccess) return e;
+    rcache_count_kernel<<<1, 1, 0, s>>>(count, counters);
+    count_launches(2);
+    return cudaGetLastError();
+}
+
 cudaError_t rcache_refresh(cudaStream_t s, const Dims& d, const double* X, const double* Phi, int* dirty, int* list,
                            int* count, double* Rc, unsigned long long* counters) {
     if (d.pairs <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
+    cudaError_t e = rcache_collect(s, d, dirty, list, count);
     if (e != cudaSuccess) return e;
-    rcache_collect_kernel<<<(unsigned)((d.pairs + 255) / 256), 256, 0, s>>>(d.pairs, dirty, list, count);
     const size_t smem = rcache_fill_smem(d.N, d.nu);
     if ((e = raise_smem_limit((const void*)rcache_fill_kernel, smem)) != cudaSuccess) return e;
     rcache_fill_kernel<<<4 * 152, RC_T, smem, s>>>(d.N, d.nu, d.G, X, Phi, list, count, Rc);

@@ -851,7 +851,7 @@ cudaError_t population_control(cudaStream_t s, const Dims& d, const StepParams& 
     const long long rlen = Rc ? (long long)d.P * (d.G + 1) * d.N * d.nu : 0;
     CombRows rows{{(double*)phi, x, Phi, Rc},
                   {(long long)d.N * d.nt * 2, (long long)d.P * d.K, (long long)d.P * phi_stride(d), rlen},
-                  Rc ? rdirty : nullptr, d.P};
+                  rdirty, d.P};
     comb_gather_kernel<<<2 * 152, 256, 0, s>>>(rows, slot, from, flag);
     count_launches(2);
     return cudaGetLastError();
