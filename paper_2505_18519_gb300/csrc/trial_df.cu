@@ -37,21 +37,30 @@ constexpr double RHO_DF = 6.5;   // largest Gershgorin half-width run in double-
 // ||V_k||_F <= ||Phi0||_F); if they do, the problem is done again on the
 // Gershgorin interval of S, in double-float if its half-width is at most
 // RHO_DF and in FP64 otherwise.
-// One problem per call; the whole block of 256 threads takes part.  s_global (with
+// One problem per call; the whole block takes part.  s_global (with
 // s_is_df): S stays in global memory and is read from there (L2) by every term, for
 // N too large for S in shared memory; shared memory then holds the vectors only.
-__device__ __forceinline__ void cheb_df_problem(long long prob, int N, int nu, const double* __restrict__ S_all,
+struct ChebShared {
+    double coef[CHEB_DF_MAX + 2];
+    dfl coefd[CHEB_DF_MAX + 2];     // the coefficients in double-float, or as integer limbs
+    ChebScratch sc;
+    int nterms, mode;
+    dfl cshift_d, irho_d;
+    double cshift, irho;
+};
+
+__device__ __forceinline__ void cheb_df_problem(ChebShared& sh, long long prob, int N, int nu, const double* __restrict__ S_all,
                                                 const double* __restrict__ Phi0, double* __restrict__ Out,
                                                 const int* __restrict__ alive, int P, int* status, int allow_df,
                                                 int s_is_df, int s_global = 0) {
-    extern __shared__ dfl smf[];
-    __shared__ double coef[CHEB_DF_MAX + 2];
-    __shared__ dfl coefd[CHEB_DF_MAX + 2];
-    __shared__ ChebScratch sc;
+    extern __shared__ __align__(16) dfl smf[];
+    double* coef = sh.coef;
+    dfl* coefd = sh.coefd;
+    ChebScratch& sc = sh.sc;
     float* red8 = sc.red8;
-    __shared__ int nterms, mode;
-    __shared__ dfl cshift_d, irho_d;
-    __shared__ double cshift, irho;
+    int &nterms = sh.nterms, &mode = sh.mode;
+    dfl &cshift_d = sh.cshift_d, &irho_d = sh.irho_d;
+    double &cshift = sh.cshift, &irho = sh.irho;
     if (alive && !alive[prob / P]) return;
     const double* Sg = S_all + prob * (long long)N * N;
     const dfl* Sgd = reinterpret_cast<const dfl*>(Sg);
@@ -254,7 +263,8 @@ __global__ void __launch_bounds__(256) chebyshev_expm_df_kernel(int N, int nu, c
                                                                 const double* __restrict__ Phi0, double* __restrict__ Out,
                                                                 const int* __restrict__ alive, int P, int* status,
                                                                 int allow_df, int s_is_df, int s_global) {
-    cheb_df_problem(blockIdx.x, N, nu, S_all, Phi0, Out, alive, P, status, allow_df, s_is_df, s_global);
+    __shared__ ChebShared sh;
+    cheb_df_problem(sh, blockIdx.x, N, nu, S_all, Phi0, Out, alive, P, status, allow_df, s_is_df, s_global);
 }
 
 // The problems list[0 .. *count), grid-stride (the tensor-core kernel's redo list).
@@ -264,11 +274,239 @@ __global__ void __launch_bounds__(256) chebyshev_expm_df_list_kernel(int N, int 
                                                                      const int* __restrict__ alive, int P, int* status,
                                                                      int s_is_df, const int* __restrict__ list,
                                                                      const int* __restrict__ count) {
+    __shared__ ChebShared sh;
     const int n = *count;
     for (int i = blockIdx.x; i < n; i += gridDim.x) {
-        cheb_df_problem(list[i], N, nu, S_all, Phi0, Out, alive, P, status, 1, s_is_df);
+        cheb_df_problem(sh, list[i], N, nu, S_all, Phi0, Out, alive, P, status, 1, s_is_df);
         __syncthreads();   // the shared memory is reused by the next problem
     }
+}
+
+// ---------------------------------------------------------------- FP64 path: fixed point
+// The FP64 path's series in fixed point.  FP64 multiply-adds issue at two per clock and SM
+// here, 32-bit integer ones with a 64-bit sum at some sixteen times that, and every
+// quantity of the recurrence is bounded: t = (S - c) / rho has norm about 1 and the
+// columns of V_k = T_k(t) Phi0 do not outgrow those of Phi0.  So t is held in units of
+// 2^-54, column a of V in units of 2^(b_a - 58) with 2^b_a >= 1.25 of its norm, and the
+// coefficients in units of 2^-58 of a power of two above their sum, each value as
+// h 2^28 + l (|l| <= 2^27).  A product is h h' 2^56 + (h l' + l h') 2^28, three integer
+// multiply-adds (the dropped l l' are below a rounding of an FP64 sum of the same length: 2^-58
+// of the column's bound per term, of either sign), and
+//     V_k = 2 t V_(k-1) - V_(k-2)
+// takes no FP64 arithmetic at all.  Rounding: 2^-59 of the column's bound per term.
+//
+// What bounds it: the integer pipe, 3 C multiply-adds for C + 1 shared-memory reads per
+// thread and column of S.  A thread owns one row and C columns of V (consecutive threads
+// consecutive rows: S, stored transposed, is read without bank conflicts, V as
+// broadcasts).  On one GB300, against the FP64 recurrence: 16384 problems of 50 orbitals and 10
+// columns 4.87 ms against 17.1, 4096 of them 1.30 against 4.36, 1024 of 8 and 4 0.064 against
+// 0.111 (the Lanczos run and the coefficients then); errors against 64 bits as before (2e-15).
+//
+// The interval's estimate may miss part of the spectrum; with at most FX_GROW half-widths
+// of Gershgorin's bound in it no step overflows before the check on the growth of V (its
+// norm, each column in its own units, and each entry) ends the attempt.  Problems
+// outside that, and non-finite or extreme values, take the FP64 recurrence.
+// The FP64 recurrence, out of line: its registers are not the fixed-point loop's.
+__device__ __noinline__ void cheb_fp64_problem(ChebShared& sh, long long prob, int N, int nu, const double* S_all,
+                                               const double* Phi0, double* Out, const int* alive, int P, int* status) {
+    cheb_df_problem(sh, prob, N, nu, S_all, Phi0, Out, alive, P, status, 0, 0);
+}
+
+constexpr double FX_GROW = 6.0;
+constexpr int FX_LIMIT = 1 << 30;   // largest high part of an entry of V: its column's bound
+
+__device__ __forceinline__ int2 fx_split(long long v) {
+    const int l = ((int)v << 4) >> 4;
+    return make_int2((int)((v - l) >> 28), l);
+}
+
+template <int C>
+__global__ void __launch_bounds__(512) chebyshev_expm_fix_kernel(int N, int nu, const double* __restrict__ S_all,
+                                                                 const double* __restrict__ Phi0,
+                                                                 double* __restrict__ Out, const int* __restrict__ alive,
+                                                                 int P, int* status) {
+    extern __shared__ __align__(16) dfl smf[];
+    __shared__ ChebShared sh;
+    __shared__ int colb[64];        // b_a
+    __shared__ int cexp;            // the coefficients' power of two
+    const long long prob = blockIdx.x;
+    if (alive && !alive[prob / P]) return;
+    const double* Sg = S_all + prob * (long long)N * N;
+    const int tid = threadIdx.x, nth = blockDim.x;
+    const int ncg = (nu + C - 1) / C, nup = ncg * C, items = N * ncg;
+    for (int e = tid; e < N * N; e += nth) smf[e] = df_from(Sg[e]);
+    __syncthreads();
+    cheb_interval(N, &smf[0].hi, 2, sh.sc);
+    int2* T = reinterpret_cast<int2*>(smf);                     // t, transposed: T[j N + i] = t_ij
+    int2* Vp = T + ((size_t)N * N + 1) / 2 * 2;                 // N x nup, columns past nu zero
+    int2* Vc = Vp + (size_t)N * nup;                            // 16-byte aligned with even nup
+    long long* acc = reinterpret_cast<long long*>(Vc + (size_t)N * nup);
+    bool odd = false;               // problems left to FP64
+    if (tid < nu) {
+        float s = 0.f;
+        double mx = 0.0;
+        for (int i = 0; i < N; ++i) {
+            const double x = Phi0[i * nu + tid];
+            mx = fmax(mx, fabs(x));
+            odd |= !isfinite(x);
+            s = fmaf((float)x, (float)x, s);
+        }
+        if (mx == 0.0) {
+            colb[tid] = 0;
+        } else {
+            odd |= mx < 1e-15 || mx > 1e15;
+            colb[tid] = odd ? 0 : ilogbf(sqrtf(s) * 1.2502f) + 1;
+        }
+    }
+    __syncthreads();
+    float ps = 0.f;
+    for (int e = tid; e < N * nu; e += nth) {
+        const float f = ldexpf((float)Phi0[e], -colb[e % nu]);
+        ps = fmaf(f, f, ps);
+    }
+    const float grow_limit = 1.5625f * block_sum_f(ps, sh.sc.red8) + 1e-6f;   // 1.25 of the norm of Phi0, columns scaled
+
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        const double c = attempt == 0 ? sh.sc.est_c : sh.sc.gers_c, rho = attempt == 0 ? sh.sc.est_rho : sh.sc.gers_rho;
+        const double far = fmax(fabs(sh.sc.gers_c + sh.sc.gers_rho - c), fabs(sh.sc.gers_c - sh.sc.gers_rho - c));
+        odd |= !(far <= FX_GROW * rho) || !(fabs(c) + rho < 300.0);
+        if (__syncthreads_or(odd)) break;
+        if (tid == 0) {
+            sh.nterms = cheb_coefs(c, rho, 1e-18, sh.coef, status);
+            cexp = ilogb(exp(c + rho)) + 1;
+        }
+        const double ir = 1.0 / rho;
+        for (int e = tid; e < N * N; e += nth) {
+            const int i = e / N, j = e - i * N;
+            const double t = (i == j ? Sg[e] - c : Sg[e]) * ir;
+            T[(size_t)j * N + i] = fx_split(__double2ll_rn(t * 0x1p54));
+        }
+        __syncthreads();
+        const int m = sh.nterms, ce = cexp;
+        int2* ci = reinterpret_cast<int2*>(sh.coefd);
+        const double cu = ldexp(1.0, 58 - ce);
+        for (int k = tid; k <= m; k += nth) ci[k] = fx_split(__double2ll_rn(sh.coef[k] * cu));
+        __syncthreads();
+        // a term of the sum in units of 2^(ce + b_a - 60)
+        auto term = [&](int2 q, int2 v) -> long long {
+            const long long x = (long long)q.x * v.y + (long long)q.y * v.x;
+            return (long long)q.x * v.x + ((x + (1 << 27)) >> 28);
+        };
+        for (int e = tid; e < N * nup; e += nth) {
+            const int i = e / nup, a = e - i * nup;
+            const int2 v = a < nu ? fx_split(__double2ll_rn(ldexp(Phi0[i * nu + a], 58 - colb[a]))) : make_int2(0, 0);
+            Vp[e] = v;
+            acc[e] = term(ci[0], v);
+        }
+        __syncthreads();
+        bool grew = false;
+        for (int k = 1; k <= m && !grew; ++k) {
+            const int2* Vs = k == 1 ? Vp : Vc;
+            int2* Vd = k == 1 ? Vc : Vp;
+            const int2 ck = ci[k];
+            float ss = 0.f;
+            for (int it = tid; it < items; it += nth) {
+                const int cg = it / N, i = it - cg * N;
+                const int2* Tc = T + i;
+                const int2* Vj = Vs + cg * C;
+                long long h[C], x[C];
+#pragma unroll
+                for (int q = 0; q < C; ++q) h[q] = x[q] = 0;
+#pragma unroll 2
+                for (int j = 0; j < N; ++j) {
+                    const int2 t = Tc[(size_t)j * N];
+                    int2 v[C];
+                    if constexpr (C % 2 == 0) {               // nup and the columns even: 16-byte aligned
+#pragma unroll
+                        for (int q = 0; q < C; q += 2) {
+                            const int4 u = *reinterpret_cast<const int4*>(Vj + (size_t)j * nup + q);
+                            v[q] = make_int2(u.x, u.y);
+                            v[q + 1] = make_int2(u.z, u.w);
+                        }
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < C; ++q) v[q] = Vj[(size_t)j * nup + q];
+                    }
+#pragma unroll
+                    for (int q = 0; q < C; ++q) {
+                        h[q] += (long long)t.x * v[q].x;
+                        x[q] += (long long)t.x * v[q].y;
+                        x[q] += (long long)t.y * v[q].x;
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    const int o = i * nup + cg * C + q;
+                    long long v;
+                    if (k == 1) {
+                        v = h[q] * 4 + ((x[q] + (1 << 25)) >> 26);
+                    } else {
+                        const int2 b = Vp[o];
+                        v = h[q] * 8 + ((x[q] + (1 << 24)) >> 25) - ((long long)b.x * (1 << 28) + b.y);
+                    }
+                    const int2 w = fx_split(v);
+                    Vd[o] = w;
+                    acc[o] += term(ck, w);
+                    if (cg * C + q < nu) {
+                        const float f = (float)w.x * 0x1p-30f;
+                        ss = fmaf(f, f, ss);
+                        if (abs(w.x) > FX_LIMIT) ss = INFINITY;
+                    }
+                }
+            }
+            grew = block_sum_f(ss, sh.sc.red8) > grow_limit;   // uniform across the block
+            if (k >= 2) { int2* t = Vp; Vp = Vc; Vc = t; }
+        }
+        if (grew) {                 // the estimate missed part of the spectrum: start again
+            __syncthreads();
+            continue;
+        }
+        __syncthreads();
+        double* o = Out + prob * (long long)N * nu;
+        for (int e = tid; e < N * nu; e += nth) {
+            const int i = e / nu, a = e - i * nu;
+            o[e] = ldexp((double)acc[i * nup + a], ce + colb[a] - 60);
+        }
+        return;
+    }
+    __syncthreads();
+    cheb_fp64_problem(sh, prob, N, nu, S_all, Phi0, Out, alive, P, status);
+}
+
+static size_t fix_smem(int N, int nu, int C) {
+    const size_t nup = (size_t)(nu + C - 1) / C * C;
+    return (3 * (size_t)N * nup + ((size_t)N * N + 1) / 2 * 2) * 8;
+}
+
+// Columns per thread and threads per block: as many warps per SM as shared memory lets in (16
+// when it holds four problems), then the fewest clocks a thread spends per column of S: 3 c
+// multiply-adds at two warps per clock, two shared-memory wavefronts for S, one per column or pair.
+static bool fix_shape(int N, int nu, int& C, int& threads) {
+    double best = 0.0;
+    for (int c = 1; c <= 8; ++c) {
+        const size_t smem = fix_smem(N, nu, c);
+        if (smem > 200 * 1024) continue;
+        const int resident = (int)((220 * 1024) / (smem + sizeof(ChebShared) + 2048));
+        const int t = resident >= 4 ? 128 : resident >= 2 ? 256 : 512;
+        const double cost = (double)((N * ((nu + c - 1) / c) + t - 1) / t) * t * (1.5 * c + 2.0 + (c % 2 ? c : c / 2));
+        if (best == 0.0 || cost < best) {
+            best = cost;
+            C = c;
+            threads = t;
+        }
+    }
+    return best > 0.0;
+}
+
+template <int C>
+static cudaError_t launch_fix(cudaStream_t s, int N, int nu, long long problems, const double* S_all, const double* Phi0,
+                              double* Out, const int* alive, int P, int* status, int threads) {
+    const size_t bytes = fix_smem(N, nu, C);
+    const cudaError_t e = raise_smem_limit((const void*)chebyshev_expm_fix_kernel<C>, bytes);
+    if (e != cudaSuccess) return e;
+    chebyshev_expm_fix_kernel<C><<<(unsigned)problems, threads, bytes, s>>>(N, nu, S_all, Phi0, Out, alive, P, status);
+    count_launches(1);
+    return cudaGetLastError();
 }
 
 // Same contract as trial_orbitals (S_all is only read).
@@ -291,6 +529,20 @@ static cudaError_t trial_orbitals_lanczos(cudaStream_t s, int N, int nu, long lo
     if (!trial_orbitals_df_supported(N, nu) && !s_global) {   // the Gershgorin FP64 kernel
         if (s_is_df) return cudaErrorInvalidValue;
         return trial_orbitals_gershgorin(s, N, nu, problems, S_all, Phi0, Out, alive, P, status, threads);
+    }
+    int C = 1, fth = 128;
+    if (!allow_df && !s_is_df && nu <= 64 && fix_shape(N, nu, C, fth)) {
+        auto go = [&](auto f) { return f(s, N, nu, problems, S_all, Phi0, Out, alive, P, status, fth); };
+        switch (C) {
+        case 1: return go(launch_fix<1>);
+        case 2: return go(launch_fix<2>);
+        case 3: return go(launch_fix<3>);
+        case 4: return go(launch_fix<4>);
+        case 5: return go(launch_fix<5>);
+        case 6: return go(launch_fix<6>);
+        case 7: return go(launch_fix<7>);
+        default: return go(launch_fix<8>);
+        }
     }
     cudaError_t e = raise_smem_limit((const void*)chebyshev_expm_df_kernel, bytes);
     if (e != cudaSuccess) return e;
