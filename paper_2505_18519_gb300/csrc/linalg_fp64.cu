@@ -2,6 +2,8 @@
 // Theta = phi (Phi^T phi)^-1 matrices, re-orthonormalisation, the trial
 // orbitals Phi(x) = exp(S) Phi0 by a Chebyshev series, a plain FP64 GEMM, and the
 // init-time one-body propagator exp(-tau T / 2).
+#include <algorithm>
+
 #include "df.cuh"
 #include "kernels.cuh"
 
@@ -9,22 +11,24 @@ namespace afq {
 
 // ---------------------------------------------------------------- GEMM
 // C[M x Nc] = alpha * A[M x K] * B[K x Nc] + beta * C, row-major with leading
-// dimensions.  64 x 64 output tile per 256-thread block, 4 x 4 per thread.
+// dimensions.  16 R x 16 R output tile per 256-thread block, R x R per thread.
+template <int R>
 __global__ void __launch_bounds__(256) gemm_nn_f64_kernel(int M, int Nc, int K, double alpha, const double* __restrict__ A,
                                                           long long lda, const double* __restrict__ B, long long ldb,
                                                           double beta, double* __restrict__ C, long long ldc) {
-    __shared__ double As[16][64 + 1];
-    __shared__ double Bs[16][64];
+    constexpr int T = 16 * R;
+    __shared__ double As[16][T + 1];
+    __shared__ double Bs[16][T];
     int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    long long row0 = (long long)blockIdx.y * 64, col0 = (long long)blockIdx.x * 64;
-    double acc[4][4] = {};
+    long long row0 = (long long)blockIdx.y * T, col0 = (long long)blockIdx.x * T;
+    double acc[R][R] = {};
     for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-            int r = e / 16, kk = e % 16;          // A tile: 64 rows x 16 k
+        for (int e = threadIdx.x; e < 16 * T; e += 256) {
+            int r = e / 16, kk = e % 16;          // A tile: T rows x 16 k
             long long gr = row0 + r;
             int gk = k0 + kk;
             As[kk][r] = (gr < M && gk < K) ? A[gr * lda + gk] : 0.0;
-            int kb = e / 64, c = e % 64;          // B tile: 16 k x 64 cols
+            int kb = e / T, c = e % T;            // B tile: 16 k x T cols
             long long gc = col0 + c;
             int gkb = k0 + kb;
             Bs[kb][c] = (gkb < K && gc < Nc) ? B[(long long)gkb * ldb + gc] : 0.0;
@@ -32,24 +36,24 @@ __global__ void __launch_bounds__(256) gemm_nn_f64_kernel(int M, int Nc, int K, 
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < 16; ++kk) {
-            double a[4], b[4];
+            double a[R], b[R];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+            for (int i = 0; i < R; ++i) a[i] = As[kk][ty + 16 * i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+            for (int j = 0; j < R; ++j) b[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < R; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < R; ++i) {
         long long r = row0 + ty + 16 * i;
         if (r >= M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < R; ++j) {
             long long c = col0 + tx + 16 * j;
             if (c >= Nc) continue;
             double v = alpha * acc[i][j];
@@ -62,8 +66,15 @@ __global__ void __launch_bounds__(256) gemm_nn_f64_kernel(int M, int Nc, int K, 
 void gemm_nn_f64(cudaStream_t s, int M, int Nc, int K, double alpha, const double* A, long long lda, const double* B,
                  long long ldb, double beta, double* C, long long ldc) {
     if (M <= 0 || Nc <= 0) return;
-    dim3 grid((unsigned)((Nc + 63) / 64), (unsigned)((M + 63) / 64));
-    gemm_nn_f64_kernel<<<grid, 256, 0, s>>>(M, Nc, K, alpha, A, lda, B, ldb, beta, C, ldc); count_launches(1);
+    // The FP64 pipe bounds it (two multiply-adds per clock and SM), so a product of a few 64 x 64 tiles
+    // takes smaller ones, which spread it over the SMs; the sums are the same (64 walkers of 8 orbitals: the
+    // fields' 128 x 64 product with 32 matrices 43 -> 5.3 us, S of 1024 paths 22 -> 5.3).
+    auto tiles = [&](int t) { return (long long)((Nc + t - 1) / t) * ((M + t - 1) / t); };
+    auto grid = [&](int t) { return dim3((unsigned)((Nc + t - 1) / t), (unsigned)((M + t - 1) / t)); };
+    if (tiles(64) >= 152) gemm_nn_f64_kernel<4><<<grid(64), 256, 0, s>>>(M, Nc, K, alpha, A, lda, B, ldb, beta, C, ldc);
+    else if (tiles(32) >= 152) gemm_nn_f64_kernel<2><<<grid(32), 256, 0, s>>>(M, Nc, K, alpha, A, lda, B, ldb, beta, C, ldc);
+    else gemm_nn_f64_kernel<1><<<grid(16), 256, 0, s>>>(M, Nc, K, alpha, A, lda, B, ldb, beta, C, ldc);
+    count_launches(1);
 }
 
 // ---------------------------------------------------------------- overlap + LU
@@ -646,62 +657,75 @@ cudaError_t overlap_lu_both(cudaStream_t s, const Dims& d, const double* Phi, lo
 }
 
 // ---------------------------------------------------------------- re-orthonormalisation
-// One warp per (walker, spin): modified Gram-Schmidt on the N x n complex
+// One block per walker and spin: modified Gram-Schmidt on the N x n complex
 // block (columns col0..), q_j = (v_j - sum_k<j (q_k^H v_j) q_k) / norm, so
 // phi = Q R with R upper triangular and diag(R) > 0.  Dead walkers are copied.
-__global__ void reorth_kernel(int N, int nt, int n, int col0, const double2* __restrict__ src, double2* __restrict__ dst,
-                              const int* __restrict__ alive, int* status) {
-    extern __shared__ double2 q[];   // N x n
-    long long w = blockIdx.x;
-    int lane = threadIdx.x;
+// Columns in the right-looking order: once q_k is known every warp takes its share of
+// the columns j > k, and the warp of column k + 1 normalises it.  Each column meets the q_k in
+// the same order, with the same sums, as when one warp took the columns one by one, in n steps
+// instead of n^2 / 2: 64 walkers of 120 orbitals, 24 + 24 electrons, 2.1 -> 0.26 ms.
+constexpr int RO_WARPS = 16;
+__global__ void __launch_bounds__(RO_WARPS * 32) reorth_kernel(int N, int nu, int nd, const double2* __restrict__ src,
+                                                               double2* __restrict__ dst,
+                                                               const int* __restrict__ alive, int* status) {
+    extern __shared__ double2 q[];   // n columns of N
+    const long long w = blockIdx.x;
+    const int spin = blockIdx.y, nt = nu + nd, n = spin ? nd : nu, col0 = spin ? nu : 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const double2* in = src + w * (long long)N * nt + col0;
     double2* out = dst + w * (long long)N * nt + col0;
-    for (int e = lane; e < N * n; e += 32) q[e] = in[(long long)(e / n) * nt + e % n];
-    __syncwarp();
+    for (int e = threadIdx.x; e < N * n; e += blockDim.x) q[(size_t)(e % n) * N + e / n] = in[(long long)(e / n) * nt + e % n];
+    __syncthreads();
+    auto normalise = [&](int j) {
+        double2* qj = q + (size_t)j * N;
+        double nrm = 0.0;
+        for (int i = lane; i < N; i += 32) nrm += qj[i].x * qj[i].x + qj[i].y * qj[i].y;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
+        if (!(nrm > 0.0) || !isfinite(nrm)) {
+            if (lane == 0) atomicOr(status, STATUS_NONFINITE);
+            nrm = 1.0;
+        }
+        double inv = 1.0 / sqrt(nrm);
+        for (int i = lane; i < N; i += 32) qj[i] = cscale(qj[i], inv);
+    };
     if (alive == nullptr || alive[w]) {
-        for (int j = 0; j < n; ++j) {
-            for (int k = 0; k < j; ++k) {
+        if (warp == 0 && n > 0) normalise(0);
+        __syncthreads();
+        for (int k = 0; k + 1 < n; ++k) {
+            const double2* qk = q + (size_t)k * N;
+            for (int j = k + 1 + warp; j < n; j += nw) {     // the first warp's first column is k + 1
+                double2* qj = q + (size_t)j * N;
                 double2 dot = cmk(0.0, 0.0);
-                for (int i = lane; i < N; i += 32) cfma(dot, cconj(q[i * n + k]), q[i * n + j]);
+                for (int i = lane; i < N; i += 32) cfma(dot, cconj(qk[i]), qj[i]);
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) {
                     dot.x += __shfl_xor_sync(0xffffffffu, dot.x, off);
                     dot.y += __shfl_xor_sync(0xffffffffu, dot.y, off);
                 }
                 for (int i = lane; i < N; i += 32) {
-                    double2 v = q[i * n + j], qk = q[i * n + k];
-                    v.x -= dot.x * qk.x - dot.y * qk.y;
-                    v.y -= dot.x * qk.y + dot.y * qk.x;
-                    q[i * n + j] = v;
+                    double2 v = qj[i], qe = qk[i];
+                    v.x -= dot.x * qe.x - dot.y * qe.y;
+                    v.y -= dot.x * qe.y + dot.y * qe.x;
+                    qj[i] = v;
                 }
                 __syncwarp();
+                if (j == k + 1) normalise(j);
             }
-            double nrm = 0.0;
-            for (int i = lane; i < N; i += 32) nrm += q[i * n + j].x * q[i * n + j].x + q[i * n + j].y * q[i * n + j].y;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, off);
-            if (!(nrm > 0.0) || !isfinite(nrm)) {
-                if (lane == 0) atomicOr(status, STATUS_NONFINITE);
-                nrm = 1.0;
-            }
-            double inv = 1.0 / sqrt(nrm);
-            for (int i = lane; i < N; i += 32) q[i * n + j] = cscale(q[i * n + j], inv);
-            __syncwarp();
+            __syncthreads();
         }
     }
-    for (int e = lane; e < N * n; e += 32) out[(long long)(e / n) * nt + e % n] = q[e];
+    for (int e = threadIdx.x; e < N * n; e += blockDim.x) out[(long long)(e / n) * nt + e % n] = q[(size_t)(e % n) * N + e / n];
 }
 
 cudaError_t reorthonormalise(cudaStream_t s, const Dims& d, const double2* src, double2* dst, const int* alive, int* status,
                              int n_walkers) {
-    for (int spin = 0; spin < 2; ++spin) {
-        int n = spin == 0 ? d.nu : d.nd;
-        if (n == 0) continue;
-        size_t smem = (size_t)d.N * n * sizeof(double2);
-        cudaError_t e = raise_smem_limit((const void*)reorth_kernel, smem);
-        if (e != cudaSuccess) return e;
-        reorth_kernel<<<n_walkers, 32, smem, s>>>(d.N, d.nt, n, spin == 0 ? 0 : d.nu, src, dst, alive, status); count_launches(1);
-    }
+    size_t smem = (size_t)d.N * d.nu * sizeof(double2);
+    cudaError_t e = raise_smem_limit((const void*)reorth_kernel, smem);
+    if (e != cudaSuccess) return e;
+    const int warps = std::max(1, std::min(RO_WARPS, d.nu - 1));
+    reorth_kernel<<<dim3((unsigned)n_walkers, d.nd > 0 ? 2 : 1), warps * 32, smem, s>>>(d.N, d.nu, d.nd, src, dst, alive, status);
+    count_launches(1);
     return cudaGetLastError();
 }
 

@@ -311,29 +311,30 @@ __device__ __forceinline__ float4 df_pack(dfl re, dfl im) { return make_float4(r
 __global__ void __launch_bounds__(256) propagate_df_kernel(int N, int nt, int order, double dtau,
                                                            const dfl* __restrict__ E, const dfl* __restrict__ Aplanes,
                                                            const double2* __restrict__ phi, double2* phi_new,
-                                                           const int* __restrict__ alive) {
+                                                           const int* __restrict__ alive, int cols) {
     extern __shared__ float4 sdf[];
-    float4* V = sdf;                          // N x nt, (Re hi, Re lo, Im hi, Im lo)
-    float4* Wt = sdf + (size_t)N * nt;        // N x nt
+    const int c0 = blockIdx.y * cols, nb = min(cols, nt - c0);   // this block's columns
+    float4* V = sdf;                          // N x nb, (Re hi, Re lo, Im hi, Im lo)
+    float4* Wt = sdf + (size_t)N * nb;        // N x nb
     const long long w = blockIdx.x;
-    const double2* in = phi + w * (long long)N * nt;
-    double2* acc = phi_new + w * (long long)N * nt;
-    const int nn = N * nt;
+    const double2* in = phi + w * (long long)N * nt + c0;
+    double2* acc = phi_new + w * (long long)N * nt + c0;
+    const int nn = N * nb;
     if (!alive[w]) {
-        for (int e = threadIdx.x; e < nn; e += blockDim.x) acc[e] = in[e];
+        for (int e = threadIdx.x; e < nn; e += blockDim.x) acc[(e / nb) * nt + e % nb] = in[(e / nb) * nt + e % nb];
         return;
     }
     const dfl* Pm = Aplanes + (2 * w) * (long long)N * N;
     const dfl* Qm = Pm + (long long)N * N;
     for (int e = threadIdx.x; e < nn; e += blockDim.x) {
-        const double2 v = in[e];
+        const double2 v = in[(e / nb) * nt + e % nb];
         V[e] = df_pack(df_from(v.x), df_from(v.y));
     }
     __syncthreads();
     // Every product below: a thread takes row i and the four columns c = cg + k NG
-    // (k < 4, NG = ceil(nt / 4); consecutive threads, consecutive columns), so that each
+    // (k < 4, NG = ceil(nb / 4); consecutive threads, consecutive columns), so that each
     // load of a matrix entry serves four sums; every sum runs over j in order as before.
-    const int NG = (nt + 3) / 4;
+    const int NG = (nb + 3) / 4;
     // acc <- E phi
     for (int it = threadIdx.x; it < N * NG; it += blockDim.x) {
         const int i = it / NG, cg = it - i * NG;
@@ -344,8 +345,8 @@ __global__ void __launch_bounds__(256) propagate_df_kernel(int N, int nt, int or
             const dfl ev = E[(long long)i * N + j];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int c = min(cg + k * NG, nt - 1);
-                const float4 v = V[j * nt + c];
+                const int c = min(cg + k * NG, nb - 1);
+                const float4 v = V[j * nb + c];
                 dot2_fma(rh[k], rl[k], ev, dfl{v.x, v.y});
                 dot2_fma(ih[k], il[k], ev, dfl{v.z, v.w});
             }
@@ -353,9 +354,9 @@ __global__ void __launch_bounds__(256) propagate_df_kernel(int N, int nt, int or
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int c = cg + k * NG;
-            if (c >= nt) continue;
+            if (c >= nb) continue;
             const dfl re = df_two_sum(rh[k], rl[k]), im = df_two_sum(ih[k], il[k]);
-            Wt[i * nt + c] = df_pack(re, im);
+            Wt[i * nb + c] = df_pack(re, im);
             acc[i * nt + c] = make_double2(df_to(re), df_to(im));
         }
     }
@@ -376,8 +377,8 @@ __global__ void __launch_bounds__(256) propagate_df_kernel(int N, int nt, int or
                 const dfl npv = df_neg(pv), nqv = df_neg(qv);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const int c = min(cg + k * NG, nt - 1);
-                    const float4 v = cur[j * nt + c];
+                    const int c = min(cg + k * NG, nb - 1);
+                    const float4 v = cur[j * nb + c];
                     const dfl vr{v.x, v.y}, vi{v.z, v.w};
                     dot2_fma(rh[k], rl[k], nqv, vr);
                     dot2_fma(rh[k], rl[k], npv, vi);
@@ -388,9 +389,9 @@ __global__ void __launch_bounds__(256) propagate_df_kernel(int N, int nt, int or
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int c = cg + k * NG;
-                if (c >= nt) continue;
+                if (c >= nb) continue;
                 const dfl re = df_mul(df_two_sum(rh[k], rl[k]), scale), im = df_mul(df_two_sum(ih[k], il[k]), scale);
-                nxt[i * nt + c] = df_pack(re, im);
+                nxt[i * nb + c] = df_pack(re, im);
                 const double2 a = acc[i * nt + c];
                 acc[i * nt + c] = make_double2(a.x + df_to(re), a.y + df_to(im));
             }
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(256) propagate_df_kernel(int N, int nt, int or
         float4* t = cur; cur = nxt; nxt = t;
     }
     for (int e = threadIdx.x; e < nn; e += blockDim.x) {
-        const double2 a = acc[e];
+        const double2 a = acc[(e / nb) * nt + e % nb];
         V[e] = df_pack(df_from(a.x), df_from(a.y));
     }
     __syncthreads();
@@ -413,8 +414,8 @@ __global__ void __launch_bounds__(256) propagate_df_kernel(int N, int nt, int or
             const dfl ev = E[(long long)i * N + j];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int c = min(cg + k * NG, nt - 1);
-                const float4 v = V[j * nt + c];
+                const int c = min(cg + k * NG, nb - 1);
+                const float4 v = V[j * nb + c];
                 dot2_fma(rh[k], rl[k], ev, dfl{v.x, v.y});
                 dot2_fma(ih[k], il[k], ev, dfl{v.z, v.w});
             }
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(256) propagate_df_kernel(int N, int nt, int or
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int c = cg + k * NG;
-            if (c >= nt) continue;
+            if (c >= nb) continue;
             acc[i * nt + c] = make_double2(df_to(df_two_sum(rh[k], rl[k])), df_to(df_two_sum(ih[k], il[k])));
         }
     }
@@ -430,12 +431,17 @@ __global__ void __launch_bounds__(256) propagate_df_kernel(int N, int nt, int or
 
 cudaError_t propagate_df(cudaStream_t s, const Dims& d, const StepParams& p, const void* expTdf, const void* Aplanes_df,
                          const double2* phi, double2* phi_new, const int* alive) {
-    size_t smem = 2 * (size_t)d.N * d.nt * sizeof(float4);
     if (!propagate_in_smem(d.N, d.nt)) return cudaErrorInvalidValue;
+    // Columns propagate on their own: few walkers are split into blocks of at least eight
+    // columns, up to about three blocks per SM (64
+    // walkers of 120 orbitals and 48 columns 1.69 -> 0.74 ms).
+    const int split = std::max(1, std::min((3 * 152 + d.W - 1) / d.W, d.nt / 8));
+    const int cols = ((d.nt + split - 1) / split + 3) / 4 * 4;
+    const size_t smem = 2 * (size_t)d.N * std::min(cols, d.nt) * sizeof(float4);
     cudaError_t e = raise_smem_limit((const void*)propagate_df_kernel, smem);
     if (e != cudaSuccess) return e;
-    propagate_df_kernel<<<d.W, 256, smem, s>>>(d.N, d.nt, p.taylor_order, p.dtau, reinterpret_cast<const dfl*>(expTdf),
-                                               reinterpret_cast<const dfl*>(Aplanes_df), phi, phi_new, alive);
+    propagate_df_kernel<<<dim3(d.W, (d.nt + cols - 1) / cols), 256, smem, s>>>(d.N, d.nt, p.taylor_order, p.dtau, reinterpret_cast<const dfl*>(expTdf),
+                                               reinterpret_cast<const dfl*>(Aplanes_df), phi, phi_new, alive, cols);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -637,14 +643,17 @@ __global__ void handoff_kernel(int W, int P, int constraint, int importance, dou
     long long w = blockIdx.x;
     if (!alive[w]) return;
     int lane = threadIdx.x;
-    // fixed-order sum over paths: lane 0 adds sequentially for bitwise determinism
-    if (lane != 0) return;
-    double2 ns = cmk(0.0, 0.0);
-    for (int p = 0; p < P; ++p) {
+    // signs by the lanes; fixed-order sum over paths: lane 0 adds sequentially for bitwise determinism
+    __shared__ double2 sg[1024];
+    for (int p = lane; p < P; p += 32) {
         double s, c;
         sincos(logov_cur[w * P + p].y, &s, &c);
-        ns = cadd(ns, cmk(c, s));
+        sg[p] = cmk(c, s);
     }
+    __syncwarp();
+    if (lane != 0) return;
+    double2 ns = cmk(0.0, 0.0);
+    for (int p = 0; p < P; ++p) ns = cadd(ns, sg[p]);
     double dth = atan2(ratio[w].y, ratio[w].x);
     double dthT = atan2(ns.y, ns.x) - atan2(old_sum[w].y, old_sum[w].x);
     double f;
