@@ -358,6 +358,10 @@ static size_t layout(const afqmc_config* c, char* base, Workspace* ws) {
     w.Pslice = d.slices > 1 ? (double*)take(NN * 8) : nullptr;
     w.Vtmp = d.slices > 1 ? (double2*)take(pairs * N * nu * 16) : nullptr;
     w.Udf = c->precision != AFQMC_PRECISION_FP64 ? take(K * NN * 8) : nullptr;
+    if (c->precision == AFQMC_PRECISION_FP64) {
+        w.uexp = (int*)take(NN * 4);
+        w.lexp = (int*)take(NN * 4);
+    }
     w.T = (double*)take(NN * 8);
     w.expT = (double*)take(NN * 8);
     // the double-float propagation needs its work arrays in shared memory
@@ -532,6 +536,10 @@ static cudaError_t form_S(afqmc_ctx* ctx, const double* X, long long M) {
     if (w.Uimg && trial_on_tc(ctx) && s_in_df(ctx))
         return sprop_tc(ctx->stream, M, d.K, NN, X, w.Uimg, w.Sprop, w.status, d.wait_polls);
     if (s_in_df(ctx)) return gemm_df(ctx->stream, (int)M, (int)NN, d.K, X, w.Udf, w.Sprop, w.xdf);
+    // in fixed point where the series runs on its Lanczos interval; on Gershgorin's (S beyond shared
+    // memory) the series magnifies the rounding of S by e^(its excess), so S stays as it was there
+    if (w.uexp && d.K == d.KU && trial_orbitals_df_supported(d.N, d.nu) && gemm_fix_supported(M, NN, d.K))
+        return gemm_fix(ctx->stream, (int)M, NN, d.K, X, w.U, w.uexp, w.Sprop);
     gemm_nn_f64(ctx->stream, (int)M, (int)NN, d.K, 1.0, X, d.K, w.U, NN, 0.0, w.Sprop, NN);
     return cudaGetLastError();
 }
@@ -752,6 +760,11 @@ extern "C" afqmc_status afqmc_init_trial(const afqmc_config* cfg, const double* 
         if (e == cudaSuccess) e = cudaMemsetAsync(w.status, 0, 4, s);
         if (e != cudaSuccess) { st = fail(AFQMC_ERR_CUDA, "copying inputs: %s", cudaGetErrorString(e)); break; }
         StepParams p = params_of(cfg);
+        if (w.uexp && ((e = gemm_fix_prepare(s, d.KU, (long long)NN, w.U, w.uexp)) != cudaSuccess ||
+                       (e = gemm_fix_prepare(s, d.G, (long long)NN, w.L, w.lexp)) != cudaSuccess)) {
+            st = fail(AFQMC_ERR_CUDA, "exponents of U and L: %s", cudaGetErrorString(e));
+            break;
+        }
         if (w.fd && (e = contract_fp64d_prepare(s, d, w.h, w.L, w.fd, cfg->precision == AFQMC_PRECISION_FP64 ? FD_CHUNK : REFINE_CHUNK)) !=
                         cudaSuccess) {
             st = fail(AFQMC_ERR_CUDA, "digits of h and L: %s", cudaGetErrorString(e));
@@ -862,6 +875,8 @@ static afqmc_status step_rest(afqmc_ctx* ctx) {
         CK(fields(s, d, p, w.counters, w.vbar, w.sumS, w.weight, w.alive, (double*)w.y, w.logshift));
         if (w.expTdf) {   // mixed precision: field planes and propagation in double-float
             CK(gemm_df(s, 2 * d.W, d.N * d.N, d.G, (const double*)w.y, w.Ldf, w.Aplanes, w.xdf));
+        } else if (w.lexp && gemm_fix_supported(2 * d.W, (long long)d.N * d.N, d.G)) {
+            CK(gemm_fix(s, 2 * d.W, (long long)d.N * d.N, d.G, (const double*)w.y, w.L, w.lexp, w.Aplanes));
         } else {
             gemm_nn_f64(s, 2 * d.W, d.N * d.N, d.G, 1.0, (const double*)w.y, d.G, w.L, (long long)d.N * d.N, 0.0,
                         w.Aplanes, (long long)d.N * d.N);

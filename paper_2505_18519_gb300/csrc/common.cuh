@@ -186,6 +186,8 @@ struct Workspace {
     // error-controlled FP64 refinement of the tensor-core contraction (null when off)
     double* refine_th2;   // W*P   ||Theta_p||_F^2
     int* refine_items;    // W*P   pairs to recompute in FP64
+    int* uexp;            // N*N   FP64 path: exponents of the entries of U_k over k (gemm_fix.cu)
+    int* lexp;            // N*N   the same of L_g
     int* refine_n;        // 1     their number
     int* refine_base;     // W     first of each walker's in refine_items
     int* refine_count;    // W     number of each walker's

@@ -1,0 +1,159 @@
+// C = X U for the FP64 path's sums over hidden variables and auxiliary fields
+// (S_p = sum_k x_pk U_k, the field planes sum_g y_wg L_g) in fixed point: 32-bit
+// integer multiply-adds with 64-bit sums, which issue at some sixteen times the rate
+// of FP64 ones here.
+//
+// A row of X and a column of U (one entry of every matrix) each share an exponent, so an
+// element keeps the digits that matter to its own sum.  Values become
+// integers of 28 + b bits, h 2^28 + l with |l| <= 2^27, and a product
+// h h' 2^56 + (h l' + l h') 2^28; the dropped l l' is below 2^-(b + b') of the two
+// largest entries' product.  b + b' = 62 - log2 K keeps the sums of h h' within 63 bits
+// (56 bits of each operand at K = 50, 55 at 250): each product is off by 2^-56 (2^-55)
+// of the largest entries' product at most, of either sign, where an FP64 sum rounds its
+// partial sums at 2^-53.
+//
+// What bounds it: the integer pipe, 3 R^2 multiply-adds a thread and k for 2 R
+// shared-memory reads.  Against the FP64 GEMM (0.8 of the FP64 pipe) on one GB300:
+// S of 16384 paths, 50 orbitals and variables 4.41 -> 1.41 ms, of 4096 1.11 -> 0.37; the planes of
+// 512 walkers, 250 fields 1.30 -> 0.43.
+#include <algorithm>
+
+#include "digits64.cuh"
+#include "kernels.cuh"
+
+namespace afq {
+
+namespace {
+
+constexpr int GF_R = 4, GF_T = 16 * GF_R, GF_K = 16;
+
+// exponent e with |m| 2^-e < 1 of the largest |entry| m
+__device__ __forceinline__ int gf_exp(double m) { return m > 0.0 ? ilogb(m) + 1 : 0; }
+
+__device__ __forceinline__ int2 gf_split(double x, int e) {
+    const long long v = dg64_fix(x, e);
+    const int l = ((int)v << 4) >> 4;
+    return make_int2((int)((v - l) >> 28), l);
+}
+
+__global__ void gf_colexp_kernel(int K, long long Nc, const double* __restrict__ U, int* __restrict__ uexp) {
+    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < Nc; c += (long long)gridDim.x * blockDim.x) {
+        double m = 0.0;
+        bool bad = false;
+        for (int k = 0; k < K; ++k) {
+            const double v = fabs(U[(long long)k * Nc + c]);
+            bad |= !isfinite(v);
+            m = fmax(m, v);
+        }
+        uexp[c] = bad ? DG64_NAN : gf_exp(m);
+    }
+}
+
+__global__ void __launch_bounds__(256) gemm_fix_kernel(int M, long long Nc, int K, const double* __restrict__ X,
+                                                       const double* __restrict__ U, const int* __restrict__ uexp,
+                                                       double* __restrict__ C, int bx, int bu) {
+    __shared__ int2 Xs[GF_K][GF_T + 1], Us[GF_K][GF_T];
+    __shared__ int xe[GF_T], ue[GF_T];
+    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+    const long long row0 = (long long)blockIdx.y * GF_T, col0 = (long long)blockIdx.x * GF_T;
+    {   // exponents of the tile's rows: four threads a row
+        const long long r = row0 + tid / 4;
+        double m = 0.0;
+        bool bad = false;
+        if (r < M)
+            for (int k = tid & 3; k < K; k += 4) {
+                const double v = fabs(X[r * K + k]);
+                bad |= !isfinite(v);
+                m = fmax(m, v);
+            }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+            bad |= __shfl_xor_sync(0xffffffffu, (int)bad, o) != 0;
+        }
+        if ((tid & 3) == 0) xe[tid / 4] = bad ? DG64_NAN : gf_exp(m);
+        if (tid < GF_T) ue[tid] = col0 + tid < Nc ? uexp[col0 + tid] : 0;
+    }
+    __syncthreads();
+    long long h[GF_R][GF_R] = {}, x[GF_R][GF_R] = {};
+    for (int k0 = 0; k0 < K; k0 += GF_K) {
+#pragma unroll
+        for (int q = 0; q < GF_K * GF_T / 256; ++q) {
+            const int e = tid + q * 256;
+            const int r = e / GF_K, kk = e % GF_K;              // X tile: 64 rows x 16 k
+            const long long gr = row0 + r;
+            Xs[kk][r] = gr < M && k0 + kk < K ? gf_split(X[gr * K + k0 + kk], 28 + bx - xe[r]) : make_int2(0, 0);
+            const int kb = e / GF_T, c = e % GF_T;              // U tile: 16 k x 64 columns
+            const long long gc = col0 + c;
+            Us[kb][c] = gc < Nc && k0 + kb < K ? gf_split(U[(long long)(k0 + kb) * Nc + gc], 28 + bu - ue[c]) : make_int2(0, 0);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < GF_K; ++kk) {
+            int2 a[GF_R], b[GF_R];
+#pragma unroll
+            for (int i = 0; i < GF_R; ++i) a[i] = Xs[kk][ty + 16 * i];
+#pragma unroll
+            for (int j = 0; j < GF_R; ++j) b[j] = Us[kk][tx + 16 * j];
+#pragma unroll
+            for (int i = 0; i < GF_R; ++i)
+#pragma unroll
+                for (int j = 0; j < GF_R; ++j) {
+                    h[i][j] += (long long)a[i].x * b[j].x;
+                    x[i][j] += (long long)a[i].x * b[j].y;
+                    x[i][j] += (long long)a[i].y * b[j].x;
+                }
+        }
+        if ((k0 & 48) == 48)                                    // 64 terms: the cross sums stay below 2^62
+#pragma unroll
+            for (int i = 0; i < GF_R; ++i)
+#pragma unroll
+                for (int j = 0; j < GF_R; ++j) {
+                    h[i][j] += x[i][j] >> 28;
+                    x[i][j] &= (1 << 28) - 1;
+                }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < GF_R; ++i) {
+        const int rl = ty + 16 * i;
+        if (row0 + rl >= M) continue;
+#pragma unroll
+        for (int j = 0; j < GF_R; ++j) {
+            const int cl = tx + 16 * j;
+            if (col0 + cl >= Nc) continue;
+            const int er = xe[rl], ec = ue[cl];
+            double v = __longlong_as_double(0x7FF8000000000000LL);
+            if (er != DG64_NAN && ec != DG64_NAN)
+                v = ldexp((double)(h[i][j] + ((x[i][j] + (1 << 27)) >> 28)), er + ec - bx - bu);
+            C[(row0 + rl) * Nc + col0 + cl] = v;
+        }
+    }
+}
+
+}  // namespace
+
+// From this many tiles on the integer pipes are filled; fewer go to the FP64 kernel's small tiles.
+bool gemm_fix_supported(long long M, long long Nc, int K) {
+    return K >= 1 && K <= 4096 && ((M + GF_T - 1) / GF_T) * ((Nc + GF_T - 1) / GF_T) >= 152;
+}
+
+cudaError_t gemm_fix_prepare(cudaStream_t s, int K, long long Nc, const double* U, int* uexp) {
+    if (Nc <= 0 || K <= 0) return cudaSuccess;
+    gf_colexp_kernel<<<(unsigned)std::min<long long>((Nc + 255) / 256, 1024), 256, 0, s>>>(K, Nc, U, uexp);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t gemm_fix(cudaStream_t s, int M, long long Nc, int K, const double* X, const double* U, const int* uexp, double* C) {
+    if (!gemm_fix_supported(M, Nc, K)) return cudaErrorInvalidValue;
+    int lg = 0;
+    while ((1 << lg) < K) ++lg;
+    const int b = std::min(58, 62 - lg), bx = b / 2, bu = b - bx;
+    const dim3 grid((unsigned)((Nc + GF_T - 1) / GF_T), (unsigned)((M + GF_T - 1) / GF_T));
+    gemm_fix_kernel<<<grid, 256, 0, s>>>(M, Nc, K, X, U, uexp, C, bx, bu);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+}  // namespace afq
