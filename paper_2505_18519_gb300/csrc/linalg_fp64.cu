@@ -376,6 +376,200 @@ __global__ void overlap_lu_kernel(int N, int nu, int nt, int n, int col0, int sp
     }
 }
 
+// The listed pairs (few: the refinement's) with Theta or B, one block per pair at a time: the
+// arithmetic of overlap_lu_kernel entry by entry, in the same order, with the products, the
+// trailing updates of the LU and the columns of A^-1 spread over the block.  One warp per pair took
+// 0.78 ms for a list of any length up to a wave (24 electrons, 120 orbitals), bound by the FP64
+// pipe's latency; now 0.33 ms (18 pairs), and 1.6 ms against 3.0 for 165 pairs of 40 electrons and 200 orbitals.
+constexpr int OVL_LT = 256;
+__global__ void __launch_bounds__(OVL_LT) overlap_lu_listed_kernel(int N, int nu, int nt, int n, int col0, int spin, int P,
+                                                                   const double* __restrict__ Phi, long long Phi_stride,
+                                                                   const double2* __restrict__ phi,
+                                                                   double2* __restrict__ logdet,
+                                                                   double2* __restrict__ Theta, int* status,
+                                                                   int trial_side, const int* __restrict__ list,
+                                                                   const int* __restrict__ n_list, int cphi) {
+    extern __shared__ double2 sm[];
+    double2* A = sm;
+    double2* Ainv = A + (size_t)n * n;
+    double2* dinv = Ainv + (size_t)n * n;
+    int* perm = reinterpret_cast<int*>(dinv + n);
+    __shared__ int s_singular;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int count = *n_list;
+    for (int li = blockIdx.x; li < count; li += gridDim.x) {
+        const long long pair = list[li], w = pair / P;
+        const double* Ph = Phi + pair * Phi_stride;
+        const double2* ph = phi + w * (long long)N * nt + col0;
+        double2* Th = Theta + pair * (long long)N * nt + col0;
+        bool bad = false;
+        for (int e = tid; e < n * n; e += OVL_LT) {
+            int a = e / n, b = e - a * n;
+            double2 s = cmk(0.0, 0.0);
+            if (cphi) {
+                const double2* Pc = reinterpret_cast<const double2*>(Ph);
+                for (int i = 0; i < N; ++i) {
+                    const double2 f = Pc[(long long)i * nu + a];
+                    const double2 g = ph[(long long)i * nt + b];
+                    s.x = fma(f.x, g.x, fma(f.y, g.y, s.x));
+                    s.y = fma(f.x, g.y, fma(-f.y, g.x, s.y));
+                }
+            } else {
+                for (int i = 0; i < N; ++i) {
+                    double f = Ph[(long long)i * nu + a];
+                    double2 g = ph[(long long)i * nt + b];
+                    s.x = fma(f, g.x, s.x);
+                    s.y = fma(f, g.y, s.y);
+                }
+            }
+            A[e] = s;
+            bad |= !isfinite(s.x) || !isfinite(s.y);
+        }
+        for (int r = tid; r < n; r += OVL_LT) perm[r] = r;
+        if (tid == 0) s_singular = 0;
+        if (__syncthreads_or(bad)) {
+            if (tid == 0) {
+                logdet[pair * 2 + spin] = cmk(__longlong_as_double(0x7FF8000000000000LL), __longlong_as_double(0x7FF8000000000000LL));
+                atomicOr(status, STATUS_NONFINITE);
+            }
+            for (int e = tid; e < N * n; e += OVL_LT) Th[(long long)(e / n) * nt + e % n] = cmk(0.0, 0.0);
+            __syncthreads();
+            continue;
+        }
+        double2 z = cmk(1.0, 0.0);   // of warp 0
+        int zexp = 0;
+        bool odd = false;
+        for (int k = 0; k < n; ++k) {
+            if (warp == 0) {
+                double best = -1.0;
+                int bi = k;
+                for (int r = k + lane; r < n; r += 32) {
+                    double m = fabs(A[r * n + k].x) + fabs(A[r * n + k].y);
+                    if (m > best) { best = m; bi = r; }
+                }
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) {
+                    double ob = __shfl_down_sync(0xffffffffu, best, off);
+                    int oi = __shfl_down_sync(0xffffffffu, bi, off);
+                    if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+                }
+                best = __shfl_sync(0xffffffffu, best, 0);
+                bi = __shfl_sync(0xffffffffu, bi, 0);
+                if (!(best > 0.0)) {
+                    if (lane == 0) s_singular = 1;
+                } else {
+                    if (bi != k) {
+                        for (int c = lane; c < n; c += 32) {
+                            double2 t = A[k * n + c];
+                            A[k * n + c] = A[bi * n + c];
+                            A[bi * n + c] = t;
+                        }
+                        if (lane == 0) { int t = perm[k]; perm[k] = perm[bi]; perm[bi] = t; }
+                        odd = !odd;
+                    }
+                    __syncwarp();
+                    const double2 piv = A[k * n + k];
+                    const double q = 1.0 / fma(piv.x, piv.x, piv.y * piv.y);
+                    const double2 rinv = cmk(piv.x * q, -piv.y * q);   // 1 / piv
+                    if (lane == 0) dinv[k] = rinv;
+                    z = cmul(z, piv);
+                    {
+                        const double mz = fmax(fabs(z.x), fabs(z.y));
+                        int ex = (int)((__double_as_longlong(mz) >> 52) & 0x7FF) - 1023;
+                        ex = max(-1000, min(1000, ex));
+                        const double f = __longlong_as_double((long long)(1023 - ex) << 52);   // 2^-ex, exact
+                        z = cmk(z.x * f, z.y * f);
+                        zexp += ex;
+                    }
+                    for (int r = k + 1 + lane; r < n; r += 32) A[r * n + k] = cmul(A[r * n + k], rinv);
+                }
+            }
+            __syncthreads();
+            if (s_singular) break;
+            int m = n - k - 1;
+            for (int e = tid; e < m * m; e += OVL_LT) {
+                int r = k + 1 + e / m, c = k + 1 + e % m;
+                double2 t = A[r * n + c];
+                double2 l = A[r * n + k], u = A[k * n + c];
+                t.x -= l.x * u.x - l.y * u.y;
+                t.y -= l.x * u.y + l.y * u.x;
+                A[r * n + c] = t;
+            }
+            __syncthreads();
+        }
+        if (s_singular) {
+            if (tid == 0) {
+                logdet[pair * 2 + spin] = cmk(-INFINITY, 0.0);
+                atomicOr(status, STATUS_SINGULAR);
+            }
+            for (int e = tid; e < N * n; e += OVL_LT) Th[(long long)(e / n) * nt + e % n] = cmk(0.0, 0.0);
+            __syncthreads();
+            continue;
+        }
+        if (tid == 0) {
+            const double logabs = 0.5 * log(fma(z.x, z.x, z.y * z.y)) + zexp * 0.69314718055994530942;
+            logdet[pair * 2 + spin] = odd ? cmk(logabs, atan2(-z.y, -z.x)) : cmk(logabs, atan2(z.y, z.x));
+        }
+        // A^-1: forward substitution row by row over the block, each entry's terms in increasing j
+        for (int e = tid; e < n * n; e += OVL_LT) Ainv[e] = cmk(perm[e / n] == e % n ? 1.0 : 0.0, 0.0);
+        __syncthreads();
+        for (int j = 0; j + 1 < n; ++j) {
+            const int m = n - j - 1;
+            for (int e = tid; e < m * n; e += OVL_LT) {
+                const int r = j + 1 + e / n, c = e % n;
+                double2 s = Ainv[r * n + c];
+                double2 l = A[r * n + j], yj = Ainv[j * n + c];
+                s.x -= l.x * yj.x - l.y * yj.y;
+                s.y -= l.x * yj.y + l.y * yj.x;
+                Ainv[r * n + c] = s;
+            }
+            __syncthreads();
+        }
+        // backward: column c by one thread (its terms run the other way), columns over the warps
+        {
+            const int per = (n + OVL_LT / 32 - 1) / (OVL_LT / 32), c = warp * per + lane;
+            if (lane < per && c < n)
+                for (int r = n - 1; r >= 0; --r) {
+                    double2 s = Ainv[r * n + c];
+                    for (int j = r + 1; j < n; ++j) {
+                        double2 u = A[r * n + j], xj = Ainv[j * n + c];
+                        s.x -= u.x * xj.x - u.y * xj.y;
+                        s.y -= u.x * xj.y + u.y * xj.x;
+                    }
+                    Ainv[r * n + c] = cmul(s, dinv[r]);
+                }
+        }
+        __syncthreads();
+        if (trial_side) {            // B = Phi A^-T (conj(Phi) for complex trial orbitals)
+            for (int e = tid; e < N * n; e += OVL_LT) {
+                int i = e / n, b = e - i * n;
+                double2 s = cmk(0.0, 0.0);
+                if (cphi) {
+                    const double2* rowc = reinterpret_cast<const double2*>(Ph) + (long long)i * nu;
+                    for (int a = 0; a < n; ++a) cfma(s, cmk(rowc[a].x, -rowc[a].y), Ainv[b * n + a]);
+                } else {
+                    const double* row = Ph + (long long)i * nu;
+                    for (int a = 0; a < n; ++a) {
+                        const double2 t = Ainv[b * n + a];
+                        s.x = fma(row[a], t.x, s.x);
+                        s.y = fma(row[a], t.y, s.y);
+                    }
+                }
+                Th[(long long)i * nt + b] = s;
+            }
+        } else {                     // Theta = phi A^-1
+            for (int e = tid; e < N * n; e += OVL_LT) {
+                int i = e / n, b = e - i * n;
+                double2 s = cmk(0.0, 0.0);
+                const double2* row = ph + (long long)i * nt;
+                for (int a = 0; a < n; ++a) cfma(s, row[a], Ainv[a * n + b]);
+                Th[(long long)i * nt + b] = s;
+            }
+        }
+        __syncthreads();   // the next pair's A
+    }
+}
+
 static size_t overlap_smem_per_warp(int n, bool theta) {
     return ((size_t)n * n * (theta ? 2 : 1) + n + (n + 1) / 2 + 1) * sizeof(double2);
 }
@@ -392,6 +586,14 @@ cudaError_t overlap_lu(cudaStream_t s, const Dims& d, int spin, const double* Ph
     if (b_df && (!PhiD || trial_side != OVL_TRIAL)) return cudaErrorInvalidValue;
     int col0 = spin == 0 ? 0 : d.nu;
     size_t per = overlap_smem_per_warp(n, Theta != nullptr);
+    if (list && Theta && n > 0 && trial_side != OVL_INVERSE && !th2 && !alive && !PhiD && !Apre && per <= 220 * 1024) {
+        cudaError_t e = raise_smem_limit((const void*)overlap_lu_listed_kernel, per);
+        if (e != cudaSuccess) return e;
+        overlap_lu_listed_kernel<<<(unsigned)std::min<long long>(pairs, 2 * 152), OVL_LT, per, s>>>(
+            d.N, d.nu, d.nt, n, col0, spin, P, Phi, Phi_stride, phi, logdet, Theta, status, trial_side, list, n_list, d.cphi);
+        count_launches(1);
+        return cudaGetLastError();
+    }
     int wpb = d.ov_wpb > 0 ? d.ov_wpb : 4;
     while (wpb > 1 && per * wpb > 200 * 1024) wpb >>= 1;
     if (per * wpb > 220 * 1024) return cudaErrorInvalidValue;
