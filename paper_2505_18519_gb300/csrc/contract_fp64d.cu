@@ -475,12 +475,18 @@ __global__ void __launch_bounds__(FDY_THREADS, 1)
 // (ri = 1), each half N8 elements of K; KC chunks of D digits.  bexp[pair]: the
 // pair's exponent; bsh[pair]: the right shift that brings its Z into 2^zbits.  With a list
 // the walker's pairs are its listed ones, in the order of the list.
+// A block reads its columns of B into shared memory in one go (staged; they fit but for the
+// largest N) and forms exponents and digits from there: read from global memory column by
+// column, the loads' latency bound it (48 blocks of 200
+// orbitals and 40 electrons 110 us, now 75).
+constexpr int FDB_T = 512;
 template <int BITS>
-__global__ void __launch_bounds__(256) fd_b_image_kernel(int N, int N8, int nt, int col0, int n, int P, int PB, int MT,
+__global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt, int col0, int n, int P, int PB, int MT,
                                                          int KC, int zbits, long long w0,
                                                          const double2* __restrict__ Bm, uint8_t* __restrict__ out,
-                                                         int* __restrict__ bexp, int* __restrict__ bsh, PairList list) {
+                                                         int* __restrict__ bexp, int* __restrict__ bsh, PairList list, int staged) {
     constexpr int D = Dg64<BITS>::D;
+    extern __shared__ double2 sB[];                                    // column q (pair q / n, a = q % n) at q NS
     __shared__ double smax[64], sl1[64];
     __shared__ int sbad[64], se[64];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -493,12 +499,23 @@ __global__ void __launch_bounds__(256) fd_b_image_kernel(int N, int N8, int nt, 
     if (tid < np) spair[tid] = list.count ? (long long)list.items[list.base[w0 + wl] + m * PB + tid] : w0 * P + lp0 + tid;
     __syncthreads();
     const double2* B0 = Bm + col0;
-    for (int q = warp; q < np * n; q += 8) {
-        const double2* Bq = B0 + spair[q / n] * N * nt + q % n;
+    const int NS = N | 1, Nn = N * n;
+    if (staged) {
+        for (int e = tid; e < np * Nn; e += FDB_T) {
+            const int p = e / Nn, i = (e - p * Nn) / n, a = e - p * Nn - i * n;
+            sB[(p * n + a) * NS + i] = B0[(spair[p] * N + i) * nt + a];
+        }
+        __syncthreads();
+    }
+    // column q: entry i at Bq[i step]
+    const long long step = staged ? 1 : nt;
+    auto column = [&](int q) { return staged ? sB + q * NS : B0 + spair[q / n] * N * nt + q % n; };
+    for (int q = warp; q < np * n; q += FDB_T / 32) {
+        const double2* Bq = column(q);
         double mx = 0.0, l1 = 0.0;
         bool bad = false;
         for (int i = lane; i < N; i += 32) {
-            const double2 v = Bq[(long long)i * nt];
+            const double2 v = Bq[i * step];
             bad |= !isfinite(v.x) || !isfinite(v.y);
             mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
             l1 += fabs(v.x) + fabs(v.y);
@@ -538,21 +555,21 @@ __global__ void __launch_bounds__(256) fd_b_image_kernel(int N, int N8, int nt, 
     __syncthreads();
     uint8_t* base = out + (size_t)blockIdx.x * KC * D * FD_ADIG;
     const int h8 = N8 >> 3;
-    for (int e = tid; e < KC * 128 * 8; e += 256) {
+    for (int e = tid; e < KC * 128 * 8; e += FDB_T) {
         const int r = e & 127, u = (e >> 7) & 7, c = e >> 10;
         const int ri = r >> 6, q = r & 63;
         const int k8 = c * 8 + u;
         const int kim = k8 >= h8;
         long long F[8];
         const bool ok = q < np * n && k8 < 2 * h8;
-        const double2* Bq = B0 + spair[ok ? q / n : 0] * N * nt + (ok ? q % n : 0);
+        const double2* Bq = column(ok ? q : 0);
         const int be = ok ? se[q / n] : 0;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             const int i = (k8 - (kim ? h8 : 0)) * 8 + t;
             F[t] = 0;
             if (ok && i < N) {
-                const double2 v = Bq[(long long)i * nt];
+                const double2 v = Bq[i * step];
                 const long long f = dg64_fix((ri ^ kim) ? v.y : v.x, be);
                 F[t] = (kim && !ri) ? -f : f;
             }
@@ -1124,6 +1141,13 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
     cudaError_t e = raise_smem_limit((const void*)fd_y_kernel<BITS>, s.smem_y);
     for (int q = 0; q < 2 && e == cudaSuccess; ++q)
         if (s.sp[q].n) e = raise_smem_limit((const void*)contract_fp64d_kernel<BITS>, s.sp[q].smem);
+    size_t bsm[2] = {0, 0};                                            // B columns of a block, 0: not staged
+    for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+        const size_t b = (size_t)s.sp[q].PB * s.sp[q].n * (d.N | 1) * sizeof(double2);
+        if (b > 220 * 1024) continue;
+        bsm[q] = b;
+        if (b) e = raise_smem_limit((const void*)fd_b_image_kernel<BITS>, b);
+    }
     if (e != cudaSuccess) return e;
     for (long long w0 = 0; w0 < W; w0 += s.WB) {
         const long long wb = std::min(s.WB, W - w0);
@@ -1142,9 +1166,9 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
         for (int q = 0; q < 2; ++q) {
             const FdSpin& f = s.sp[q];
             if (f.n == 0) continue;
-            fd_b_image_kernel<BITS><<<(unsigned)(wb * f.MT), 256, 0, st>>>(d.N, s.N8, d.nt, q ? d.nu : 0, f.n, d.P, f.PB,
+            fd_b_image_kernel<BITS><<<(unsigned)(wb * f.MT), FDB_T, bsm[q], st>>>(d.N, s.N8, d.nt, q ? d.nu : 0, f.n, d.P, f.PB,
                                                                          f.MT, s.KC, s.zbits, w0, Bm, w.aimg[q],
-                                                                         w.bexp[q], w.bsh[q], list);
+                                                                         w.bexp[q], w.bsh[q], list, bsm[q] > 0);
             FdZArgs a;
             a.n = f.n; a.G1 = s.G1; a.N8 = s.N8; a.KC = s.KC; a.ksteps = s.zsteps; a.NT = f.NT; a.nbuf = f.nbuf; a.ngrp = f.ngrp; a.GB = f.GB;
             a.NCT = f.NCT; a.P = d.P; a.PB = f.PB; a.MT = f.MT; a.S = f.S; a.T = f.T; a.NSEG = f.NSEG;
