@@ -134,8 +134,8 @@ typedef struct {
                            the error-controlled refinement.  Each measurement estimates every pair's
                            contraction error as (2/N) u sum_g ||L_g||_2^2 ||Theta_p||_F^2 (u = 2^-20; fp16x6:
                            2^-24) and recomputes
-                           in double-float (FP32 pairs, about 44 bits) the pairs with the largest ||Theta_p||_F
-                           until the estimated error of the
+                           in double-float (FP32 pairs, about 44 bits; above 128 orbitals with FP64 accuracy,
+                           as integer digit products) the pairs with the largest ||Theta_p||_F until the estimated error of the
                            walker's average, 2 sqrt(sum of the kept pairs' squared errors) / |sum_p S_p|,
                            is at most refine_tol / 2.  0 turns it off.  Default 1e-4.  Not used by the
                            walker-side tensor-core form (N <= 64, n_up + n_dn <= 40), which keeps no Theta */
@@ -210,7 +210,8 @@ void afqmc_config_default(afqmc_config* cfg);
  * the state and per-pair buffers it holds, for the walker-side contraction forms,
  * Y_g = L_g phi_w: in FP64 (n_chol + 1) N 2 (n_up + n_dn) 64-bit integers per walker
  * of a chunk and the digits of the chunk's pairs (about 4 GB at most) and of h and
- * L_g (16 MB on the 50-orbital system, 1.1 GB at 200 orbitals), or the split-FP16 images
+ * L_g (16 MB on the 50-orbital system, 1.1 GB at 200 orbitals; the mixed path's refinement
+ * above 128 orbitals takes the same with 1 GB for the chunk), or the split-FP16 images
  * of it (6.2 MB per walker on the 50-orbital system). */
 size_t afqmc_workspace_bytes(const afqmc_config* cfg);
 

@@ -71,12 +71,24 @@ __host__ __device__ __forceinline__ Fp64Layout fp64_layout(int N, int nu, int nd
 // OWN: M entries owned per thread (n_up^2 + n_dn^2 <= OWN * CT); the double-float
 // mode with OWN = 8 fits two blocks per SM (slab layout, at most 128 registers;
 // the FP64 instances keep the same 128-register budget).
-// Runs per listed pair of the split double-float refinement: up to 16, as many
-// as the partial-sum space (part_cap double2 values) holds for n pairs.
-__device__ __forceinline__ int split_count(long long n, long long part_cap) {
+// Runs per listed pair of the split double-float refinement: of 16 and the numbers that fill
+// one to four waves of `blocks` blocks with n pairs (up to 64, eight matrices a run), the one whose waves
+// take the least time, as far as the partial-sum space (part_cap double2 values) holds it.  With 16 for
+// every n, four and eight pairs of 95 and 120 orbitals left three quarters and half of the blocks
+// idle: those two 6.3 -> 2.6 ms; the 18 to 22 pairs a step of 64 x 64 pairs of 120 orbitals
+// (16 runs of 20 pairs: two waves, the second nearly empty) 5.7 -> 4.1.
+__device__ __forceinline__ int split_count(long long n, long long part_cap, long long blocks, int G1) {
     if (n <= 0) return 1;
-    const long long g = part_cap / n;
-    return (int)(g < 1 ? 1 : (g > 16 ? 16 : g));
+    const long long most = min(part_cap / n, (long long)max(16, min(64, G1 / 8)));
+    long long best = max(1LL, min(16LL, most)), waves = (n * best + blocks - 1) / blocks;
+    for (int k = 1; k <= 4; ++k) {
+        const long long g = min(k * blocks / n, most);
+        if (g >= 1 && k * best < waves * g) {               // k / g < waves / best
+            best = g;
+            waves = k;
+        }
+    }
+    return (int)best;
 }
 
 template <bool SLAB, bool DF, int OWN>
@@ -113,7 +125,7 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
     // with epart, the matrices of each listed pair are split into gs runs, one work
     // item each, so that a few listed pairs still fill the GPU
     const long long n_list = items ? (long long)*n_items : (long long)gridDim.x;
-    const int gs = epart ? split_count(n_list, part_cap) : 1;
+    const int gs = epart ? split_count(n_list, part_cap, gridDim.x, G + 1) : 1;
     const long long n_work = n_list * gs;
     for (long long item = blockIdx.x; item < n_work; item += gridDim.x) {
     const long long pair = items ? (long long)items[item / gs] : item;
@@ -297,9 +309,10 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
 
 // E_L of the listed pairs from their runs' partial sums, in run order.
 __global__ void refine_sum_kernel(const int* __restrict__ items, const int* __restrict__ n_items,
-                                  const double2* __restrict__ epart, long long part_cap, double2* __restrict__ epair) {
+                                  const double2* __restrict__ epart, long long part_cap, long long blocks, int G1,
+                                  double2* __restrict__ epair) {
     const long long n = *n_items;
-    const int gs = split_count(n, part_cap);
+    const int gs = split_count(n, part_cap, blocks, G1);
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < n; it += (long long)gridDim.x * blockDim.x) {
         double2 e = epart[it * gs];
         for (int r = 1; r < gs; ++r) e = cadd(e, epart[it * gs + r]);
@@ -570,7 +583,7 @@ static cudaError_t launch_fp64_shape(cudaStream_t s, const Dims& d, int JB, size
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, CT, smem);
         if (e != cudaSuccess) return e;
         const long long cap = (long long)sms * (per_sm > 0 ? per_sm : 1);
-        if (epart) blocks = blocks * 16;   // up to 16 runs per listed pair
+        if (epart) blocks = blocks * 64;   // up to 64 runs per listed pair
         if (blocks > cap) blocks = cap;
     }
     contract_fp64_kernel<SLAB, DF, OWN><<<(unsigned)blocks, CT, smem, s>>>(d.N, d.nu, d.nd, d.G, JB, h, L, Phi, Theta,
@@ -578,7 +591,7 @@ static cudaError_t launch_fp64_shape(cudaStream_t s, const Dims& d, int JB, size
                                                                            epart, part_cap);
     count_launches(1);
     if (epart) {
-        refine_sum_kernel<<<64, 256, 0, s>>>(items, n_items, epart, part_cap, epair);
+        refine_sum_kernel<<<64, 256, 0, s>>>(items, n_items, epart, part_cap, blocks, d.G + 1, epair);
         count_launches(1);
     }
     return cudaGetLastError();

@@ -145,7 +145,7 @@ cudaError_t contract_fp64_listed(cudaStream_t s, const Dims& d, const double* h,
                                  const int* n_items, long long max_items, const void* hdf = nullptr,
                                  const void* Ldf = nullptr, void* part = nullptr, long long part_cap = 0);
 // (part, part_cap: with the double-float copies, space for part_cap double2 partial
-// sums; each listed pair's matrices are then split into up to 16 runs, one block
+// sums; each listed pair's matrices are then split into up to 64 runs, one block
 // each, and the runs' sums added in order: a few listed pairs fill the GPU.)
 // Walker-side FP64 form (Y_g = X_g phi_w once per block of a walker's pairs,
 // Z = Phi_p^T Y_g, Q = Z A_p^-1; Tr Q and Tr Q^2 are those of M_g): needs A^-1
