@@ -95,16 +95,24 @@ __global__ void __launch_bounds__(256) walker_average_kernel(int P, int G, const
         sS[p] = cmk(c, s);
     }
     __syncthreads();
-    double2 sumS = cmk(0.0, 0.0), se = cmk(0.0, 0.0);
-    for (int p = 0; p < P; ++p) {
-        sumS = cadd(sumS, sS[p]);
-        se = cadd(se, cmul(sS[p], epair[w * P + p]));
+    // the walker's sums by one warp: the FP64 pipe takes 16 clocks for each warp's instruction, and
+    // eight warps formed the same sums (64 walkers x 16 paths 21 us, now 16; 8 x 64 102 us, now 88)
+    __shared__ double2 s_inv;
+    if (threadIdx.x < 32) {
+        double2 sumS = cmk(0.0, 0.0), se = cmk(0.0, 0.0);
+        for (int p = 0; p < P; ++p) {
+            sumS = cadd(sumS, sS[p]);
+            se = cadd(se, cmul(sS[p], epair[w * P + p]));
+        }
+        const double2 inv = cdiv(cmk(1.0, 0.0), sumS);
+        if (threadIdx.x == 0) {
+            sumS_out[w] = sumS;
+            ebar[w] = cmul(se, inv);
+            s_inv = inv;
+        }
     }
-    double2 inv = cdiv(cmk(1.0, 0.0), sumS);
-    if (threadIdx.x == 0) {
-        sumS_out[w] = sumS;
-        ebar[w] = cmul(se, inv);
-    }
+    __syncthreads();
+    const double2 inv = s_inv;
     for (int g = threadIdx.x; g < G; g += blockDim.x) {
         double2 sv = cmk(0.0, 0.0);
         for (int p = 0; p < P; ++p) cfma(sv, sS[p], vpair[(w * P + p) * (long long)G + g]);
@@ -227,7 +235,8 @@ __global__ void __launch_bounds__(256) propagate_kernel(int N, int nt, int order
     }
     const double* Pm = Aplanes + (2 * w) * (long long)N * N;
     const double* Qm = Pm + (long long)N * N;
-    double st = sqrt(dtau);
+    const bool mine = threadIdx.x < nn;   // warps without an element leave the FP64 pipe to the others
+    const double st = mine ? sqrt(dtau) : 0.0;
     for (int e = threadIdx.x; e < nn; e += blockDim.x) V[e] = in[e];
     __syncthreads();
     // V <- E V ; acc <- V
@@ -247,7 +256,7 @@ __global__ void __launch_bounds__(256) propagate_kernel(int N, int nt, int order
     for (int e = threadIdx.x; e < nn; e += blockDim.x) V[e] = Wt[e];
     __syncthreads();
     for (int m = 1; m <= order; ++m) {
-        double inv = 1.0 / m;
+        const double inv = mine ? 1.0 / m : 0.0;
         for (int e = threadIdx.x; e < nn; e += blockDim.x) {
             int i = e / nt, c = e - i * nt;
             double pr = 0.0, pi = 0.0, qr = 0.0, qi = 0.0;   // (P V), (Q V)
