@@ -1,7 +1,7 @@
 // C = X U for the FP64 path's sums over hidden variables and auxiliary fields
 // (S_p = sum_k x_pk U_k, the field planes sum_g y_wg L_g) in fixed point: 32-bit
-// integer multiply-adds with 64-bit sums, which issue at some sixteen times the rate
-// of FP64 ones here.
+// integer multiply-adds with 64-bit sums, which issue at eight times the rate
+// of FP64 ones here (16 against 2 per clock and SM), three to a product.
 //
 // A row of X and a column of U (one entry of every matrix) each share an exponent, so an
 // element keeps the digits that matter to its own sum.  Values become
@@ -12,8 +12,8 @@
 // of the largest entries' product at most, of either sign, where an FP64 sum rounds its
 // partial sums at 2^-53.
 //
-// What bounds it: the integer pipe, 3 R^2 multiply-adds a thread and k for 2 R
-// shared-memory reads.  Against the FP64 GEMM (0.8 of the FP64 pipe) on one GB300:
+// What bounds it: that pipe (15 multiply-adds per clock and SM), 3 R^2 of them a thread and k for
+// 2 R shared-memory reads.  Against the FP64 GEMM (0.8 of the FP64 pipe) on one GB300:
 // S of 16384 paths, 50 orbitals and variables 4.41 -> 1.41 ms, of 4096 1.11 -> 0.37; the planes of
 // 512 walkers, 250 fields 1.30 -> 0.43.
 #include <algorithm>

@@ -284,7 +284,8 @@ __global__ void __launch_bounds__(256) chebyshev_expm_df_list_kernel(int N, int 
 
 // ---------------------------------------------------------------- FP64 path: fixed point
 // The FP64 path's series in fixed point.  FP64 multiply-adds issue at two per clock and SM
-// here, 32-bit integer ones with a 64-bit sum at some sixteen times that, and every
+// here, 32-bit integer ones with a 64-bit sum at sixteen (measured: 15 in gemm_fix_kernel, 18 here with
+// the other pipes' work beside them), and every
 // quantity of the recurrence is bounded: t = (S - c) / rho has norm about 1 and the
 // columns of V_k = T_k(t) Phi0 do not outgrow those of Phi0.  So t is held in units of
 // 2^-54, column a of V in units of 2^(b_a - 58) with 2^b_a >= 1.25 of its norm, and the
@@ -295,8 +296,8 @@ __global__ void __launch_bounds__(256) chebyshev_expm_df_list_kernel(int N, int 
 //     V_k = 2 t V_(k-1) - V_(k-2)
 // takes no FP64 arithmetic at all.  Rounding: 2^-59 of the column's bound per term.
 //
-// What bounds it: the integer pipe, 3 C multiply-adds for C + 1 shared-memory reads per
-// thread and column of S.  A thread owns one row and C columns of V (consecutive threads
+// What bounds it: that pipe, 3 C multiply-adds per thread and column of S beside the shared-memory
+// reads of S and of C entries of V.  A thread owns one row and C columns of V (consecutive threads
 // consecutive rows: S, stored transposed, is read without bank conflicts, V as
 // broadcasts).  On one GB300, against the FP64 recurrence: 16384 problems of 50 orbitals and 10
 // columns 4.87 ms against 17.1, 4096 of them 1.30 against 4.36, 1024 of 8 and 4 0.064 against
