@@ -227,6 +227,13 @@ __device__ __forceinline__ bool fd_mma_loop(FdPipe& p, uint32_t taddr, const uin
     }
 }
 
+// The largest |x| of a group as the bits of a double (the order of non-negative doubles is that of their
+// bits): FP64 comparisons would take the FP64 pipe, 16 clocks a warp.  Infinities and NaN come out above all.
+__device__ __forceinline__ unsigned long long fd_abs_bits(double x) {
+    return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+constexpr unsigned long long FD_INF_BITS = 0x7FF0000000000000ull;
+
 // 2^e, |e| <= 1000.
 __device__ __forceinline__ double fd_p2(int e) {
     return __longlong_as_double((long long)(1023 + max(-1000, min(1000, e))) << 52);
@@ -298,18 +305,15 @@ __global__ void __launch_bounds__(256) fd_phi_image_kernel(int N, int nt, int KC
     const long long wf = R0 / (2 * nt), wl = min(wb - 1, (R0 + 127) / (2 * nt));
     for (long long w = wf + warp; w <= wl; w += 8) {   // at most 65 walkers (2 nt >= 2)
         const double2* ph = phi + (w0 + w) * (long long)N * nt;
-        double m = 0.0;
-        bool bad = false;
+        unsigned long long m = 0;
         for (int e = lane; e < N * nt; e += 32) {
             const double2 v = ph[e];
-            bad |= !isfinite(v.x) || !isfinite(v.y);
-            m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
+            m = max(m, max(fd_abs_bits(v.x), fd_abs_bits(v.y)));
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-        bad = __any_sync(0xffffffffu, bad);
+        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (lane == 0) {
-            const int e = bad ? DG64_NAN : dg64_exp<BITS>(m);
+            const int e = m >= FD_INF_BITS ? DG64_NAN : dg64_exp<BITS>(__longlong_as_double((long long)m));
             se[w - wf] = e;
             pexp[w] = e;                               // every block of the walker writes the same
         }
@@ -477,8 +481,9 @@ __global__ void __launch_bounds__(FDY_THREADS, 1)
 // the walker's pairs are its listed ones, in the order of the list.
 // A block reads its columns of B into shared memory in one go (staged; they fit but for the
 // largest N) and forms exponents and digits from there: read from global memory column by
-// column, the loads' latency bound it (48 blocks of 200
-// orbitals and 40 electrons 110 us, now 75).
+// column, the loads' latency bound it, and the
+// FP64 pipe by the maxima's comparisons, integer ones now (48 blocks of 200 orbitals and 40 electrons 110 us,
+// staged 75; 64 blocks of 8 and 4 20 us staged, now 16).
 constexpr int FDB_T = 512;
 template <int BITS>
 __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt, int col0, int n, int P, int PB, int MT,
@@ -487,8 +492,9 @@ __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt
                                                          int* __restrict__ bexp, int* __restrict__ bsh, PairList list, int staged) {
     constexpr int D = Dg64<BITS>::D;
     extern __shared__ double2 sB[];                                    // column q (pair q / n, a = q % n) at q NS
-    __shared__ double smax[64], sl1[64];
-    __shared__ int sbad[64], se[64];
+    __shared__ unsigned long long smax[64];
+    __shared__ double sl1[64];
+    __shared__ int se[64];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long wl = blockIdx.x / MT;
     const int m = blockIdx.x % MT;
@@ -512,35 +518,33 @@ __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt
     auto column = [&](int q) { return staged ? sB + q * NS : B0 + spair[q / n] * N * nt + q % n; };
     for (int q = warp; q < np * n; q += FDB_T / 32) {
         const double2* Bq = column(q);
-        double mx = 0.0, l1 = 0.0;
-        bool bad = false;
+        unsigned long long mx = 0;
+        double l1 = 0.0;
         for (int i = lane; i < N; i += 32) {
             const double2 v = Bq[i * step];
-            bad |= !isfinite(v.x) || !isfinite(v.y);
-            mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
+            mx = max(mx, max(fd_abs_bits(v.x), fd_abs_bits(v.y)));
             l1 += fabs(v.x) + fabs(v.y);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
             l1 += __shfl_xor_sync(0xffffffffu, l1, o);
         }
-        bad = __any_sync(0xffffffffu, bad);
         if (lane == 0) {
             smax[q] = mx;
             sl1[q] = l1;
-            sbad[q] = bad;
         }
     }
     __syncthreads();
     if (tid < np) {
-        double mx = 0.0, l1 = 0.0;
-        int bad = 0;
+        unsigned long long mb = 0;
+        double l1 = 0.0;
         for (int a = 0; a < n; ++a) {
-            mx = fmax(mx, smax[tid * n + a]);
+            mb = max(mb, smax[tid * n + a]);
             l1 = fmax(l1, sl1[tid * n + a]);
-            bad |= sbad[tid * n + a];
         }
+        const bool bad = mb >= FD_INF_BITS;
+        const double mx = bad ? 0.0 : __longlong_as_double((long long)mb);
         const int e = bad ? DG64_NAN : dg64_exp<BITS>(mx);
         se[tid] = e;
         int sh = 0;
