@@ -892,8 +892,8 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
                     if (u < n) {
                         th += xr.x;
                         uh += xi.x;
-                        tl += xr.y - prx;
-                        ul += xi.y - prx;
+                        tl += (long long)xr.y - prx;      // a low half may be at the end of 32 bits
+                        ul += (long long)xi.y - prx;
                     }
                     xr.y >>= px; xi.y >>= px; yr.y >>= px; yi.y >>= px;
                     if (u >= n) {
