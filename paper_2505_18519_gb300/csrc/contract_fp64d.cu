@@ -39,7 +39,7 @@
 // refinement, api.cu has the rule) blocks of walkers and tiles without listed pairs end at once.
 //
 // Accuracy: operands to 63 (62) bits of the largest entry of their group (a matrix
-// X_g; a walker; a pair's B; one walker's Y_g of one spin), products exact, Y rounded
+// X_g; a column of a walker; a pair's B with its columns in the units those leave; one walker's Y_g of one spin), products exact, Y rounded
 // at 2^-57 (2^-55) of the product of its groups' largest entries, Z at 2^-56 of its
 // bound for Tr Z^2 and up to four bits finer for Tr Z: below the rounding of an FP64 sum
 // of the same length.  Against quad precision, 8 to 200 orbitals: pair energies 3e-17 to
@@ -292,50 +292,60 @@ __global__ void fd_x_image_kernel(int N, int KCX, int JT, int NTY, int G1, const
 }
 
 // ---------------------------------------------------------------- digits of the walkers
-// Block: 128 rows R = (w nt + c) 2 + ri of the chunk's walkers laid end to end
-// (Re/Im of column c), K = i; the exponent of a walker from all its columns.
+// Block: 64 columns of the chunk's walkers laid end to end, rows r = 2 column + (Re, Im), K = i.
+// A column has an exponent of its own, cexp[w nt + c]: Z D and D^-1 Z have the traces of Z, so the
+// column taken as phi 2^cexp here and B's as B 2^-cexp leave them as they are, and no column loses
+// digits to a longer one.  bad[w] (cleared before): a non-finite entry.
 template <int BITS>
 __global__ void __launch_bounds__(256) fd_phi_image_kernel(int N, int nt, int KCX, long long w0, long long wb,
                                                            const double2* __restrict__ phi, uint8_t* __restrict__ out,
-                                                           int* __restrict__ pexp) {
+                                                           int* __restrict__ cexp, unsigned int* __restrict__ bad) {
     constexpr int D = Dg64<BITS>::D;
-    __shared__ int se[130];
-    const long long R0 = (long long)blockIdx.x * 128, rows = wb * 2 * nt;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long wf = R0 / (2 * nt), wl = min(wb - 1, (R0 + 127) / (2 * nt));
-    for (long long w = wf + warp; w <= wl; w += 8) {   // at most 65 walkers (2 nt >= 2)
-        const double2* ph = phi + (w0 + w) * (long long)N * nt;
+    __shared__ unsigned long long smax[4][64];
+    __shared__ int se[64];
+    const long long C0 = (long long)blockIdx.x * 64, cols = wb * nt;
+    const int tid = threadIdx.x;
+    {
+        const int q = tid & 63, part = tid >> 6;
+        const long long C = C0 + q, w = C / nt;
         unsigned long long m = 0;
-        for (int e = lane; e < N * nt; e += 32) {
-            const double2 v = ph[e];
-            m = max(m, max(fd_abs_bits(v.x), fd_abs_bits(v.y)));
+        if (C < cols) {
+            const double2* ph = phi + (w0 + w) * (long long)N * nt + C % nt;
+            for (int i = part; i < N; i += 4) {
+                const double2 v = ph[(long long)i * nt];
+                m = max(m, max(fd_abs_bits(v.x), fd_abs_bits(v.y)));
+            }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) {
-            const int e = m >= FD_INF_BITS ? DG64_NAN : dg64_exp<BITS>(__longlong_as_double((long long)m));
-            se[w - wf] = e;
-            pexp[w] = e;                               // every block of the walker writes the same
+        smax[part][q] = m;
+    }
+    __syncthreads();
+    if (tid < 64) {
+        const unsigned long long m = max(max(smax[0][tid], smax[1][tid]), max(smax[2][tid], smax[3][tid]));
+        const bool inf = m >= FD_INF_BITS;
+        const int e = inf ? DG64_NAN : dg64_exp<BITS>(__longlong_as_double((long long)m));
+        se[tid] = e;
+        const long long C = C0 + tid;
+        if (C < cols) {
+            cexp[C] = inf ? 0 : e;
+            if (inf) bad[C / nt] = 1;
         }
     }
     __syncthreads();
     uint8_t* base = out + (size_t)blockIdx.x * KCX * D * FD_ADIG;
-    for (int e = threadIdx.x; e < KCX * 128 * 8; e += 256) {
+    for (int e = tid; e < KCX * 128 * 8; e += 256) {
         const int r = e & 127, u = (e >> 7) & 7, c = e >> 10;
-        const long long R = R0 + r;
         long long F[8];
-        const long long w = R / (2 * nt);
-        const int cc = (int)(R % (2 * nt));
-        const bool ok = R < rows;
-        const int pe = ok ? se[w - wf] : 0;
-        const double2* ph = phi + (w0 + w) * (long long)N * nt + (cc >> 1);
+        const long long C = C0 + (r >> 1);
+        const bool ok = C < cols;
+        const int pe = ok ? se[r >> 1] : 0;
+        const double2* ph = phi + (w0 + C / nt) * (long long)N * nt + C % nt;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             const int i = c * 64 + 8 * u + t;
             F[t] = 0;
             if (ok && i < N) {
                 const double2 v = ph[(long long)i * nt];
-                F[t] = dg64_fix((cc & 1) ? v.y : v.x, pe);
+                F[t] = dg64_fix((r & 1) ? v.y : v.x, pe);
             }
         }
         dg64_unit<BITS>(F, [&](int q, uint4 v) {
@@ -348,7 +358,7 @@ __global__ void __launch_bounds__(256) fd_phi_image_kernel(int N, int nt, int KC
 // Block: row tile blockIdx.x / n_gblk, matrices [gb GPB, (gb + 1) GPB); tiles (g, jt).
 // Y[s][((wl G1 + g) n_s + b) 2 + ri][i < N8], the pairs (i, i + 1) of i % 8 = 0 first, then those
 // of 2, 4, 6 (GEMM-Z's threads take eight values each, neighbours 16 bytes apart), as integers in units of
-// 2^(UNIT - XTRA - pexp[wl] - xexp[g]); ymax[(wl 2 + s) G1 + g] = max |Y| >> 32.
+// 2^(UNIT - XTRA - cexp - xexp[g]), cexp the column's; ymax[(wl 2 + s) G1 + g] = max |Y| >> 32.
 template <int BITS>
 __global__ void __launch_bounds__(FDY_THREADS, 1)
     fd_y_kernel(int N8, int nu, int nd, int G1, int KCX, int ksteps, int JT, int NTY, int nbuf, int S, int GPB, int n_gblk,
@@ -477,7 +487,7 @@ __global__ void __launch_bounds__(FDY_THREADS, 1)
 // Block: walker w0 + blockIdx.x / MT, pairs m PB .. of the walker, one spin.  Row
 // r = 64 ri + p_l n + a: [Re B[:, a] | -Im B[:, a]] (ri = 0), [Im B[:, a] | Re B[:, a]]
 // (ri = 1), each half N8 elements of K; KC chunks of D digits.  bexp[pair]: the
-// pair's exponent; bsh[pair]: the right shift that brings its Z into 2^zbits.  With a list
+// pair's exponent, that of the columns B 2^-cexp (the walkers' cexp); bsh[pair]: the right shift that brings its Z into 2^zbits.  With a list
 // the walker's pairs are its listed ones, in the order of the list.
 // A block reads its columns of B into shared memory in one go (staged; they fit but for the
 // largest N) and forms exponents and digits from there: read from global memory column by
@@ -487,14 +497,14 @@ __global__ void __launch_bounds__(FDY_THREADS, 1)
 constexpr int FDB_T = 512;
 template <int BITS>
 __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt, int col0, int n, int P, int PB, int MT,
-                                                         int KC, int zbits, long long w0,
+                                                         int KC, int zbits, long long w0, const int* __restrict__ cexp,
                                                          const double2* __restrict__ Bm, uint8_t* __restrict__ out,
                                                          int* __restrict__ bexp, int* __restrict__ bsh, PairList list, int staged) {
     constexpr int D = Dg64<BITS>::D;
     extern __shared__ double2 sB[];                                    // column q (pair q / n, a = q % n) at q NS
     __shared__ unsigned long long smax[64];
     __shared__ double sl1[64];
-    __shared__ int se[64];
+    __shared__ int se[64], sce[64];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long wl = blockIdx.x / MT;
     const int m = blockIdx.x % MT;
@@ -502,6 +512,7 @@ __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt
     if (np <= 0) return;
     const long long lp0 = wl * P + (long long)m * PB;                  // first pair, in the chunk
     __shared__ long long spair[64];
+    if (tid < n) sce[tid] = cexp[wl * nt + col0 + tid];
     if (tid < np) spair[tid] = list.count ? (long long)list.items[list.base[w0 + wl] + m * PB + tid] : w0 * P + lp0 + tid;
     __syncthreads();
     const double2* B0 = Bm + col0;
@@ -537,21 +548,26 @@ __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt
     }
     __syncthreads();
     if (tid < np) {
-        unsigned long long mb = 0;
-        double l1 = 0.0;
+        bool bad = false;
+        int e = INT_MAX;
         for (int a = 0; a < n; ++a) {
-            mb = max(mb, smax[tid * n + a]);
-            l1 = fmax(l1, sl1[tid * n + a]);
+            const unsigned long long m = smax[tid * n + a];
+            bad |= m >= FD_INF_BITS;
+            if (m > 0 && m < FD_INF_BITS) e = min(e, dg64_exp<BITS>(__longlong_as_double((long long)m)) + sce[a]);
         }
-        const bool bad = mb >= FD_INF_BITS;
-        const double mx = bad ? 0.0 : __longlong_as_double((long long)mb);
-        const int e = bad ? DG64_NAN : dg64_exp<BITS>(mx);
+        if (e == INT_MAX) e = 0;
+        if (bad) e = DG64_NAN;
         se[tid] = e;
         int sh = 0;
-        if (!bad && mx > 0.0) {
-            // |Z'| <= (l1 2^e / 2^(TOT - 1)) 2^54 before the shift; l1 / mx <= 2 N8 <= 512
-            const double b0 = (l1 / mx) * (1.0 + 1e-9);
-            sh = max(0, ilogb(b0) + 1 + 54 - zbits);
+        if (!bad) {
+            // |Z'| <= b0 2^54 before the shift, b0 the largest sum of a column's integers over 2^(TOT - 1)
+            double b0 = 0.0;
+            for (int a = 0; a < n; ++a) {
+                const double m = __longlong_as_double((long long)smax[tid * n + a]);
+                if (m > 0.0)
+                    b0 = fmax(b0, fmin(sl1[tid * n + a] / m, 2.0 * N) * ldexp(m, e - sce[a] - (Dg64<BITS>::TOT - 1)));
+            }
+            if (b0 > 0.0) sh = max(0, ilogb(b0 * (1.0 + 1e-9)) + 1 + 54 - zbits);
         }
         bexp[lp0 + tid] = e;
         bsh[lp0 + tid] = sh;
@@ -567,7 +583,7 @@ __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt
         long long F[8];
         const bool ok = q < np * n && k8 < 2 * h8;
         const double2* Bq = column(ok ? q : 0);
-        const int be = ok ? se[q / n] : 0;
+        const int be = ok ? se[q / n] - sce[q % n] : 0;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             const int i = (k8 - (kim ? h8 : 0)) * 8 + t;
@@ -589,7 +605,8 @@ struct FdZArgs {
     int n, G1, N8, KC, ksteps, NT, nbuf, ngrp, GB, NCT, P, PB, MT, S, T, RUN, NRUN, NSEG;
     long long pairs;                        // of the chunk
     const uint8_t* Bimg;
-    const int *bexp, *bsh, *pexp, *xexp;
+    const int *bexp, *bsh, *xexp;
+    const unsigned int* bad;                // walkers with a non-finite entry
     const long long* Y;
     const unsigned int* ymax;               // of this spin: entry (wl 2) G1 + g
     double2 *vpart, *expart;                // [pair][g], [segment][pair]
@@ -714,7 +731,7 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
         __syncwarp();
     } else if (warp >= FDZ_FIN / 32) {
         // ---- the sums of a tile to FP64: lane q takes the (pair, g) q, q + 32, ..
-        const int pw = A.pexp[wl];
+        const bool bad = A.bad[wl] != 0;
         for (int q = lane; q < combos; q += 32) sex[q] = cmk(0.0, 0.0);
         for (int t = t0; t < t1; ++t) {
             const int rb = (t - t0) & 1, use = (t - t0) >> 1;
@@ -739,13 +756,13 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
                 }
                 double2 v, ex;
                 const int eb = sbexp[pl];
-                if (xe == DG64_NAN || pw == DG64_NAN || eb == DG64_NAN) {
+                if (xe == DG64_NAN || bad || eb == DG64_NAN) {
                     const double nan = __longlong_as_double(0x7FF8000000000000LL);
                     v = cmk(nan, nan);
                     ex = v;
                 } else {
                     // value of Z' = 1: 2^(UNIT + shift - bexp - yexp), in two exact factors
-                    const int ey = fd_yshift<BITS>(ym) - (Dg64<BITS>::UNIT - Dg64<BITS>::XTRA) + pw + xe;
+                    const int ey = fd_yshift<BITS>(ym) - (Dg64<BITS>::UNIT - Dg64<BITS>::XTRA) + xe;
                     const int sc = Dg64<BITS>::UNIT + sbsh[pl] - eb - ey;
                     const double f1 = fd_p2(sc >> 1), f2 = fd_p2(sc - (sc >> 1));
                     const double el = fd_p2(-min(FD_XTRA, sbsh[pl])), eh = fd_p2(FD_LOW);
@@ -1096,9 +1113,9 @@ size_t fd_align(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct FdWork {
     uint8_t *ximg, *pimg, *aimg[2];
-    int *xexp, *pexp, *bexp[2], *bsh[2];
+    int *xexp, *cexp, *bexp[2], *bsh[2];
     long long* y[2];
-    unsigned int* ymax;
+    unsigned int *ymax, *bad;   // cleared together
     double2 *vpart[2], *expart[2];
     size_t total;
 };
@@ -1116,8 +1133,9 @@ FdWork fd_carve(void* work, const FdShape& s, int P) {
     w.ximg = take(s.ximg);
     w.xexp = reinterpret_cast<int*>(take((size_t)s.G1 * 4));
     w.pimg = take(s.pimg);
-    w.pexp = reinterpret_cast<int*>(take((size_t)s.WB * 4));
-    w.ymax = reinterpret_cast<unsigned int*>(take((size_t)s.WB * 2 * s.G1 * 4));
+    w.cexp = reinterpret_cast<int*>(take((size_t)s.WB * (s.sp[0].n + s.sp[1].n) * 4));
+    w.bad = reinterpret_cast<unsigned int*>(take((size_t)s.WB * (2 * s.G1 + 1) * 4));
+    w.ymax = w.bad + s.WB;
     for (int q = 0; q < 2; ++q) {
         if (s.sp[q].n == 0) continue;
         w.y[q] = reinterpret_cast<long long*>(take(s.y[q]));
@@ -1156,9 +1174,9 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
     for (long long w0 = 0; w0 < W; w0 += s.WB) {
         const long long wb = std::min(s.WB, W - w0);
         const long long rt = (wb * 2 * d.nt + 127) / 128;
-        fd_phi_image_kernel<BITS><<<(unsigned)rt, 256, 0, st>>>(d.N, d.nt, s.KCX, w0, wb, phi, w.pimg, w.pexp);
+        if ((e = cudaMemsetAsync(w.bad, 0, (size_t)(s.WB + wb * 2 * s.G1) * 4, st)) != cudaSuccess) return e;
+        fd_phi_image_kernel<BITS><<<(unsigned)rt, 256, 0, st>>>(d.N, d.nt, s.KCX, w0, wb, phi, w.pimg, w.cexp, w.bad);
         count_launches(1);
-        if ((e = cudaMemsetAsync(w.ymax, 0, (size_t)wb * 2 * s.G1 * 4, st)) != cudaSuccess) return e;
         // runs of matrices: about four blocks per SM, at least four matrices each
         const int want = (int)std::max(1LL, std::min<long long>((4LL * sms + rt - 1) / rt, (s.G1 + 3) / 4));
         const int gpb = (s.G1 + want - 1) / want, ngb = (s.G1 + gpb - 1) / gpb;
@@ -1171,7 +1189,7 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
             const FdSpin& f = s.sp[q];
             if (f.n == 0) continue;
             fd_b_image_kernel<BITS><<<(unsigned)(wb * f.MT), FDB_T, bsm[q], st>>>(d.N, s.N8, d.nt, q ? d.nu : 0, f.n, d.P, f.PB,
-                                                                         f.MT, s.KC, s.zbits, w0, Bm, w.aimg[q],
+                                                                         f.MT, s.KC, s.zbits, w0, w.cexp, Bm, w.aimg[q],
                                                                          w.bexp[q], w.bsh[q], list, bsm[q] > 0);
             FdZArgs a;
             a.n = f.n; a.G1 = s.G1; a.N8 = s.N8; a.KC = s.KC; a.ksteps = s.zsteps; a.NT = f.NT; a.nbuf = f.nbuf; a.ngrp = f.ngrp; a.GB = f.GB;
@@ -1183,7 +1201,7 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
             a.RUN = seg * FD_SEG;
             a.NRUN = (f.NSEG + seg - 1) / seg;
             a.pairs = wb * d.P;
-            a.Bimg = w.aimg[q]; a.bexp = w.bexp[q]; a.bsh = w.bsh[q]; a.pexp = w.pexp; a.xexp = w.xexp;
+            a.Bimg = w.aimg[q]; a.bexp = w.bexp[q]; a.bsh = w.bsh[q]; a.bad = w.bad; a.xexp = w.xexp;
             a.Y = w.y[q]; a.ymax = w.ymax + (size_t)q * s.G1;
             a.vpart = w.vpart[q]; a.expart = w.expart[q]; a.status = status;
             a.listed = list.count ? list.count + w0 : nullptr;

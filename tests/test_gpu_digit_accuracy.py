@@ -1,9 +1,12 @@
 """The FP64 contraction as integer digit products against 64-bit values computed
 here from their definition (Theta = phi (Phi^T phi)^-1, M_g = Phi^T X_g Theta), over
-the sizes where its tiles and digits change."""
+the sizes where its tiles and digits change and over walkers whose columns differ
+in norm (Theta does not depend on the scale of a column of phi)."""
 
 import numpy as np
 import pytest
+
+import afqmc_inputs as ai
 
 pytestmark = pytest.mark.gpu
 
@@ -35,8 +38,10 @@ def _noalloc(h, L, Phi, phi, P, n_up):
 
 
 def _values(h, L, Phi, phi, P, n_up):
-    """The same from the definition, and what the sums of the local energy add up to in absolute value."""
+    """The same from the definition, with the scale of every column of phi taken out first
+    (powers of two: exact), and what the sums of the local energy add up to in absolute value."""
     nt = phi.shape[2]
+    phi = phi / np.exp2(np.round(np.log2(np.linalg.norm(phi, axis=1, keepdims=True))))
     X = np.concatenate([h[None], L])
     e, v, size = [], [], []
     for p, F in enumerate(Phi):
@@ -85,7 +90,7 @@ SIZES = [
 ]
 
 
-def _check(N, nu, nd, G, W, P, seed):
+def _check(N, nu, nd, G, W, P, scale, seed):
     """Tolerance 1e-13 of the sums of absolute values: both sides round at 2^-53 (the reference at
     every sum and in the inverse, whose condition is below 1e2 here)."""
     rng = np.random.default_rng(seed)
@@ -100,6 +105,7 @@ def _check(N, nu, nd, G, W, P, seed):
             cond = np.linalg.cond(Phi[:, :, :n].transpose(0, 2, 1) @ np.repeat(spin, P, axis=0))
             assert np.max(cond) < 1e2
     assert N * G > 128                                                    # the digit products run
+    phi = phi * scale(rng, phi.shape[2])[None, None, :]
     _, e, v = _noalloc(h, L, Phi, phi, P, nu)
     we, wv, size = _values(h, L, Phi, phi, P, nu)
     assert np.max(np.abs(e - we) / size) < 1e-13
@@ -108,7 +114,35 @@ def _check(N, nu, nd, G, W, P, seed):
 
 @pytest.mark.parametrize("N,nu,nd,G,W,P", SIZES)
 def test_digit_contraction_has_64_bit_accuracy(N, nu, nd, G, W, P):
-    _check(N, nu, nd, G, W, P, 100 + N)
+    _check(N, nu, nd, G, W, P, lambda rng, n: np.ones(n), 100 + N)
+
+
+@pytest.mark.parametrize("N,nu,nd,G,W,P", SIZES)
+def test_columns_of_unequal_norm_keep_the_accuracy(N, nu, nd, G, W, P):
+    """Norms from 1e-6 to 1 (and, in turn, one column far beyond), not powers of two."""
+    _check(N, nu, nd, G, W, P, lambda rng, n: 10.0 ** -rng.uniform(0, 6, n), 200 + N)
+    _check(N, nu, nd, G, W, P, lambda rng, n: np.where(np.arange(n) == n - 1, 3e-40, 1.0), 300 + N)
+
+
+def test_context_of_unequal_columns_keeps_the_accuracy():
+    """The same through a loaded state and the FP64 measurement."""
+    N, nu, nd, G, W, P, K = 20, 5, 4, 30, 3, 6, 3
+    rng = np.random.default_rng(9)
+    s = ai.make_system(ai.SystemSpec(N, nu, nd, G, K, True, 77))
+    phi = np.concatenate([_orthonormal(rng, W, N, nu), np.zeros((W, N, nd))], axis=2)
+    phi[:, :, nu:] = phi[:, :, :nd]
+    Phi = _pairs_near(rng, phi, P, N, nu)
+    phi = phi * 10.0 ** -rng.uniform(0, 6, nu + nd)
+    cfg = lib.make_config(N, nu, nd, G, K, W, P, 0.005, 3, n_burn=0)
+    assert lib.fp64_digits(cfg)
+    ctx = lib.Context(cfg, s.h, s.L, s.Phi0, s.U)
+    ctx.load_state_arrays(dict(step=0, phi_up=phi[:, :, :nu], phi_dn=phi[:, :, nu:], weight=np.ones(W),
+                               x=np.zeros((W, P, K)), Phi=Phi.reshape(W, P, N, nu)))
+    ctx.energy()
+    e = ctx.observables()["e_local"].reshape(-1)
+    ctx.close()
+    we, _, size = _values(s.h, s.L, Phi, phi, P, nu)
+    assert np.max(np.abs(e - we) / size) < 1e-13
 
 
 def test_trace_of_z_at_the_ends_of_its_low_half():
