@@ -303,10 +303,12 @@ __global__ void __launch_bounds__(256) chebyshev_expm_df_list_kernel(int N, int 
 // columns 4.87 ms against 17.1, 4096 of them 1.30 against 4.36, 1024 of 8 and 4 0.064 against
 // 0.111 (the Lanczos run and the coefficients then); errors against 64 bits as before (2e-15).
 //
-// The interval's estimate may miss part of the spectrum; with at most FX_GROW half-widths
-// of Gershgorin's bound in it no step overflows before the check on the growth of V (its
-// norm, each column in its own units, and each entry) ends the attempt.  Problems
-// outside that, and non-finite or extreme values, take the FP64 recurrence.
+// The interval's estimate may miss part of the spectrum.  V is checked after every step, in 64 bits: an
+// entry beyond its column's bound (FX_LIMIT, one unit) or a norm above its limit ends the attempt.  Until then no
+// step overflows: Gershgorin's bound lies within FX_GROW half-widths, so the rows of t have
+// absolute sums of at most FX_GROW, and |2 t V_(k-1) - V_(k-2)| <= 13 units < 2^62; the sums of
+// t's low halves stay below 2^27 2^30 sqrt(N) ||V||, with the norm's limit (below 63^2 / N) less than 2^63.
+// Problems outside that, and non-finite or extreme values, take the FP64 recurrence.
 // The FP64 recurrence, out of line: its registers are not the fixed-point loop's.
 __device__ __noinline__ void cheb_fp64_problem(ChebShared& sh, long long prob, int N, int nu, const double* S_all,
                                                const double* Phi0, double* Out, const int* alive, int P, int* status) {
@@ -314,7 +316,7 @@ __device__ __noinline__ void cheb_fp64_problem(ChebShared& sh, long long prob, i
 }
 
 constexpr double FX_GROW = 6.0;
-constexpr int FX_LIMIT = 1 << 30;   // largest high part of an entry of V: its column's bound
+constexpr long long FX_LIMIT = 1ll << 58;   // largest entry of V: its column's bound
 
 __device__ __forceinline__ int2 fx_split(long long v) {
     const int l = ((int)v << 4) >> 4;
@@ -365,7 +367,8 @@ __global__ void __launch_bounds__(512) chebyshev_expm_fix_kernel(int N, int nu, 
         const float f = ldexpf((float)Phi0[e], -colb[e % nu]);
         ps = fmaf(f, f, ps);
     }
-    const float grow_limit = 1.5625f * block_sum_f(ps, sh.sc.red8) + 1e-6f;   // 1.25 of the norm of Phi0, columns scaled
+    // 1.25 of the norm of Phi0, columns scaled (0.8 at most each: the second limit is above that norm by itself)
+    const float grow_limit = fminf(1.5625f * block_sum_f(ps, sh.sc.red8) + 1e-6f, 3969.f / (float)N);
 
     for (int attempt = 0; attempt < 2; ++attempt) {
         const double c = attempt == 0 ? sh.sc.est_c : sh.sc.gers_c, rho = attempt == 0 ? sh.sc.est_rho : sh.sc.gers_rho;
@@ -451,7 +454,7 @@ __global__ void __launch_bounds__(512) chebyshev_expm_fix_kernel(int N, int nu, 
                     if (cg * C + q < nu) {
                         const float f = (float)w.x * 0x1p-30f;
                         ss = fmaf(f, f, ss);
-                        if (abs(w.x) > FX_LIMIT) ss = INFINITY;
+                        if (v > FX_LIMIT || v < -FX_LIMIT) ss = INFINITY;   // before the high part is cut to 32 bits
                     }
                 }
             }
