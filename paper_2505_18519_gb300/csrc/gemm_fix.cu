@@ -13,7 +13,8 @@
 // partial sums at 2^-53.
 //
 // What bounds it: that pipe (15 multiply-adds per clock and SM), 3 R^2 of them a thread and k for
-// 2 R shared-memory reads.  Against the FP64 GEMM (0.8 of the FP64 pipe) on one GB300:
+// 2 R shared-memory reads; few rows, whose tiles of 64 x 64 leave SMs idle, take smaller ones (the sums are
+// integers: the same for every tile).  Against the FP64 GEMM (0.8 of the FP64 pipe) on one GB300:
 // S of 16384 paths, 50 orbitals and variables 4.41 -> 1.41 ms, of 4096 1.11 -> 0.37; the planes of
 // 512 walkers, 250 fields 1.30 -> 0.43.
 #include <algorithm>
@@ -25,7 +26,7 @@ namespace afq {
 
 namespace {
 
-constexpr int GF_R = 4, GF_T = 16 * GF_R, GF_K = 16;
+constexpr int GF_K = 16;
 
 // exponent e with |m| 2^-e < 1 of the largest |entry| m
 __device__ __forceinline__ int gf_exp(double m) { return m > 0.0 ? ilogb(m) + 1 : 0; }
@@ -49,56 +50,59 @@ __global__ void gf_colexp_kernel(int K, long long Nc, const double* __restrict__
     }
 }
 
+// 16 R x 16 R output tile per block, R x R per thread.
+template <int R>
 __global__ void __launch_bounds__(256) gemm_fix_kernel(int M, long long Nc, int K, const double* __restrict__ X,
                                                        const double* __restrict__ U, const int* __restrict__ uexp,
                                                        double* __restrict__ C, int bx, int bu) {
-    __shared__ int2 Xs[GF_K][GF_T + 1], Us[GF_K][GF_T];
-    __shared__ int xe[GF_T], ue[GF_T];
+    constexpr int T = 16 * R, TPR = 256 / T;
+    __shared__ int2 Xs[GF_K][T + 1], Us[GF_K][T];
+    __shared__ int xe[T], ue[T];
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    const long long row0 = (long long)blockIdx.y * GF_T, col0 = (long long)blockIdx.x * GF_T;
-    {   // exponents of the tile's rows: four threads a row
-        const long long r = row0 + tid / 4;
+    const long long row0 = (long long)blockIdx.y * T, col0 = (long long)blockIdx.x * T;
+    {   // exponents of the tile's rows: TPR threads a row
+        const long long r = row0 + tid / TPR;
         double m = 0.0;
         bool bad = false;
         if (r < M)
-            for (int k = tid & 3; k < K; k += 4) {
+            for (int k = tid % TPR; k < K; k += TPR) {
                 const double v = fabs(X[r * K + k]);
                 bad |= !isfinite(v);
                 m = fmax(m, v);
             }
 #pragma unroll
-        for (int o = 1; o < 4; o <<= 1) {
+        for (int o = 1; o < TPR; o <<= 1) {
             m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
             bad |= __shfl_xor_sync(0xffffffffu, (int)bad, o) != 0;
         }
-        if ((tid & 3) == 0) xe[tid / 4] = bad ? DG64_NAN : gf_exp(m);
-        if (tid < GF_T) ue[tid] = col0 + tid < Nc ? uexp[col0 + tid] : 0;
+        if (tid % TPR == 0) xe[tid / TPR] = bad ? DG64_NAN : gf_exp(m);
+        if (tid < T) ue[tid] = col0 + tid < Nc ? uexp[col0 + tid] : 0;
     }
     __syncthreads();
-    long long h[GF_R][GF_R] = {}, x[GF_R][GF_R] = {};
+    long long h[R][R] = {}, x[R][R] = {};
     for (int k0 = 0; k0 < K; k0 += GF_K) {
 #pragma unroll
-        for (int q = 0; q < GF_K * GF_T / 256; ++q) {
+        for (int q = 0; q < R; ++q) {
             const int e = tid + q * 256;
-            const int r = e / GF_K, kk = e % GF_K;              // X tile: 64 rows x 16 k
+            const int r = e / GF_K, kk = e % GF_K;              // X tile: T rows x 16 k
             const long long gr = row0 + r;
             Xs[kk][r] = gr < M && k0 + kk < K ? gf_split(X[gr * K + k0 + kk], 28 + bx - xe[r]) : make_int2(0, 0);
-            const int kb = e / GF_T, c = e % GF_T;              // U tile: 16 k x 64 columns
+            const int kb = e / T, c = e % T;              // U tile: 16 k x T columns
             const long long gc = col0 + c;
             Us[kb][c] = gc < Nc && k0 + kb < K ? gf_split(U[(long long)(k0 + kb) * Nc + gc], 28 + bu - ue[c]) : make_int2(0, 0);
         }
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < GF_K; ++kk) {
-            int2 a[GF_R], b[GF_R];
+            int2 a[R], b[R];
 #pragma unroll
-            for (int i = 0; i < GF_R; ++i) a[i] = Xs[kk][ty + 16 * i];
+            for (int i = 0; i < R; ++i) a[i] = Xs[kk][ty + 16 * i];
 #pragma unroll
-            for (int j = 0; j < GF_R; ++j) b[j] = Us[kk][tx + 16 * j];
+            for (int j = 0; j < R; ++j) b[j] = Us[kk][tx + 16 * j];
 #pragma unroll
-            for (int i = 0; i < GF_R; ++i)
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int j = 0; j < GF_R; ++j) {
+                for (int j = 0; j < R; ++j) {
                     h[i][j] += (long long)a[i].x * b[j].x;
                     x[i][j] += (long long)a[i].x * b[j].y;
                     x[i][j] += (long long)a[i].y * b[j].x;
@@ -106,20 +110,20 @@ __global__ void __launch_bounds__(256) gemm_fix_kernel(int M, long long Nc, int 
         }
         if ((k0 & 48) == 48)                                    // 64 terms: the cross sums stay below 2^62
 #pragma unroll
-            for (int i = 0; i < GF_R; ++i)
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int j = 0; j < GF_R; ++j) {
+                for (int j = 0; j < R; ++j) {
                     h[i][j] += x[i][j] >> 28;
                     x[i][j] &= (1 << 28) - 1;
                 }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < GF_R; ++i) {
+    for (int i = 0; i < R; ++i) {
         const int rl = ty + 16 * i;
         if (row0 + rl >= M) continue;
 #pragma unroll
-        for (int j = 0; j < GF_R; ++j) {
+        for (int j = 0; j < R; ++j) {
             const int cl = tx + 16 * j;
             if (col0 + cl >= Nc) continue;
             const int er = xe[rl], ec = ue[cl];
@@ -133,10 +137,10 @@ __global__ void __launch_bounds__(256) gemm_fix_kernel(int M, long long Nc, int 
 
 }  // namespace
 
-// From this many tiles on the integer pipes are filled; fewer go to the FP64 kernel's small tiles.
-bool gemm_fix_supported(long long M, long long Nc, int K) {
-    return K >= 1 && K <= 4096 && ((M + GF_T - 1) / GF_T) * ((Nc + GF_T - 1) / GF_T) >= 152;
-}
+// By the sizes of U alone: a row's arithmetic does not depend on how many rows a call holds, so blocks of
+// walkers and parts of a batch give the bits of the whole.  Below 12 orbitals there is little to gain (8 orbitals and
+// variables: 16384 rows 39 -> 23 us, but 4.2 -> 6.2 up to 256); at 12 it is 107 -> 53 and 4.2 -> 6.2.
+bool gemm_fix_supported(long long Nc, int K) { return K >= 1 && K <= 4096 && Nc >= 144; }
 
 cudaError_t gemm_fix_prepare(cudaStream_t s, int K, long long Nc, const double* U, int* uexp) {
     if (Nc <= 0 || K <= 0) return cudaSuccess;
@@ -146,12 +150,16 @@ cudaError_t gemm_fix_prepare(cudaStream_t s, int K, long long Nc, const double* 
 }
 
 cudaError_t gemm_fix(cudaStream_t s, int M, long long Nc, int K, const double* X, const double* U, const int* uexp, double* C) {
-    if (!gemm_fix_supported(M, Nc, K)) return cudaErrorInvalidValue;
+    if (!gemm_fix_supported(Nc, K)) return cudaErrorInvalidValue;
+    if (M <= 0) return cudaSuccess;
     int lg = 0;
     while ((1 << lg) < K) ++lg;
     const int b = std::min(58, 62 - lg), bx = b / 2, bu = b - bx;
-    const dim3 grid((unsigned)((Nc + GF_T - 1) / GF_T), (unsigned)((M + GF_T - 1) / GF_T));
-    gemm_fix_kernel<<<grid, 256, 0, s>>>(M, Nc, K, X, U, uexp, C, bx, bu);
+    auto tiles = [&](int t) { return (long long)((Nc + t - 1) / t) * ((M + t - 1) / t); };
+    auto grid = [&](int t) { return dim3((unsigned)((Nc + t - 1) / t), (unsigned)((M + t - 1) / t)); };
+    if (tiles(64) >= 152) gemm_fix_kernel<4><<<grid(64), 256, 0, s>>>(M, Nc, K, X, U, uexp, C, bx, bu);
+    else if (tiles(32) >= 152) gemm_fix_kernel<2><<<grid(32), 256, 0, s>>>(M, Nc, K, X, U, uexp, C, bx, bu);
+    else gemm_fix_kernel<1><<<grid(16), 256, 0, s>>>(M, Nc, K, X, U, uexp, C, bx, bu);
     count_launches(1);
     return cudaGetLastError();
 }

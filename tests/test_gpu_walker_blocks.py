@@ -1,0 +1,65 @@
+"""Results that do not depend on how many rows, walkers or pairs a call holds: every
+arithmetic is chosen by the sizes of the system, so that blocks of walkers (a sharded run) and part
+of a set of samples give the bits of the whole."""
+
+import numpy as np
+import pytest
+
+import afqmc_inputs as ai
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2505_18519_gb300 import afqmc as lib  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2505_18519_gb300 import build
+    build.build()
+    lib.load_library()
+
+
+def _blocks(spec, W, blocks, P, steps=2, **kw):
+    s = ai.make_system(spec)
+    def ctx(w, off):
+        cfg = lib.make_config(spec.N, spec.n_up, spec.n_dn, spec.n_chol, spec.K, w, P, 0.005, 4321, n_burn=2,
+                              walker_offset=off, **kw)
+        return lib.Context(cfg, s.h, s.L, s.Phi0, s.U)
+    cuts = np.cumsum([0] + blocks)
+    assert cuts[-1] == W
+    whole, parts = ctx(W, 0), [ctx(b, int(o)) for b, o in zip(blocks, cuts)]
+    for c in [whole] + parts:
+        c.step(steps)
+        c.energy()
+    a, b = whole.state_arrays(), [c.state_arrays() for c in parts]
+    a["e_local"] = whole.observables()["e_local"]
+    for q, c in zip(b, parts):
+        q["e_local"] = c.observables()["e_local"]
+    for c in [whole] + parts:
+        c.close()
+    for key in ("phi_up", "phi_dn", "weight", "x", "Phi", "e_local"):
+        assert np.array_equal(a[key], np.concatenate([q[key] for q in b])), key
+
+
+@pytest.mark.parametrize("spec,W,blocks,P,kw", [
+    (ai.SystemSpec(50, 10, 10, 250, 50, True, 90), 128, [64, 64], 4, {}),             # field planes of 256 and 128 rows
+    (ai.SystemSpec(50, 10, 10, 60, 50, True, 91), 40, [3, 37], 16, {}),               # S of 640, 48 and 592 rows
+    (ai.SystemSpec(8, 4, 4, 32, 8, False, 92), 700, [1, 699], 16, {}),                # the smallest system
+])
+def test_walker_blocks_of_the_fp64_path(spec, W, blocks, P, kw):
+    _blocks(spec, W, blocks, P, **kw)
+
+
+@pytest.mark.parametrize("N,K", [(50, 50), (8, 8), (24, 100)])
+def test_part_of_the_samples(N, K):
+    s = ai.make_system(ai.SystemSpec(N, 3, 2, 4, K, True, 95))
+    x = np.random.default_rng(1).standard_normal((5000, K))
+    ctx = lib.Context(lib.make_config(N, 3, 2, 4, K, 5000, 1, 0.005, 3, n_burn=0), s.h, s.L, s.Phi0, s.U)
+    whole = ctx.trial_orbitals(x)
+    for n in (1, 70, 1000):
+        assert np.array_equal(ctx.trial_orbitals(x[:n]), whole[:n]), n
+    ctx.close()
