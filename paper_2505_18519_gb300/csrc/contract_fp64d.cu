@@ -45,8 +45,9 @@
 // of the same length.  Against quad precision, 8 to 200 orbitals: pair energies 3e-17 to
 // 3e-16 (the FP64 kernels 6e-17 to 6e-16), force bias 1e-16 to 2e-15 (1e-16 to 2e-15).
 //
-// Sums over matrices are taken in segments of a fixed number of column tiles, added
-// in order, so results do not depend on how the work is split.
+// Everything of one (pair, g) is exact up to its rounding to FP64 (v and Tr Z^2, stored), and
+// the sums over g are taken by the last kernel in one order: results do not depend on how the work is split, on the
+// other pairs or on the column tiles.
 #include <algorithm>
 
 #include "digits64.cuh"
@@ -65,7 +66,7 @@ constexpr int FDZ_THREADS = FDZ_FIN + 32;
 constexpr uint32_t FD_ADIG = 16384;       // one digit of a 64-element K chunk of a 128-row operand
 constexpr int FD_MAXS = 9;                // stages of the A ring
 constexpr size_t FD_SMEM_MAX = 225 * 1024;   // dynamic; static use is below 2 KB of 227 KB
-constexpr int FD_SEG = 4;                 // column tiles per partial sum
+constexpr int FD_RUN = 4;                 // column tiles of a block at least
 constexpr uint32_t FD_POLLS = 1u << 26;   // polls before a wait gives up (wait_polls sets the mixed path's)
 
 // Byte offset of the 16-byte unit u (K elements 8u .. 8u + 7) of row r in a K-major
@@ -602,14 +603,13 @@ __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt
 
 // ---------------------------------------------------------------- GEMM-Z and the traces
 struct FdZArgs {
-    int n, G1, N8, KC, ksteps, NT, nbuf, ngrp, GB, NCT, P, PB, MT, S, T, RUN, NRUN, NSEG;
-    long long pairs;                        // of the chunk
+    int n, G1, N8, KC, ksteps, NT, nbuf, ngrp, GB, NCT, P, PB, MT, S, T, RUN, NRUN;
     const uint8_t* Bimg;
     const int *bexp, *bsh, *xexp;
     const unsigned int* bad;                // walkers with a non-finite entry
     const long long* Y;
     const unsigned int* ymax;               // of this spin: entry (wl 2) G1 + g
-    double2 *vpart, *expart;                // [pair][g], [segment][pair]
+    double2 *vpart, *xpart;                 // Tr Z and Tr Z^2 of [pair][g]
     int* status;
     const int* listed;                      // nullable: pairs of each walker (of the chunk), P at most
 };
@@ -662,8 +662,7 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
     const int combos = A.PB * GB, parts = A.T > 32 ? A.T / 32 : 1;
     int2* Ms = reinterpret_cast<int2*>(ring + (size_t)S * FD_ADIG);
     FdRed* red = reinterpret_cast<FdRed*>(Ms + A.ngrp * 128 * (ldc + 1));   // [2][combos parts]
-    double2* sex = reinterpret_cast<double2*>(red + 2 * combos * parts);
-    uchar2* tab = reinterpret_cast<uchar2*>(sex + combos);
+    uchar2* tab = reinterpret_cast<uchar2*>(red + 2 * combos * parts);
     __shared__ FdPipe pp;
     __shared__ uint64_t rfull[2], rempty[2];
     __shared__ int sbexp[64], sbsh[64];
@@ -732,7 +731,6 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
     } else if (warp >= FDZ_FIN / 32) {
         // ---- the sums of a tile to FP64: lane q takes the (pair, g) q, q + 32, ..
         const bool bad = A.bad[wl] != 0;
-        for (int q = lane; q < combos; q += 32) sex[q] = cmk(0.0, 0.0);
         for (int t = t0; t < t1; ++t) {
             const int rb = (t - t0) & 1, use = (t - t0) >> 1;
             const int gn = min(GB, G1 - t * GB);
@@ -771,20 +769,10 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
                     ex = cmk(xr * f1 * f2 * f1 * f2, xi * f1 * f2 * f1 * f2);
                 }
                 A.vpart[(lp0 + pl) * (long long)G1 + g] = v;
-                if (g > 0) sex[q] = cadd(sex[q], ex);
+                A.xpart[(lp0 + pl) * (long long)G1 + g] = ex;
             }
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&rempty[rb]);
-            if ((t + 1) % FD_SEG == 0 || t + 1 == t1) {               // a segment ends: its sum per pair
-                for (int p = lane; p < np; p += 32) {
-                    double2 x = sex[p * GB];
-                    for (int q = 1; q < GB; ++q) x = cadd(x, sex[p * GB + q]);
-                    A.expart[(long long)(t / FD_SEG) * A.pairs + lp0 + p] = x;
-                }
-                __syncwarp();
-                for (int q = lane; q < combos; q += 32) sex[q] = cmk(0.0, 0.0);
-                __syncwarp();
-            }
         }
         if (failed && lane == 0) atomicOr(A.status, STATUS_TIMEOUT);
     } else if (warp >= FDY_THREADS / 32) {
@@ -957,7 +945,7 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
 // One warp per pair of the chunk (pair0 the first): v_g = sum_s Tr Z_s (g >= 1),
 // E_L = sum_s Tr Z_{s,0} + 1/2 sum_g [v_g^2 - sum_s Tr Z_{s,g}^2].  With a list (w0 the chunk's
 // first walker) pair i of a walker is its listed pair i.
-__global__ void fd_finish_kernel(long long pair0, long long pairs, int P, long long w0, PairList list, int G, int two_spins, int nseg0, int nseg1,
+__global__ void fd_finish_kernel(long long pair0, long long pairs, int P, long long w0, PairList list, int G, int two_spins,
                                  const double2* __restrict__ vp0, const double2* __restrict__ vp1,
                                  const double2* __restrict__ ex0, const double2* __restrict__ ex1,
                                  double2* __restrict__ vpair, double2* __restrict__ epair) {
@@ -971,19 +959,19 @@ __global__ void fd_finish_kernel(long long pair0, long long pairs, int P, long l
         if (i >= list.count[w]) return;
         out = list.items[list.base[w] + i];
     }
-    const double2* a = vp0 + p * (G + 1);
-    const double2* b = vp1 + p * (G + 1);
+    const double2 *a = vp0 + p * (G + 1), *b = vp1 + p * (G + 1);
+    const double2 *xa = ex0 + p * (G + 1), *xb = ex1 + p * (G + 1);
     double2 s = cmk(0.0, 0.0);
     for (int g = 1 + lane; g <= G; g += 32) {
-        double2 v = a[g];
-        if (two_spins) v = cadd(v, b[g]);
+        double2 v = a[g], x = xa[g];
+        if (two_spins) {
+            v = cadd(v, b[g]);
+            x = cadd(x, xb[g]);
+        }
         vpair[out * G + (g - 1)] = v;
-        cfma(s, v, v);
-    }
-    for (int q = lane; q < nseg0 + nseg1; q += 32) {
-        const double2 x = q < nseg0 ? ex0[(long long)q * pairs + p] : ex1[(long long)(q - nseg0) * pairs + p];
-        s.x -= x.x;
-        s.y -= x.y;
+        const double2 v2 = cmul(v, v);
+        s.x += v2.x - x.x;
+        s.y += v2.y - x.y;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1001,7 +989,7 @@ __global__ void fd_finish_kernel(long long pair0, long long pairs, int P, long l
 namespace {
 
 struct FdSpin {
-    int n, PB, MT, GB, NT, nbuf, ngrp, NCT, S, T, NSEG;
+    int n, PB, MT, GB, NT, nbuf, ngrp, NCT, S, T;
     size_t smem, aimg;          // A image bytes per walker
 };
 
@@ -1017,7 +1005,7 @@ inline int fd_up(int x, int m) { return (x + m - 1) / m * m; }
 
 size_t fd_z_smem(int D, int NT, int GB, int n, int PB, int T, int S, int ngrp) {
     return 1024 + 2 * (size_t)fd_bslot(D, NT) + (size_t)S * FD_ADIG + (size_t)ngrp * 128 * (((GB * n) | 1) + 1) * 8 +
-           (size_t)PB * GB * ((T > 32 ? T / 32 : 1) * 2 * sizeof(FdRed) + 16) + (size_t)fd_up(n * (n + 1), 16);
+           (size_t)PB * GB * (T > 32 ? T / 32 : 1) * 2 * sizeof(FdRed) + (size_t)fd_up(n * (n + 1), 16);
 }
 
 // Clocks per column of a column tile, by which tiles are compared (K step of 16): the
@@ -1061,7 +1049,6 @@ bool fd_spin(const FdShape& s, int n, int P, FdSpin& f) {
                 f.GB = gb; f.NT = NT; f.nbuf = nbuf; f.ngrp = ngrp; f.S = S; f.T = T;
                 f.smem = fd_z_smem(s.D, NT, gb, n, f.PB, T, S, ngrp);
                 f.NCT = (s.G1 + gb - 1) / gb;
-                f.NSEG = (f.NCT + FD_SEG - 1) / FD_SEG;
             }
         }
     }
@@ -1097,7 +1084,7 @@ bool fd_shape(int N, int nu, int nd, int G, long long W, int P, size_t chunk, Fd
     size_t per = 0;
     for (int q = 0; q < 2; ++q) {
         const size_t y = (size_t)s.G1 * s.sp[q].n * 2 * s.N8 * 8;
-        per += y + s.sp[q].aimg + (size_t)P * 16 * (s.G1 + s.sp[q].NSEG);
+        per += y + s.sp[q].aimg + (size_t)P * 32 * s.G1;
     }
     s.WB = std::max(1LL, std::min(W, (long long)(chunk / per)));
     for (int q = 0; q < 2; ++q) {
@@ -1116,7 +1103,7 @@ struct FdWork {
     int *xexp, *cexp, *bexp[2], *bsh[2];
     long long* y[2];
     unsigned int *ymax, *bad;   // cleared together
-    double2 *vpart[2], *expart[2];
+    double2 *vpart[2], *xpart[2];
     size_t total;
 };
 
@@ -1143,7 +1130,7 @@ FdWork fd_carve(void* work, const FdShape& s, int P) {
         w.bexp[q] = reinterpret_cast<int*>(take(wp * 4));
         w.bsh[q] = reinterpret_cast<int*>(take(wp * 4));
         w.vpart[q] = reinterpret_cast<double2*>(take(wp * s.G1 * 16));
-        w.expart[q] = reinterpret_cast<double2*>(take(wp * s.sp[q].NSEG * 16));
+        w.xpart[q] = reinterpret_cast<double2*>(take(wp * s.G1 * 16));
     }
     return w;
 }
@@ -1193,17 +1180,15 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
                                                                          w.bexp[q], w.bsh[q], list, bsm[q] > 0);
             FdZArgs a;
             a.n = f.n; a.G1 = s.G1; a.N8 = s.N8; a.KC = s.KC; a.ksteps = s.zsteps; a.NT = f.NT; a.nbuf = f.nbuf; a.ngrp = f.ngrp; a.GB = f.GB;
-            a.NCT = f.NCT; a.P = d.P; a.PB = f.PB; a.MT = f.MT; a.S = f.S; a.T = f.T; a.NSEG = f.NSEG;
-            // whole segments per block: about eight blocks per SM while a block keeps a segment
+            a.NCT = f.NCT; a.P = d.P; a.PB = f.PB; a.MT = f.MT; a.S = f.S; a.T = f.T;
+            // about eight blocks per SM, of FD_RUN column tiles at least
             const long long wm = wb * f.MT;
-            const long long runs = std::max(1LL, std::min<long long>(f.NSEG, (8LL * sms + wm - 1) / wm));
-            const int seg = (int)((f.NSEG + runs - 1) / runs);
-            a.RUN = seg * FD_SEG;
-            a.NRUN = (f.NSEG + seg - 1) / seg;
-            a.pairs = wb * d.P;
+            const long long runs = std::max(1LL, std::min<long long>((f.NCT + FD_RUN - 1) / FD_RUN, (8LL * sms + wm - 1) / wm));
+            a.RUN = (int)((f.NCT + runs - 1) / runs);
+            a.NRUN = (f.NCT + a.RUN - 1) / a.RUN;
             a.Bimg = w.aimg[q]; a.bexp = w.bexp[q]; a.bsh = w.bsh[q]; a.bad = w.bad; a.xexp = w.xexp;
             a.Y = w.y[q]; a.ymax = w.ymax + (size_t)q * s.G1;
-            a.vpart = w.vpart[q]; a.expart = w.expart[q]; a.status = status;
+            a.vpart = w.vpart[q]; a.xpart = w.xpart[q]; a.status = status;
             a.listed = list.count ? list.count + w0 : nullptr;
             contract_fp64d_kernel<BITS><<<(unsigned)(wm * a.NRUN), FDZ_THREADS, f.smem, st>>>(a, FD_POLLS);
             count_launches(2);
@@ -1211,8 +1196,8 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
         }
         const long long pairs = wb * d.P;
         fd_finish_kernel<<<(unsigned)((pairs * 32 + 255) / 256), 256, 0, st>>>(
-            w0 * d.P, pairs, d.P, w0, list, d.G, d.nd > 0, s.sp[0].NSEG, d.nd > 0 ? s.sp[1].NSEG : 0, w.vpart[0],
-            d.nd > 0 ? w.vpart[1] : w.vpart[0], w.expart[0], d.nd > 0 ? w.expart[1] : w.expart[0], vpair, epair);
+            w0 * d.P, pairs, d.P, w0, list, d.G, d.nd > 0, w.vpart[0], d.nd > 0 ? w.vpart[1] : w.vpart[0], w.xpart[0],
+            d.nd > 0 ? w.xpart[1] : w.xpart[0], vpair, epair);
         count_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

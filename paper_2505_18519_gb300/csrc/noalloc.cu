@@ -18,7 +18,7 @@
 // The contraction runs as integer digit products on the tensor cores
 // (contract_fp64d: the FP64 accuracy of the FP64 kernel) when the digits of h and L,
 // formed again by every call, and the work of one walker fit the second array, else (and for the
-// smallest batches of the smallest systems) as the FP64 kernel.  On one GB300: 1024 pairs of 50
+// smallest systems) as the FP64 kernel.  On one GB300: 1024 pairs of 50
 // orbitals, 32 per walker, 1.71 ms against 30.9 (1 per walker 11.7 against 30.9), one pair 0.34
 // against 4.7; 150 pairs of 120 orbitals 7.5 against 116; 8 orbitals with 32 matrices, one pair 0.14 against
 // 0.21; with 16 matrices, 32 pairs 0.120 against 0.111.
@@ -143,7 +143,13 @@ extern "C" afqmc_status afqmc_local_energy_noalloc(int N, int n_up, int n_dn, in
     part[1].W = part[0].W < d.W;
     part[1].P = std::max(1, (int)(n_pairs - part[0].pairs));
     part[1].pairs = n_pairs - part[0].pairs;
-    bool digits = (long long)N * n_chol > 128 || n_pairs > 128;
+    // by the sizes of the system and the pairs per walker alone, so that part of a batch gives the bits of the whole:
+    // a walker of as many pairs as the scratch takes has to fit, and fewer then do
+    Dims full = d;
+    full.W = 1;
+    full.P = (int)std::min<size_t>(pairs_per_walker, (kNoallocScratchBytes - fixed) / per_pair);
+    full.pairs = full.P;
+    bool digits = (long long)N * n_chol > 128 && full.P > 0 && digit_chunk(full) > 0;
     size_t chunk[2] = {0, 0};
     for (int q = 0; q < 2; ++q)
         if (digits && part[q].W) digits = (chunk[q] = digit_chunk(part[q])) > 0;

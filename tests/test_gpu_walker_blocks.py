@@ -1,6 +1,6 @@
 """Results that do not depend on how many rows, walkers or pairs a call holds: every
-arithmetic is chosen by the sizes of the system, so that blocks of walkers (a sharded run) and part
-of a set of samples give the bits of the whole."""
+arithmetic is chosen by the sizes of the system, so that blocks of walkers (a sharded run), part
+of a set of samples and part of a batch of pairs give the bits of the whole."""
 
 import numpy as np
 import pytest
@@ -63,3 +63,22 @@ def test_part_of_the_samples(N, K):
     for n in (1, 70, 1000):
         assert np.array_equal(ctx.trial_orbitals(x[:n]), whole[:n]), n
     ctx.close()
+
+
+@pytest.mark.parametrize("N,nu,nd,G,P", [(8, 1, 1, 16, 16), (50, 10, 7, 40, 6), (20, 2, 2, 90, 24)])
+def test_part_of_a_batch_of_pairs(N, nu, nd, G, P):
+    rng = np.random.default_rng(2)
+    W = 300 // P
+    s = ai.make_system(ai.SystemSpec(N, nu, nd, G, 3, True, 96))
+    phi = rng.standard_normal((W, N, nu + nd)) + 1j * rng.standard_normal((W, N, nu + nd))
+    Phi = rng.standard_normal((W * P, N, nu))
+    dev = torch.device("cuda")
+    args = [torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in (s.h, s.L, Phi, phi.view(np.float64))]
+    def values(n):
+        out = [torch.empty(2 * k, dtype=torch.float64, device=dev) for k in (n, n, n * G)]
+        lib.local_energy_noalloc(N, nu, nd, G, n, P, *args, *out)
+        return [o.cpu().numpy() for o in out]
+    whole = values(W * P)
+    for n in (1, P - 1, P, 2 * P + 1):
+        for got, want in zip(values(n), whole):
+            assert np.array_equal(got, want[:got.size]), n
