@@ -37,21 +37,18 @@ constexpr double RHO_DF = 6.5;   // largest Gershgorin half-width run in double-
 // ||V_k||_F <= ||Phi0||_F); if they do, the problem is done again on the
 // Gershgorin interval of S, in double-float if its half-width is at most
 // RHO_DF and in FP64 otherwise.
-// One problem per call; the whole block of 256 threads takes part.  s_global (with
+// One problem per call; the whole block takes part.  s_global (with
 // s_is_df): S stays in global memory and is read from there (L2) by every term, for
 // N too large for S in shared memory; shared memory then holds the vectors only.
-__device__ __forceinline__ void cheb_df_problem(long long prob, int N, int nu, const double* __restrict__ S_all,
+// The shared variables are the caller's (coef .. irho).
+__device__ __forceinline__ void cheb_df_problem(double* coef, dfl* coefd, ChebScratch& sc, int& nterms, int& mode,
+                                                dfl& cshift_d, dfl& irho_d, double& cshift, double& irho,
+                                                long long prob, int N, int nu, const double* __restrict__ S_all,
                                                 const double* __restrict__ Phi0, double* __restrict__ Out,
                                                 const int* __restrict__ alive, int P, int* status, int allow_df,
                                                 int s_is_df, int s_global = 0) {
-    extern __shared__ dfl smf[];
-    __shared__ double coef[CHEB_DF_MAX + 2];
-    __shared__ dfl coefd[CHEB_DF_MAX + 2];
-    __shared__ ChebScratch sc;
+    extern __shared__ __align__(16) dfl smf[];
     float* red8 = sc.red8;
-    __shared__ int nterms, mode;
-    __shared__ dfl cshift_d, irho_d;
-    __shared__ double cshift, irho;
     if (alive && !alive[prob / P]) return;
     const double* Sg = S_all + prob * (long long)N * N;
     const dfl* Sgd = reinterpret_cast<const dfl*>(Sg);
@@ -257,7 +254,13 @@ __global__ void __launch_bounds__(256) chebyshev_expm_df_kernel(int N, int nu, c
                                                                 const double* __restrict__ Phi0, double* __restrict__ Out,
                                                                 const int* __restrict__ alive, int P, int* status,
                                                                 int allow_df, int s_is_df, int s_global) {
-    cheb_df_problem(blockIdx.x, N, nu, S_all, Phi0, Out, alive, P, status, allow_df, s_is_df, s_global);
+    __shared__ double coef[CHEB_DF_MAX + 2];
+    __shared__ dfl coefd[CHEB_DF_MAX + 2];
+    __shared__ ChebScratch sc;
+    __shared__ int nterms, mode;
+    __shared__ dfl cshift_d, irho_d;
+    __shared__ double cshift, irho;
+    cheb_df_problem(coef, coefd, sc, nterms, mode, cshift_d, irho_d, cshift, irho, blockIdx.x, N, nu, S_all, Phi0, Out, alive, P, status, allow_df, s_is_df, s_global);
 }
 
 // The problems list[0 .. *count), grid-stride (the tensor-core kernel's redo list).
@@ -267,9 +270,15 @@ __global__ void __launch_bounds__(256) chebyshev_expm_df_list_kernel(int N, int 
                                                                      const int* __restrict__ alive, int P, int* status,
                                                                      int s_is_df, const int* __restrict__ list,
                                                                      const int* __restrict__ count) {
+    __shared__ double coef[CHEB_DF_MAX + 2];
+    __shared__ dfl coefd[CHEB_DF_MAX + 2];
+    __shared__ ChebScratch sc;
+    __shared__ int nterms, mode;
+    __shared__ dfl cshift_d, irho_d;
+    __shared__ double cshift, irho;
     const int n = *count;
     for (int i = blockIdx.x; i < n; i += gridDim.x) {
-        cheb_df_problem(list[i], N, nu, S_all, Phi0, Out, alive, P, status, 1, s_is_df);
+        cheb_df_problem(coef, coefd, sc, nterms, mode, cshift_d, irho_d, cshift, irho, list[i], N, nu, S_all, Phi0, Out, alive, P, status, 1, s_is_df);
         __syncthreads();   // the shared memory is reused by the next problem
     }
 }
@@ -301,66 +310,20 @@ __global__ void __launch_bounds__(256) chebyshev_expm_df_list_kernel(int N, int 
 // absolute sums of at most FX_GROW, and |2 t V_(k-1) - V_(k-2)| <= 13 units < 2^62; the sums of
 // t's low halves stay below 2^27 2^30 sqrt(N) ||V||, with the norm's limit (below 63^2 / N) less than 2^63.
 // Problems outside that, and non-finite or extreme values, take the FP64 recurrence.
-// What the block's threads share.
 struct ChebShared {
     double coef[CHEB_DF_MAX + 2];
-    int2 limbs[CHEB_DF_MAX + 2];    // the coefficients as integers
-    ChebScratch sc;                 // both intervals (cheb_interval)
-    int nterms;
+    dfl coefd[CHEB_DF_MAX + 2];     // the coefficients as integer limbs
+    ChebScratch sc;
+    int nterms, mode;
+    dfl cshift_d, irho_d;
+    double cshift, irho;
 };
 
-// The FP64 recurrence (cheb_df_problem's, on the intervals at hand), out of line: its registers are not
-// the fixed-point loop's.
+// The FP64 recurrence, out of line: its registers are not the fixed-point loop's.
 __device__ __noinline__ void cheb_fp64_problem(ChebShared& sh, long long prob, int N, int nu, const double* S_all,
-                                               const double* Phi0, double* Out, int* status) {
-    extern __shared__ int4 fxm[];
-    const double* Sg = S_all + prob * (long long)N * N;
-    const int tid = threadIdx.x, nth = blockDim.x, nn = N * nu;
-    double* S = reinterpret_cast<double*>(fxm);
-    double* Vp = S + (size_t)N * N;
-    double* Vc = Vp + nn;
-    double* acc = Vc + nn;
-    for (int e = tid; e < N * N; e += nth) S[e] = Sg[e];
-    float ps = 0.f;
-    for (int e = tid; e < nn; e += nth) ps = fmaf((float)Phi0[e], (float)Phi0[e], ps);
-    const float grow_limit = 1.5625f * block_sum_f(ps, sh.sc.red8) + 1e-30f;   // ||V_k||_F <= 1.25 ||Phi0||_F
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        const bool check = attempt == 0;
-        const double c = check ? sh.sc.est_c : sh.sc.gers_c, rho = check ? sh.sc.est_rho : sh.sc.gers_rho, ir = 1.0 / rho;
-        if (tid == 0) sh.nterms = cheb_coefs(c, rho, 1e-18, sh.coef, status);
-        __syncthreads();
-        const int m = sh.nterms;
-        for (int e = tid; e < nn; e += nth) {
-            Vp[e] = Phi0[e];
-            acc[e] = sh.coef[0] * Phi0[e];
-        }
-        __syncthreads();
-        bool grew = false;
-        for (int k = 1; k <= m && !grew; ++k) {
-            const double* V = k == 1 ? Vp : Vc;
-            double* Vd = k == 1 ? Vc : Vp;
-            float ss = 0.f;
-            for (int e = tid; e < nn; e += nth) {
-                const int i = e / nu, a = e - i * nu;
-                double sum = 0.0;
-                for (int j = 0; j < N; ++j) sum = fma(S[(size_t)i * N + j], V[j * nu + a], sum);
-                sum = (sum - c * V[e]) * ir;
-                const double v = k == 1 ? sum : 2.0 * sum - Vp[e];
-                Vd[e] = v;
-                acc[e] = fma(sh.coef[k], v, acc[e]);
-                const float vf = __double2float_rn(v);
-                ss = fmaf(vf, vf, ss);
-            }
-            ss = block_sum_f(ss, sh.sc.red8);                  // ends with a barrier
-            grew = check && ss > grow_limit;                   // uniform across the block
-            if (k >= 2) { double* t = Vp; Vp = Vc; Vc = t; }
-        }
-        __syncthreads();
-        if (grew) continue;                                    // the estimate missed part of the spectrum
-        double* o = Out + prob * (long long)nn;
-        for (int e = tid; e < nn; e += nth) o[e] = acc[e];
-        return;
-    }
+                                               const double* Phi0, double* Out, const int* alive, int P, int* status) {
+    cheb_df_problem(sh.coef, sh.coefd, sh.sc, sh.nterms, sh.mode, sh.cshift_d, sh.irho_d, sh.cshift, sh.irho, prob, N, nu, S_all, Phi0,
+                    Out, alive, P, status, 0, 0);
 }
 
 constexpr double FX_GROW = 6.0;
@@ -376,7 +339,7 @@ __global__ void __launch_bounds__(512) chebyshev_expm_fix_kernel(int N, int nu, 
                                                                  const double* __restrict__ Phi0,
                                                                  double* __restrict__ Out, const int* __restrict__ alive,
                                                                  int P, int* status) {
-    extern __shared__ int4 fxm[];
+    extern __shared__ __align__(16) dfl smf[];
     __shared__ ChebShared sh;
     __shared__ int colb[64];        // b_a
     __shared__ int cexp;            // the coefficients' power of two
@@ -385,7 +348,6 @@ __global__ void __launch_bounds__(512) chebyshev_expm_fix_kernel(int N, int nu, 
     const double* Sg = S_all + prob * (long long)N * N;
     const int tid = threadIdx.x, nth = blockDim.x;
     const int ncg = (nu + C - 1) / C, nup = ncg * C, items = N * ncg;
-    dfl* smf = reinterpret_cast<dfl*>(fxm);
     for (int e = tid; e < N * N; e += nth) smf[e] = df_from(Sg[e]);
     __syncthreads();
     cheb_interval(N, &smf[0].hi, 2, sh.sc);
@@ -436,7 +398,7 @@ __global__ void __launch_bounds__(512) chebyshev_expm_fix_kernel(int N, int nu, 
         }
         __syncthreads();
         const int m = sh.nterms, ce = cexp;
-        int2* ci = sh.limbs;
+        int2* ci = reinterpret_cast<int2*>(sh.coefd);
         const double cu = ldexp(1.0, 58 - ce);
         for (int k = tid; k <= m; k += nth) ci[k] = fx_split(__double2ll_rn(sh.coef[k] * cu));
         __syncthreads();
@@ -523,7 +485,7 @@ __global__ void __launch_bounds__(512) chebyshev_expm_fix_kernel(int N, int nu, 
         return;
     }
     __syncthreads();
-    cheb_fp64_problem(sh, prob, N, nu, S_all, Phi0, Out, status);
+    cheb_fp64_problem(sh, prob, N, nu, S_all, Phi0, Out, alive, P, status);
 }
 
 static size_t fix_smem(int N, int nu, int C) {
