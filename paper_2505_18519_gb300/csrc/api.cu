@@ -403,6 +403,7 @@ static size_t layout(const afqmc_config* c, char* base, Workspace* ws) {
     w.logshift = (double2*)take(W * 16);
     const bool refine = refine_enabled(c);
     w.refine_th2 = refine ? (double*)take(2 * pairs * 8) : nullptr;   // per pair (and spin)
+    w.refine_part = refine && !refine_digits(c) ? take(contract_fp64_listed_part_bytes(d.G, d.pairs)) : nullptr;
     w.refine_items = refine ? (int*)take(pairs * 4) : nullptr;
     w.refine_n = refine ? (int*)take(4) : nullptr;
     w.refine_base = refine ? (int*)take(W * 4) : nullptr;
@@ -704,7 +705,7 @@ static afqmc_status measure(afqmc_ctx* ctx, int part = 0) {
                               w.refine_items, w.refine_n));
         else
             CK(contract_fp64_listed(s, d, w.h, w.L, w.Phi, w.Theta, w.vpair, w.epair, w.refine_items, w.refine_n,
-                                    d.pairs, w.hdf, w.Ldf, w.refine_th2, d.pairs));
+                                    d.pairs, w.hdf, w.Ldf, w.refine_part));
     }
     if ((st = prof_mark(ctx, PH_REFINE)) != AFQMC_OK) return st;
     CK(walker_average(s, d, w.logdet, w.vpair, w.epair, w.logov, w.sumS, w.vbar, w.ebar));
@@ -741,7 +742,10 @@ extern "C" afqmc_status afqmc_init_trial(const afqmc_config* cfg, const double* 
     ctx->cfg = *cfg;
     ctx->d = dims_of(cfg);
     ctx->stream = (cudaStream_t)stream;
-    layout(cfg, (char*)workspace, &ctx->ws);
+    if (layout(cfg, (char*)workspace, &ctx->ws) != need) {   // both passes take the same arrays
+        free(ctx);
+        return fail(AFQMC_ERR_ARG, "workspace layout and size differ");
+    }
     afqmc_status st = AFQMC_OK;
     do {
         const Dims& d = ctx->d;

@@ -185,6 +185,7 @@ struct Workspace {
     double2* logshift;  // W  sum_g (xi xbar - xbar^2/2)
     // error-controlled FP64 refinement of the tensor-core contraction (null when off)
     double* refine_th2;   // W*P   ||Theta_p||_F^2
+    void* refine_part;    // partial sums of the listed pairs (double-float kernel)
     int* refine_items;    // W*P   pairs to recompute in FP64
     int* uexp;            // N*N   FP64 path: exponents of the entries of U_k over k (gemm_fix.cu)
     int* lexp;            // N*N   the same of L_g

@@ -11,6 +11,8 @@
 // Theta does not fit (N = 200 with 40 + 40 electrons needs 256 KB), the SLAB
 // form keeps only the JB rows of Theta that the current column block of L_g
 // multiplies, loaded beside it (the pair's Theta stays in L2 across matrices).
+#include <algorithm>
+
 #include "df.cuh"
 #include "kernels.cuh"
 
@@ -71,21 +73,28 @@ __host__ __device__ __forceinline__ Fp64Layout fp64_layout(int N, int nu, int nd
 // OWN: M entries owned per thread (n_up^2 + n_dn^2 <= OWN * CT); the double-float
 // mode with OWN = 8 fits two blocks per SM (slab layout, at most 128 registers;
 // the FP64 instances keep the same 128-register budget).
-// Runs per listed pair of the split double-float refinement: of 16 and the numbers that fill
-// one to four waves of `blocks` blocks with n pairs (up to 64, eight matrices a run), the one whose waves
-// take the least time, as far as the partial-sum space (part_cap double2 values) holds it.  With 16 for
+// The split double-float refinement: the matrices of a listed pair make units (one matrix each up to 512), the
+// units 32 groups; a unit's terms, the units of a group and the groups are added in order, and a run (one block) takes
+// whole units, so that E_L does not depend on how many other pairs are listed.
+constexpr int RF_GROUPS = 32;
+__host__ __device__ inline int units_of(int G1) { return min(G1, 512); }
+__device__ __forceinline__ int unit_group(int u, int units) { return ((u + 1) * RF_GROUPS - 1) / units; }
+
+// Runs per listed pair: of the numbers that fill one to six waves of `blocks` blocks with n pairs,
+// the one whose waves take the least time (in units).  With 16 for
 // every n, four and eight pairs of 95 and 120 orbitals left three quarters and half of the blocks
 // idle: those two 6.3 -> 2.6 ms; the 18 to 22 pairs a step of 64 x 64 pairs of 120 orbitals
 // (16 runs of 20 pairs: two waves, the second nearly empty) 5.7 -> 4.1.
-__device__ __forceinline__ int split_count(long long n, long long part_cap, long long blocks, int G1) {
-    if (n <= 0) return 1;
-    const long long most = min(part_cap / n, (long long)max(16, min(64, G1 / 8)));
-    long long best = max(1LL, min(16LL, most)), waves = (n * best + blocks - 1) / blocks;
-    for (int k = 1; k <= 4; ++k) {
-        const long long g = min(k * blocks / n, most);
-        if (g >= 1 && k * best < waves * g) {               // k / g < waves / best
+__device__ __forceinline__ int split_count(long long n, long long blocks, int units) {
+    if (n <= 0 || n > REFINE_SPLIT) return 1;
+    long long best = 1, time = (n + blocks - 1) / blocks * units;
+    for (int k = 1; k <= 6; ++k) {
+        const long long g = min(k * blocks / n, (long long)units);
+        if (g < 1) continue;
+        const long long t = (n * g + blocks - 1) / blocks * ((units + g - 1) / g);
+        if (t < time) {
             best = g;
-            waves = k;
+            time = t;
         }
     }
     return (int)best;
@@ -98,9 +107,11 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
                                                            double2* __restrict__ vpair, double2* __restrict__ epair,
                                                            const int* __restrict__ items, const int* __restrict__ n_items,
                                                            const dfl* __restrict__ hdf, const dfl* __restrict__ Ldf,
-                                                           double2* __restrict__ epart, long long part_cap) {
+                                                           double2* __restrict__ epart, int units) {
     extern __shared__ double smc[];
     __shared__ double2 red[CT / 32];
+    __shared__ double2 s_grp, s_sum;   // thread 0's, out of the registers: E_L of the present group, of those before it
+    __shared__ int s_unit;
     const int nt = nu + nd;
     const Fp64Layout lay = fp64_layout(N, nu, nd, JB, SLAB);
     double* sPhi = smc;                                             // N x nu
@@ -122,15 +133,16 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
         if (o < nu * nu) { own_a[r] = o / nu; own_b[r] = o % nu; own_c[r] = o % nu; }
         else { int q = o - nu * nu; own_a[r] = q / nd; own_b[r] = q % nd; own_c[r] = nu + q % nd; }
     }
-    // with epart, the matrices of each listed pair are split into gs runs, one work
+    // with epart, the matrices of each listed pair are split into gs runs of units, one work
     // item each, so that a few listed pairs still fill the GPU
     const long long n_list = items ? (long long)*n_items : (long long)gridDim.x;
-    const int gs = epart ? split_count(n_list, part_cap, gridDim.x, G + 1) : 1;
+    const int gs = DF && epart ? split_count(n_list, gridDim.x, units) : 1;
     const long long n_work = n_list * gs;
     for (long long item = blockIdx.x; item < n_work; item += gridDim.x) {
     const long long pair = items ? (long long)items[item / gs] : item;
     const int run = (int)(item % gs);
-    const int g_begin = -1 + (int)((long long)(G + 1) * run / gs), g_end = -1 + (int)((long long)(G + 1) * (run + 1) / gs);
+    const int unit0 = units * run / gs, unit1 = units * (run + 1) / gs;
+    const int g_begin = -1 + (int)((long long)(G + 1) * unit0 / units), g_end = -1 + (int)((long long)(G + 1) * unit1 / units);
     const double* gPhi = Phi + pair * (long long)N * nu;
     const double2* gTh = Theta + pair * (long long)N * nt;
     dfl* const sPhiD = reinterpret_cast<dfl*>(sPhi);
@@ -147,7 +159,11 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
             if constexpr (DF) sThD[e] = gThD[e];
             else sTh[e] = gTh[e];
         }
-    double2 e_acc = cmk(0.0, 0.0);   // thread 0 accumulates E_L
+    double2 e_acc = cmk(0.0, 0.0);   // thread 0 accumulates E_L (DF: the unit's)
+    if (tid == 0) {
+        s_unit = unit0;
+        s_sum = cmk(0.0, 0.0);
+    }
     __syncthreads();
     for (int g = g_begin; g < g_end; ++g) {
         const double* Lg = (g < 0) ? h : L + (long long)g * N * N;
@@ -297,26 +313,47 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
                 e_acc.x += 0.5 * (v2.x - x.x);
                 e_acc.y += 0.5 * (v2.y - x.y);
             }
+            if constexpr (DF) {
+                const int u = s_unit;
+                if (g + 2 == (int)((long long)(G + 1) * (u + 1) / units)) {   // the unit's last matrix
+                    if (gs > 1) {
+                        epart[item / gs * units + u] = e_acc;
+                    } else {
+                        const int q = unit_group(u, units);
+                        s_grp = u == 0 || unit_group(u - 1, units) != q ? e_acc : cadd(s_grp, e_acc);
+                        if (u + 1 == units || unit_group(u + 1, units) != q) s_sum = cadd(s_sum, s_grp);
+                    }
+                    e_acc = cmk(0.0, 0.0);
+                    s_unit = u + 1;
+                }
+            }
         }
     }
     if (tid == 0) {
-        if (epart) epart[item] = e_acc;
-        else epair[pair] = e_acc;
+        if constexpr (!DF) epair[pair] = e_acc;
+        else if (gs == 1) epair[pair] = s_sum;
     }
     __syncthreads();   // the next item overwrites shared memory
     }
 }
 
-// E_L of the listed pairs from their runs' partial sums, in run order.
+// E_L of the listed pairs from their units' sums: a warp per pair, a lane per group, the groups in order.
 __global__ void refine_sum_kernel(const int* __restrict__ items, const int* __restrict__ n_items,
-                                  const double2* __restrict__ epart, long long part_cap, long long blocks, int G1,
-                                  double2* __restrict__ epair) {
+                                  const double2* __restrict__ epart, long long blocks, int units, double2* __restrict__ epair) {
+    static_assert(RF_GROUPS == 32, "a lane per group");
     const long long n = *n_items;
-    const int gs = split_count(n, part_cap, blocks, G1);
-    for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < n; it += (long long)gridDim.x * blockDim.x) {
-        double2 e = epart[it * gs];
-        for (int r = 1; r < gs; ++r) e = cadd(e, epart[it * gs + r]);
-        epair[items[it]] = e;
+    if (split_count(n, blocks, units) == 1) return;         // summed already
+    const int lane = threadIdx.x & 31, u0 = units * lane / RF_GROUPS, u1 = units * (lane + 1) / RF_GROUPS;
+    const long long warps = (long long)gridDim.x * blockDim.x / 32;
+    for (long long it = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32; it < n; it += warps) {
+        const double2* part = epart + it * units;
+        double2 e = u0 < u1 ? part[u0] : cmk(0.0, 0.0);
+#pragma unroll 4
+        for (int u = u0 + 1; u < u1; ++u) e = cadd(e, part[u]);
+        double2 sum = cmk(0.0, 0.0);
+        for (int q = 0; q < RF_GROUPS; ++q)
+            sum = cadd(sum, cmk(__shfl_sync(0xffffffffu, e.x, q), __shfl_sync(0xffffffffu, e.y, q)));
+        if (lane == 0) epair[items[it]] = sum;
     }
 }
 
@@ -571,8 +608,7 @@ template <bool SLAB, bool DF, int OWN>
 static cudaError_t launch_fp64_shape(cudaStream_t s, const Dims& d, int JB, size_t smem, const double* h,
                                      const double* L, const double* Phi, const double2* Theta, double2* vpair,
                                      double2* epair, long long blocks, const int* items, const int* n_items,
-                                     const dfl* hdf, const dfl* Ldf, double2* epart = nullptr,
-                                     long long part_cap = 0) {
+                                     const dfl* hdf, const dfl* Ldf, double2* epart = nullptr) {
     const void* k = (const void*)contract_fp64_kernel<SLAB, DF, OWN>;
     cudaError_t e = raise_smem_limit(k, smem);
     if (e != cudaSuccess) return e;
@@ -583,15 +619,16 @@ static cudaError_t launch_fp64_shape(cudaStream_t s, const Dims& d, int JB, size
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, CT, smem);
         if (e != cudaSuccess) return e;
         const long long cap = (long long)sms * (per_sm > 0 ? per_sm : 1);
-        if (epart) blocks = blocks * 64;   // up to 64 runs per listed pair
+        if (epart) blocks = blocks * units_of(d.G + 1);   // a run per unit at most
         if (blocks > cap) blocks = cap;
     }
+    const int units = epart ? units_of(d.G + 1) : 1;
     contract_fp64_kernel<SLAB, DF, OWN><<<(unsigned)blocks, CT, smem, s>>>(d.N, d.nu, d.nd, d.G, JB, h, L, Phi, Theta,
                                                                            vpair, epair, items, n_items, hdf, Ldf,
-                                                                           epart, part_cap);
+                                                                           epart, units);
     count_launches(1);
     if (epart) {
-        refine_sum_kernel<<<64, 256, 0, s>>>(items, n_items, epart, part_cap, blocks, d.G + 1, epair);
+        refine_sum_kernel<<<64, 256, 0, s>>>(items, n_items, epart, blocks, units, epair);
         count_launches(1);
     }
     return cudaGetLastError();
@@ -601,7 +638,7 @@ template <bool DF>
 static cudaError_t launch_fp64(cudaStream_t s, const Dims& d, const double* h, const double* L, const double* Phi,
                                const double2* Theta, double2* vpair, double2* epair, long long blocks, const int* items,
                                const int* n_items, const dfl* hdf = nullptr, const dfl* Ldf = nullptr,
-                               double2* epart = nullptr, long long part_cap = 0) {
+                               double2* epart = nullptr) {
     if (DF && (!hdf || !Ldf || !items)) return cudaErrorInvalidValue;
     if (!contract_fp64_supported(d.N, d.nu, d.nd)) return cudaErrorInvalidValue;
     if (blocks <= 0) return cudaSuccess;
@@ -613,9 +650,9 @@ static cudaError_t launch_fp64(cudaStream_t s, const Dims& d, const double* h, c
         const size_t smem = contract_fp64_slab_smem(d.N, d.nu, d.nd, JB);
         if (d.nu * d.nu + d.nd * d.nd <= 8 * CT)
             return launch_fp64_shape<true, true, 8>(s, d, JB, smem, h, L, Phi, Theta, vpair, epair, blocks, items,
-                                                    n_items, hdf, Ldf, epart, part_cap);
+                                                    n_items, hdf, Ldf, epart);
         return launch_fp64_shape<true, true, MAXOWN>(s, d, JB, smem, h, L, Phi, Theta, vpair, epair, blocks, items,
-                                                     n_items, hdf, Ldf, epart, part_cap);
+                                                     n_items, hdf, Ldf, epart);
     }
     const size_t smem = contract_fp64_smem(d.N, d.nu, d.nd, JB);
     if (smem > 220 * 1024)
@@ -634,13 +671,17 @@ cudaError_t contract_fp64(cudaStream_t s, const Dims& d, const double* h, const 
 cudaError_t contract_fp64_listed(cudaStream_t s, const Dims& d, const double* h, const double* L, const double* Phi,
                                  const double2* Theta, double2* vpair, double2* epair, const int* items,
                                  const int* n_items, long long max_items, const void* hdf, const void* Ldf,
-                                 void* part, long long part_cap) {
+                                 void* part) {
     if (!items || !n_items) return cudaErrorInvalidValue;
     if (hdf || Ldf)
         return launch_fp64<true>(s, d, h, L, Phi, Theta, vpair, epair, max_items, items, n_items,
                                  static_cast<const dfl*>(hdf), static_cast<const dfl*>(Ldf),
-                                 static_cast<double2*>(part), part ? part_cap : 0);
+                                 static_cast<double2*>(part));
     return launch_fp64<false>(s, d, h, L, Phi, Theta, vpair, epair, max_items, items, n_items);
+}
+
+size_t contract_fp64_listed_part_bytes(int G, long long pairs) {
+    return (size_t)std::min<long long>(pairs, REFINE_SPLIT) * units_of(G + 1) * sizeof(double2);
 }
 
 }  // namespace afq

@@ -143,10 +143,12 @@ cudaError_t refine_select(cudaStream_t s, const Dims& d, double tol, const doubl
 cudaError_t contract_fp64_listed(cudaStream_t s, const Dims& d, const double* h, const double* L, const double* Phi,
                                  const double2* Theta, double2* vpair, double2* epair, const int* items,
                                  const int* n_items, long long max_items, const void* hdf = nullptr,
-                                 const void* Ldf = nullptr, void* part = nullptr, long long part_cap = 0);
-// (part, part_cap: with the double-float copies, space for part_cap double2 partial
-// sums; each listed pair's matrices are then split into up to 64 runs, one block
-// each, and the runs' sums added in order: a few listed pairs fill the GPU.)
+                                 const void* Ldf = nullptr, void* part = nullptr);
+// (part: with the double-float copies, contract_fp64_listed_part_bytes bytes; the matrices of each listed
+// pair are then split into runs, one block each, while the list is at most REFINE_SPLIT
+// pairs: a few listed pairs fill the GPU.  The sums' order does not depend on the list.)
+constexpr long long REFINE_SPLIT = 2048;
+size_t contract_fp64_listed_part_bytes(int G, long long pairs);
 // Walker-side FP64 form (Y_g = X_g phi_w once per block of a walker's pairs,
 // Z = Phi_p^T Y_g, Q = Z A_p^-1; Tr Q and Tr Q^2 are those of M_g): needs A^-1
 // per pair and spin (overlap_lu with OVL_INVERSE) and the walkers.

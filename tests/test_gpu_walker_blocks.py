@@ -36,13 +36,14 @@ def _blocks(spec, W, blocks, P, steps=2, **kw):
         c.step(steps)
         c.energy()
     a, b = whole.state_arrays(), [c.state_arrays() for c in parts]
-    a["e_local"] = whole.observables()["e_local"]
+    a["e_local"], refined = whole.observables()["e_local"], whole.stats()["refined_pairs"]
     for q, c in zip(b, parts):
         q["e_local"] = c.observables()["e_local"]
     for c in [whole] + parts:
         c.close()
     for key in ("phi_up", "phi_dn", "weight", "x", "Phi", "e_local"):
         assert np.array_equal(a[key], np.concatenate([q[key] for q in b])), key
+    return refined
 
 
 @pytest.mark.parametrize("spec,W,blocks,P,kw", [
@@ -53,6 +54,17 @@ def _blocks(spec, W, blocks, P, steps=2, **kw):
 ])
 def test_walker_blocks_of_the_fp64_path(spec, W, blocks, P, kw):
     _blocks(spec, W, blocks, P, **kw)
+
+
+def test_walker_blocks_of_the_refined_mixed_path():
+    """Refinement of every pair, of parts of them and of none: a refined pair's sum has one order,
+    however many others are listed."""
+    spec = ai.SystemSpec(70, 14, 13, 150, 10, True, 94)
+    W, P = 24, 8
+    counts = [_blocks(spec, W, [1, 5, 18], P, steps=1, precision="fp16x6", refine_tol=tol)
+              for tol in [1e-300] + [10.0 ** (-0.15 * k) for k in range(42, 62)]]
+    listed = 2 * W * P                                    # one measurement of the step and one after it
+    assert counts[0] == listed and sum(0 < n < listed for n in counts) >= 3, counts
 
 
 @pytest.mark.parametrize("N,K", [(50, 50), (8, 8), (24, 100)])
