@@ -67,7 +67,6 @@ constexpr uint32_t FD_ADIG = 16384;       // one digit of a 64-element K chunk o
 constexpr int FD_MAXS = 9;                // stages of the A ring
 constexpr size_t FD_SMEM_MAX = 225 * 1024;   // dynamic; static use is below 2 KB of 227 KB
 constexpr int FD_RUN = 4;                 // column tiles of a block at least
-constexpr uint32_t FD_POLLS = 1u << 26;   // polls before a wait gives up (wait_polls sets the mixed path's)
 
 // Byte offset of the 16-byte unit u (K elements 8u .. 8u + 7) of row r in a K-major
 // 128-byte swizzled region.
@@ -1169,7 +1168,7 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
         const int gpb = (s.G1 + want - 1) / want, ngb = (s.G1 + gpb - 1) / gpb;
         fd_y_kernel<BITS><<<(unsigned)(rt * ngb), FDY_THREADS, s.smem_y, st>>>(
             s.N8, d.nu, d.nd, s.G1, s.KCX, s.ysteps, s.JT, s.NTY, s.ybuf, s.SY, gpb, ngb, s.yres, wb, w.pimg, w.ximg, w.y[0], w.y[1],
-            w.ymax, status, FD_POLLS, list.count ? list.count + w0 : nullptr);
+            w.ymax, status, d.wait_polls, list.count ? list.count + w0 : nullptr);
         count_launches(1);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         for (int q = 0; q < 2; ++q) {
@@ -1190,7 +1189,7 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
             a.Y = w.y[q]; a.ymax = w.ymax + (size_t)q * s.G1;
             a.vpart = w.vpart[q]; a.xpart = w.xpart[q]; a.status = status;
             a.listed = list.count ? list.count + w0 : nullptr;
-            contract_fp64d_kernel<BITS><<<(unsigned)(wm * a.NRUN), FDZ_THREADS, f.smem, st>>>(a, FD_POLLS);
+            contract_fp64d_kernel<BITS><<<(unsigned)(wm * a.NRUN), FDZ_THREADS, f.smem, st>>>(a, d.wait_polls);
             count_launches(2);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
