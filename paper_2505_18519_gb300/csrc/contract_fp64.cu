@@ -74,22 +74,29 @@ __host__ __device__ __forceinline__ Fp64Layout fp64_layout(int N, int nu, int nd
 // mode with OWN = 8 fits two blocks per SM (slab layout, at most 128 registers;
 // the FP64 instances keep the same 128-register budget).
 // The split double-float refinement: the matrices of a listed pair make units (one matrix each up to 512), the
-// units 32 groups; a unit's terms, the units of a group and the groups are added in order, and a run (one block) takes
-// whole units, so that E_L does not depend on how many other pairs are listed.
-constexpr int RF_GROUPS = 32;
-__host__ __device__ inline int units_of(int G1) { return min(G1, 512); }
-__device__ __forceinline__ int unit_group(int u, int units) { return ((u + 1) * RF_GROUPS - 1) / units; }
+// units up to 32 groups; a unit's terms, the units of a group and the groups are added in order, and a run (one block)
+// takes whole units, so that E_L does not depend on how many other pairs are listed.
+struct RefineUnits {
+    int mats, units, group;     // matrices a unit, units, units a group
+    __host__ __device__ explicit RefineUnits(int G1) {
+        mats = (G1 + 511) / 512;
+        units = (G1 + mats - 1) / mats;
+        group = (units + 31) / 32;
+    }
+};
 
-// Runs per listed pair: of the numbers that fill one to six waves of `blocks` blocks with n pairs,
+// Runs per listed pair: of the numbers that fill one to six waves of `blocks` blocks with n pairs (up to 64, eight units a
+// run: shorter ones lose more to their start than they gain beside other systems' kernels),
 // the one whose waves take the least time (in units).  With 16 for
 // every n, four and eight pairs of 95 and 120 orbitals left three quarters and half of the blocks
 // idle: those two 6.3 -> 2.6 ms; the 18 to 22 pairs a step of 64 x 64 pairs of 120 orbitals
 // (16 runs of 20 pairs: two waves, the second nearly empty) 5.7 -> 4.1.
 __device__ __forceinline__ int split_count(long long n, long long blocks, int units) {
     if (n <= 0 || n > REFINE_SPLIT) return 1;
+    const long long most = max(min(units, 16), min(64, units / 8));
     long long best = 1, time = (n + blocks - 1) / blocks * units;
     for (int k = 1; k <= 6; ++k) {
-        const long long g = min(k * blocks / n, (long long)units);
+        const long long g = min(k * blocks / n, most);
         if (g < 1) continue;
         const long long t = (n * g + blocks - 1) / blocks * ((units + g - 1) / g);
         if (t < time) {
@@ -107,7 +114,7 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
                                                            double2* __restrict__ vpair, double2* __restrict__ epair,
                                                            const int* __restrict__ items, const int* __restrict__ n_items,
                                                            const dfl* __restrict__ hdf, const dfl* __restrict__ Ldf,
-                                                           double2* __restrict__ epart, int units) {
+                                                           double2* __restrict__ epart) {
     extern __shared__ double smc[];
     __shared__ double2 red[CT / 32];
     __shared__ double2 s_grp, s_sum;   // thread 0's, out of the registers: E_L of the present group, of those before it
@@ -136,13 +143,14 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
     // with epart, the matrices of each listed pair are split into gs runs of units, one work
     // item each, so that a few listed pairs still fill the GPU
     const long long n_list = items ? (long long)*n_items : (long long)gridDim.x;
-    const int gs = DF && epart ? split_count(n_list, gridDim.x, units) : 1;
+    const RefineUnits ru(G + 1);
+    const int gs = DF && epart ? split_count(n_list, gridDim.x, ru.units) : 1;
     const long long n_work = n_list * gs;
     for (long long item = blockIdx.x; item < n_work; item += gridDim.x) {
     const long long pair = items ? (long long)items[item / gs] : item;
     const int run = (int)(item % gs);
-    const int unit0 = units * run / gs, unit1 = units * (run + 1) / gs;
-    const int g_begin = -1 + (int)((long long)(G + 1) * unit0 / units), g_end = -1 + (int)((long long)(G + 1) * unit1 / units);
+    const int unit0 = ru.units * run / gs, unit1 = ru.units * (run + 1) / gs;
+    const int g_begin = -1 + unit0 * ru.mats, g_end = min(G, -1 + unit1 * ru.mats);
     const double* gPhi = Phi + pair * (long long)N * nu;
     const double2* gTh = Theta + pair * (long long)N * nt;
     dfl* const sPhiD = reinterpret_cast<dfl*>(sPhi);
@@ -314,14 +322,13 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
                 e_acc.y += 0.5 * (v2.y - x.y);
             }
             if constexpr (DF) {
-                const int u = s_unit;
-                if (g + 2 == (int)((long long)(G + 1) * (u + 1) / units)) {   // the unit's last matrix
+                if (ru.mats == 1 || (g + 2) % ru.mats == 0 || g + 1 == G) {   // the unit's last matrix
+                    const int u = s_unit;
                     if (gs > 1) {
-                        epart[item / gs * units + u] = e_acc;
+                        epart[item / gs * ru.units + u] = e_acc;
                     } else {
-                        const int q = unit_group(u, units);
-                        s_grp = u == 0 || unit_group(u - 1, units) != q ? e_acc : cadd(s_grp, e_acc);
-                        if (u + 1 == units || unit_group(u + 1, units) != q) s_sum = cadd(s_sum, s_grp);
+                        s_grp = u % ru.group == 0 ? e_acc : cadd(s_grp, e_acc);
+                        if ((u + 1) % ru.group == 0 || u + 1 == ru.units) s_sum = cadd(s_sum, s_grp);
                     }
                     e_acc = cmk(0.0, 0.0);
                     s_unit = u + 1;
@@ -339,19 +346,18 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
 
 // E_L of the listed pairs from their units' sums: a warp per pair, a lane per group, the groups in order.
 __global__ void refine_sum_kernel(const int* __restrict__ items, const int* __restrict__ n_items,
-                                  const double2* __restrict__ epart, long long blocks, int units, double2* __restrict__ epair) {
-    static_assert(RF_GROUPS == 32, "a lane per group");
+                                  const double2* __restrict__ epart, long long blocks, RefineUnits ru, double2* __restrict__ epair) {
     const long long n = *n_items;
-    if (split_count(n, blocks, units) == 1) return;         // summed already
-    const int lane = threadIdx.x & 31, u0 = units * lane / RF_GROUPS, u1 = units * (lane + 1) / RF_GROUPS;
+    if (split_count(n, blocks, ru.units) == 1) return;      // summed already
+    const int lane = threadIdx.x & 31, u0 = ru.group * lane, u1 = min(ru.units, u0 + ru.group);
     const long long warps = (long long)gridDim.x * blockDim.x / 32;
     for (long long it = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32; it < n; it += warps) {
-        const double2* part = epart + it * units;
+        const double2* part = epart + it * ru.units;
         double2 e = u0 < u1 ? part[u0] : cmk(0.0, 0.0);
 #pragma unroll 4
         for (int u = u0 + 1; u < u1; ++u) e = cadd(e, part[u]);
         double2 sum = cmk(0.0, 0.0);
-        for (int q = 0; q < RF_GROUPS; ++q)
+        for (int q = 0; q < 32; ++q)
             sum = cadd(sum, cmk(__shfl_sync(0xffffffffu, e.x, q), __shfl_sync(0xffffffffu, e.y, q)));
         if (lane == 0) epair[items[it]] = sum;
     }
@@ -619,16 +625,15 @@ static cudaError_t launch_fp64_shape(cudaStream_t s, const Dims& d, int JB, size
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, CT, smem);
         if (e != cudaSuccess) return e;
         const long long cap = (long long)sms * (per_sm > 0 ? per_sm : 1);
-        if (epart) blocks = blocks * units_of(d.G + 1);   // a run per unit at most
+        if (epart) blocks = blocks * 64;   // up to 64 runs per listed pair
         if (blocks > cap) blocks = cap;
     }
-    const int units = epart ? units_of(d.G + 1) : 1;
     contract_fp64_kernel<SLAB, DF, OWN><<<(unsigned)blocks, CT, smem, s>>>(d.N, d.nu, d.nd, d.G, JB, h, L, Phi, Theta,
                                                                            vpair, epair, items, n_items, hdf, Ldf,
-                                                                           epart, units);
+                                                                           epart);
     count_launches(1);
     if (epart) {
-        refine_sum_kernel<<<64, 256, 0, s>>>(items, n_items, epart, blocks, units, epair);
+        refine_sum_kernel<<<64, 256, 0, s>>>(items, n_items, epart, blocks, RefineUnits(d.G + 1), epair);
         count_launches(1);
     }
     return cudaGetLastError();
@@ -681,7 +686,7 @@ cudaError_t contract_fp64_listed(cudaStream_t s, const Dims& d, const double* h,
 }
 
 size_t contract_fp64_listed_part_bytes(int G, long long pairs) {
-    return (size_t)std::min<long long>(pairs, REFINE_SPLIT) * units_of(G + 1) * sizeof(double2);
+    return (size_t)std::min<long long>(pairs, REFINE_SPLIT) * RefineUnits(G + 1).units * sizeof(double2);
 }
 
 }  // namespace afq
