@@ -401,8 +401,12 @@ int afqmc_fp64_digits(const afqmc_config* cfg);
  * a cudaDeviceReset that follows the first call, are not supported.
  * Every call shares the array, so calls that overlap on the GPU race.  A
  * singular overlap gives log|ov| = -inf for that pair (its energy and force
- * bias are then those of a zero Theta; the other pairs are unaffected). */
+ * bias are then those of a zero Theta; the other pairs are unaffected).  If a
+ * wait of the tensor-core kernels runs out (see wait_polls), every output of the call is NaN. */
 size_t afqmc_noalloc_scratch_bytes(void);
+/* wait_polls (see afqmc_config) of the calls of afqmc_local_energy_noalloc that the calling
+ * thread makes from here on; 0: the default. */
+afqmc_status afqmc_noalloc_wait_polls(int64_t polls);
 afqmc_status afqmc_local_energy_noalloc(int N, int n_up, int n_dn, int n_chol, int64_t n_pairs,
                                         int pairs_per_walker, const double* h, const double* L,
                                         const double* Phi, const double* phi, double* logov,

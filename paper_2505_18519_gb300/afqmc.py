@@ -55,7 +55,7 @@ EXPORTS = ("afqmc_config_default", "afqmc_workspace_bytes", "afqmc_init", "afqmc
            "afqmc_launch_count", "afqmc_contract_kernel", "afqmc_fp64_digits", "afqmc_autotune", "afqmc_batch_create", "afqmc_batch_step", "afqmc_batch_sync",
            "afqmc_batch_destroy", "afqmc_mlp_n_params", "afqmc_mlp_params", "afqmc_mlp_eval", "afqmc_mlp_state",
            "afqmc_fp64_fma_rate", "afqmc_local_energy_noalloc", "afqmc_noalloc_scratch_bytes",
-           "afqmc_noalloc_last_error", "afqmc_trial_orbitals", "afqmc_batch_shared_contractions")
+           "afqmc_noalloc_wait_polls", "afqmc_noalloc_last_error", "afqmc_trial_orbitals", "afqmc_batch_shared_contractions")
 
 PHASES = ("overlap", "contract", "average", "fields", "propagate", "ratio", "propose", "trial_orbitals",
           "mcmc_overlap", "accept", "finish", "comb", "refine")
@@ -136,6 +136,8 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.afqmc_mlp_state.restype = I
     lib.afqmc_noalloc_scratch_bytes.argtypes = []
     lib.afqmc_noalloc_scratch_bytes.restype = SZ
+    lib.afqmc_noalloc_wait_polls.argtypes = [ctypes.c_int64]
+    lib.afqmc_noalloc_wait_polls.restype = I
     lib.afqmc_local_energy_noalloc.argtypes = [I, I, I, I, ctypes.c_int64, I, P, P, P, P, P, P, P, P]
     lib.afqmc_local_energy_noalloc.restype = I
     lib.afqmc_fp64_fma_rate.argtypes = [D, P]
@@ -383,6 +385,15 @@ def local_energy_noalloc(N, n_up, n_dn, n_chol, n_pairs, pairs_per_walker, h, L,
     st = lib.afqmc_local_energy_noalloc(N, n_up, n_dn, n_chol, int(n_pairs), pairs_per_walker, h.data_ptr(),
                                         L.data_ptr(), Phi.data_ptr(), phi.data_ptr(), logov.data_ptr(),
                                         e_local.data_ptr(), force_bias.data_ptr(), s.cuda_stream)
+    if st != 0:
+        raise AfqmcError(st, lib.afqmc_noalloc_last_error().decode())
+
+
+def noalloc_wait_polls(polls: int):
+    """Polls before a wait of this thread's later ``local_energy_noalloc`` calls gives up and their
+    outputs become NaN (0: the default)."""
+    lib = load_library()
+    st = lib.afqmc_noalloc_wait_polls(int(polls))
     if st != 0:
         raise AfqmcError(st, lib.afqmc_noalloc_last_error().decode())
 

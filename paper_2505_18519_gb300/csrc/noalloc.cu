@@ -54,6 +54,23 @@ static size_t digit_chunk(const Dims& d) {
 }
 
 static thread_local char g_noalloc_err[256] = "";
+static thread_local uint32_t g_noalloc_polls = 0;   // limit of the calling thread's waits, 0: the default
+
+// log<Phi|phi> of the pairs, and NaN in every output if a wait of the digit products ran out: nobody reads
+// the status word, and what the kernels left out would be the values of an earlier call.
+static __global__ void noalloc_finish_kernel(long long pairs, int G, const int* __restrict__ status,
+                                             const double2* __restrict__ logdet, double2* __restrict__ logov,
+                                             double2* __restrict__ e_local, double2* __restrict__ force_bias) {
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= pairs) return;
+    if (!(*status & STATUS_TIMEOUT)) {
+        logov[p] = cadd(logdet[2 * p], logdet[2 * p + 1]);
+        return;
+    }
+    const double nan = __longlong_as_double(0x7FF8000000000000LL);
+    logov[p] = e_local[p] = cmk(nan, nan);
+    for (int g = 0; g < G; ++g) force_bias[p * G + g] = cmk(nan, nan);
+}
 
 static afqmc_status noalloc_fail(afqmc_status st, const char* msg, cudaError_t e = cudaSuccess) {
     if (e != cudaSuccess)
@@ -66,6 +83,12 @@ static afqmc_status noalloc_fail(afqmc_status st, const char* msg, cudaError_t e
 extern "C" const char* afqmc_noalloc_last_error(void) { return g_noalloc_err; }
 
 extern "C" size_t afqmc_noalloc_scratch_bytes(void) { return kNoallocScratchBytes; }
+
+extern "C" afqmc_status afqmc_noalloc_wait_polls(int64_t polls) {
+    if (polls < 0 || polls > (1ll << 31)) return noalloc_fail(AFQMC_ERR_ARG, "polls must be in [0, 2^31]");
+    g_noalloc_polls = (uint32_t)polls;
+    return AFQMC_OK;
+}
 
 extern "C" afqmc_status afqmc_local_energy_noalloc(int N, int n_up, int n_dn, int n_chol, int64_t n_pairs,
                                                    int pairs_per_walker, const double* h, const double* L,
@@ -131,6 +154,7 @@ extern "C" afqmc_status afqmc_local_energy_noalloc(int N, int n_up, int n_dn, in
     d.P = pairs_per_walker;
     d.W = (int)((n_pairs + pairs_per_walker - 1) / pairs_per_walker);
     d.pairs = n_pairs;
+    if (g_noalloc_polls) d.wait_polls = g_noalloc_polls;
     // the overlap kernel flags singular overlaps in a status word, which lives in
     // the scratch too and is cleared first (a singular pair gets log|ov| = -inf)
     int* status = reinterpret_cast<int*>(static_cast<char*>(base) + status_off);
@@ -173,7 +197,10 @@ extern "C" afqmc_status afqmc_local_energy_noalloc(int N, int n_up, int n_dn, in
         e = contract_fp64(s, d, h, L, Phi, Theta, v, el, n_pairs);
     }
     if (e != cudaSuccess) return noalloc_fail(AFQMC_ERR_CUDA, "contraction kernel", e);
-    e = combine_logdet(s, n_pairs, logdet, reinterpret_cast<double2*>(logov));
+    noalloc_finish_kernel<<<(unsigned)((n_pairs + 255) / 256), 256, 0, s>>>(n_pairs, n_chol, status, logdet,
+                                                                            reinterpret_cast<double2*>(logov), el, v);
+    count_launches(1);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return noalloc_fail(AFQMC_ERR_CUDA, "log-determinant kernel", e);
     return AFQMC_OK;
 }

@@ -49,3 +49,29 @@ def test_digit_kernels_report_a_timeout(spec):
     e = ctx.energy(walkers=True)
     ctx.close()
     assert np.max(np.abs(e["e_walker"] - oa.measure(ham, ost)["e_bar"])) < 1e-9
+
+
+def test_entry_without_allocation_gives_nan_after_a_timeout():
+    """... and not what an earlier call left in its work space; the next call has values again."""
+    N, nu, nd, G, P, n = 50, 10, 9, 60, 8, 20
+    rng = np.random.default_rng(4)
+    dev = torch.device("cuda")
+    s = ai.make_system(ai.SystemSpec(N, nu, nd, G, 3, True, 11))
+    Phi = np.linalg.qr(rng.standard_normal((n, N, nu)))[0]
+    phi = np.concatenate([Phi[::P], Phi[::P][:, :, :nd]], axis=2) + 0.05j * rng.standard_normal((3, N, nu + nd))
+    args = [torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in (s.h, s.L, Phi, phi.view(np.float64))]
+    def values():
+        out = [torch.zeros(2 * k, dtype=torch.float64, device=dev) for k in (n, n, n * G)]
+        lib.local_energy_noalloc(N, nu, nd, G, n, P, *args, *out)
+        return [o.cpu().numpy() for o in out]
+    want = values()
+    assert all(np.all(np.isfinite(o)) for o in want)
+    lib.noalloc_wait_polls(1)
+    try:
+        got = values()
+    finally:
+        lib.noalloc_wait_polls(0)
+    assert all(np.all(np.isnan(o)) for o in got)
+    assert all(np.array_equal(a, b) for a, b in zip(values(), want))
+    with pytest.raises(lib.AfqmcError):
+        lib.noalloc_wait_polls(-1)
