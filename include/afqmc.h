@@ -381,7 +381,8 @@ int afqmc_fp64_digits(const afqmc_config* cfg);
  * array of afqmc_noalloc_scratch_bytes() bytes (32 MiB), and the digits of the
  * tensor-core contraction (FP64 accuracy, see afqmc_fp64_digits; sizes whose digits
  * do not fit run the FP64 kernel) in another of 512 MiB, which a GPU holds from the
- * first call on it until exit; the caller passes only inputs and outputs.
+ * first call on it until exit (a GPU without room for it then runs the FP64 kernel); the
+ * caller passes only inputs and outputs.
  *   h           N*N                      one-body matrix                    device
  *   L           n_chol*N*N               Cholesky vectors                   device
  *   Phi         n_pairs*N*n_up           trial orbitals of each pair        device

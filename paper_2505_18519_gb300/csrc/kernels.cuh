@@ -181,6 +181,10 @@ cudaError_t contract_fp64d(cudaStream_t st, const Dims& d, void* work, const dou
                            double2* vpair, double2* epair, int* status, const PairList& list = PairList(),
                            size_t chunk = FD_CHUNK);
 
+// noalloc_work.cu: the device address of NOALLOC_WORK_BYTES bytes on the current device.
+constexpr size_t NOALLOC_WORK_BYTES = (size_t)512 << 20;
+cudaError_t noalloc_work(void** address);
+
 // contract_tc.cu
 bool contract_tc_supported(int N, int nu, int nd, bool f16);
 size_t contract_tc_image_bytes(int N, int nu, int nd, int G, bool f16);

@@ -17,8 +17,8 @@
 //
 // The contraction runs as integer digit products on the tensor cores
 // (contract_fp64d: the FP64 accuracy of the FP64 kernel) when the digits of h and L,
-// formed again by every call, and the work of one walker fit the second array, else (and for the
-// smallest systems) as the FP64 kernel.  On one GB300: 1024 pairs of 50
+// formed again by every call, and the work of one walker fit the second array (noalloc_work.cu), else (for the
+// smallest systems, and where the GPU had no room for that array at its first call) as the FP64 kernel.  On one GB300: 1024 pairs of 50
 // orbitals, 32 per walker, 1.71 ms against 30.9 (1 per walker 11.7 against 30.9), one pair 0.34
 // against 4.7; 150 pairs of 120 orbitals 7.5 against 116; 8 orbitals with 32 matrices, one pair 0.14 against
 // 0.21; with 16 matrices, 32 pairs 0.120 against 0.111.
@@ -35,21 +35,16 @@ using namespace afq;
 static constexpr size_t kNoallocScratchBytes = 32ull << 20;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
 
-// Work space of the digit products (the digits of h and L take 16 MB at 50 orbitals and 250
-// vectors, 200 MB at 120 and 600), held like the scratch.
-static constexpr size_t kNoallocWorkBytes = 512ull << 20;
-static __device__ __align__(256) unsigned char g_noalloc_work[kNoallocWorkBytes];
-
 static std::mutex g_noalloc_mu;
 static void* g_noalloc_addr[256];        // device addresses of the arrays, per device ordinal
-static void* g_noalloc_work_addr[256];
+static void* g_noalloc_work_addr[256];   // null: no room for the digits' work space at the first call
 
 // Bytes of the work space that hold the walkers worked on together, 0 where the sizes do not fit.
 static size_t digit_chunk(const Dims& d) {
     const size_t least = contract_fp64d_work_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P, 0);
-    if (least == 0 || least > kNoallocWorkBytes) return 0;
-    size_t chunk = kNoallocWorkBytes - least + 1;
-    while (contract_fp64d_work_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P, chunk) > kNoallocWorkBytes) chunk -= chunk / 8 + 1;
+    if (least == 0 || least > NOALLOC_WORK_BYTES) return 0;
+    size_t chunk = NOALLOC_WORK_BYTES - least + 1;
+    while (contract_fp64d_work_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P, chunk) > NOALLOC_WORK_BYTES) chunk -= chunk / 8 + 1;
     return std::max<size_t>(chunk, 1);   // a chunk of one byte is one walker
 }
 
@@ -138,8 +133,12 @@ extern "C" afqmc_status afqmc_local_energy_noalloc(int N, int n_up, int n_dn, in
             e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
             if (e != cudaSuccess) return noalloc_fail(AFQMC_ERR_CUDA, "cudaGetSymbolAddress", e);
             void* q = nullptr;
-            e = cudaGetSymbolAddress(&q, g_noalloc_work);
-            if (e != cudaSuccess) return noalloc_fail(AFQMC_ERR_CUDA, "cudaGetSymbolAddress", e);
+            e = noalloc_work(&q);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                if (e != cudaErrorMemoryAllocation) return noalloc_fail(AFQMC_ERR_CUDA, "cudaGetSymbolAddress", e);
+                q = nullptr;
+            }
             g_noalloc_work_addr[dev] = q;
             g_noalloc_addr[dev] = p;
         }
@@ -173,7 +172,7 @@ extern "C" afqmc_status afqmc_local_energy_noalloc(int N, int n_up, int n_dn, in
     full.W = 1;
     full.P = (int)std::min<size_t>(pairs_per_walker, (kNoallocScratchBytes - fixed) / per_pair);
     full.pairs = full.P;
-    bool digits = (long long)N * n_chol > 128 && full.P > 0 && digit_chunk(full) > 0;
+    bool digits = work && (long long)N * n_chol > 128 && full.P > 0 && digit_chunk(full) > 0;
     size_t chunk[2] = {0, 0};
     for (int q = 0; q < 2; ++q)
         if (digits && part[q].W) digits = (chunk[q] = digit_chunk(part[q])) > 0;
