@@ -376,8 +376,8 @@ static size_t layout(const afqmc_config* c, char* base, Workspace* ws) {
     w.Lt = (tck == 1 || tck == 2) ? take(contract_tc_image_bytes(d.N, d.nu, d.nd, d.G, f16c)) : nullptr;
     w.Yimg = tck == 2 ? take(contract_tcy_yimage_bytes(d.N, d.nu, d.nd, d.G, d.W, f16c)) : nullptr;
     w.tcw = tck == 5 ? take(contract_tcw_work_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P, tc_mode(c))) : nullptr;
-    // FP64: the digit form's work space where it takes the sizes, else the walker-side form's
-    if (c->precision == AFQMC_PRECISION_FP64) {
+    // FP64: the digit form's work space where it takes the sizes, else the walker-side form's; none beside a cache
+    if (c->precision == AFQMC_PRECISION_FP64 && !cache_read(c)) {
         const size_t fd = contract_fp64d_work_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P);
         const size_t ywalk = fd ? 0 : contract_fp64_walker_bytes(d.N, d.nu, d.nd, d.G, d.W, d.P);
         w.fd = fd ? take(fd) : nullptr;
