@@ -72,7 +72,6 @@ __global__ void __launch_bounds__(OT_THREADS)
     const int rows = np * n;
     const long long pair0 = w * P + (long long)m * PB;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int warp_u = __shfl_sync(0xffffffffu, warp, 0);   // the same, known to be uniform
     const float4* ph = phiD + w * (long long)N * nt + col0;   // phi_w[i, b] at ph[i nt + b]
 
     if (warp == 0) {
@@ -169,30 +168,24 @@ __global__ void __launch_bounds__(OT_THREADS)
         tc::fence_before_sync();
         __syncthreads();
         tc::fence_after_sync();
-        if (warp_u == 0) {   // one lane issues, chosen in a converged warp: operands in uniform registers
-            const uint64_t abase = tc::desc_sw128(tc::smem_u32(AD)), bbase = tc::desc_sw128(tc::smem_u32(BD));
-            const uint32_t accb = kb == 0 ? 0u : 1u;
-            __syncwarp();
-            if (tc::elect_one()) {
+        if (tid == 0) {
+            const uint32_t abase = tc::smem_u32(AD), bbase = tc::smem_u32(BD);
+            for (int s = 0; s < 4; ++s) {
 #pragma unroll
-                for (int s = 0; s < 4; ++s) {
-#pragma unroll
-                    for (int i = 0; i < DG_DIG; ++i) {
-                        // digit i of A against B digits 0 .. 4 - i, into accumulators i .. 4 (digit
-                        // 0 first: at the block's first K step it initialises every accumulator);
-                        // maxblk >= 3 (n <= 40), so two MMAs take all five
-                        const int nblk = OT_ORD - i, n1 = min(maxblk, nblk), n2 = nblk - n1;
-                        const uint64_t ad = abase + (uint64_t)((uint32_t)i * (OT_AKB >> 4) + 2u * s);
-                        const uint32_t acc = (s == 0 && i == 0) ? accb : 1u;
-                        tc::mma_f16(taddr + (uint32_t)(i * CB), ad, bbase + 2 * s, tc::idesc_f16_f32(128, n1 * CB), acc);
-                        if (n2 > 0)
-                            tc::mma_f16(taddr + (uint32_t)((i + n1) * CB), ad, bbase + (uint64_t)((uint32_t)(n1 * CB) * 8u + 2u * s),
-                                        tc::idesc_f16_f32(128, n2 * CB), acc);
+                for (int i = 0; i < DG_DIG; ++i) {
+                    // digit i of A against B digits 0 .. 4 - i, into accumulators i .. 4 (digit
+                    // 0 first: at the block's first K step it initialises every accumulator)
+                    const int nblk = OT_ORD - i;
+                    const uint64_t ad = tc::desc_sw128(abase + (uint32_t)i * OT_AKB + 32u * s);
+                    for (int j0 = 0; j0 < nblk; j0 += maxblk) {
+                        const int nb = min(maxblk, nblk - j0);
+                        const uint64_t bd = tc::desc_sw128(bbase + (uint32_t)(j0 * CB) * 128u + 32u * s);
+                        const uint32_t acc = (kb == 0 && s == 0 && i == 0) ? 0u : 1u;
+                        tc::mma_f16(taddr + (uint32_t)((i + j0) * CB), ad, bd, tc::idesc_f16_f32(128, nb * CB), acc);
                     }
                 }
-                tc::mma_commit(&mma_bar);
             }
-            __syncwarp();
+            tc::mma_commit(&mma_bar);
         }
         ++issued;
     }

@@ -34,6 +34,7 @@ def _report(name, tmp_path):
 @pytest.mark.parametrize("source,kernel,registers", [
     ("trial_df.cu", "chebyshev_expm_df_kernel", 48),        # five blocks of 256 threads
     ("trial_df.cu", "chebyshev_expm_df_list_kernel", 64),   # four, nothing spilled
+    ("overlap_tc.cu", "overlap_tc_kernel", 64),
 ])
 def test_registers_and_no_spills(source, kernel, registers, tmp_path):
     found = [v for k, v in _report(source, tmp_path).items() if kernel in k]
