@@ -539,7 +539,7 @@ static cudaError_t form_S(afqmc_ctx* ctx, const double* X, long long M) {
     if (s_in_df(ctx)) return gemm_df(ctx->stream, (int)M, (int)NN, d.K, X, w.Udf, w.Sprop, w.xdf);
     // in fixed point where the series runs on its Lanczos interval; on Gershgorin's (S beyond shared
     // memory) the series magnifies the rounding of S by e^(its excess), so S stays as it was there
-    if (w.uexp && d.K == d.KU && trial_orbitals_df_supported(d.N, d.nu) && gemm_fix_supported(NN, d.K))
+    if (w.uexp && d.K == d.KU && trial_orbitals_df_supported(d.N, d.nu) && gemm_fix_supported(d.K))
         return gemm_fix(ctx->stream, (int)M, NN, d.K, X, w.U, w.uexp, w.Sprop);
     gemm_nn_f64(ctx->stream, (int)M, (int)NN, d.K, 1.0, X, d.K, w.U, NN, 0.0, w.Sprop, NN);
     return cudaGetLastError();
@@ -879,7 +879,7 @@ static afqmc_status step_rest(afqmc_ctx* ctx) {
         CK(fields(s, d, p, w.counters, w.vbar, w.sumS, w.weight, w.alive, (double*)w.y, w.logshift));
         if (w.expTdf) {   // mixed precision: field planes and propagation in double-float
             CK(gemm_df(s, 2 * d.W, d.N * d.N, d.G, (const double*)w.y, w.Ldf, w.Aplanes, w.xdf));
-        } else if (w.lexp && gemm_fix_supported((long long)d.N * d.N, d.G)) {
+        } else if (w.lexp && gemm_fix_supported(d.G)) {
             CK(gemm_fix(s, 2 * d.W, (long long)d.N * d.N, d.G, (const double*)w.y, w.L, w.lexp, w.Aplanes));
         } else {
             gemm_nn_f64(s, 2 * d.W, d.N * d.N, d.G, 1.0, (const double*)w.y, d.G, w.L, (long long)d.N * d.N, 0.0,

@@ -137,10 +137,10 @@ __global__ void __launch_bounds__(256) gemm_fix_kernel(int M, long long Nc, int 
 
 }  // namespace
 
-// By the sizes of U alone: a row's arithmetic does not depend on how many rows a call holds, so blocks of
-// walkers and parts of a batch give the bits of the whole.  Below 12 orbitals there is little to gain (8 orbitals and
-// variables: 16384 rows 39 -> 23 us, but 4.2 -> 6.2 up to 256); at 12 it is 107 -> 53 and 4.2 -> 6.2.
-bool gemm_fix_supported(long long Nc, int K) { return K >= 1 && K <= 4096 && Nc >= 144; }
+// By the length of the sums alone: a row's arithmetic does not depend on how many rows a call holds, so blocks of
+// walkers and parts of a batch give the bits of the whole.  A few rows of the smallest systems lose 2 us to the second
+// pass over them (8 orbitals and variables, up to 256 rows: 4.2 us in FP64, 6.2 here), 16384 rows gain (39 -> 23).
+bool gemm_fix_supported(int K) { return K >= 1 && K <= 4096; }
 
 cudaError_t gemm_fix_prepare(cudaStream_t s, int K, long long Nc, const double* U, int* uexp) {
     if (Nc <= 0 || K <= 0) return cudaSuccess;
@@ -150,8 +150,8 @@ cudaError_t gemm_fix_prepare(cudaStream_t s, int K, long long Nc, const double* 
 }
 
 cudaError_t gemm_fix(cudaStream_t s, int M, long long Nc, int K, const double* X, const double* U, const int* uexp, double* C) {
-    if (!gemm_fix_supported(Nc, K)) return cudaErrorInvalidValue;
-    if (M <= 0) return cudaSuccess;
+    if (!gemm_fix_supported(K)) return cudaErrorInvalidValue;
+    if (M <= 0 || Nc <= 0) return cudaSuccess;
     int lg = 0;
     while ((1 << lg) < K) ++lg;
     const int b = std::min(58, 62 - lg), bx = b / 2, bu = b - bx;

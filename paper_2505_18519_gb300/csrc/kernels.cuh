@@ -21,7 +21,7 @@ void gemm_nn_f64(cudaStream_t s, int M, int Nc, int K, double alpha, const doubl
                  long long ldb, double beta, double* C, long long ldc);
 // gemm_fix.cu: C[M x Nc] = X[M x K] U[K x Nc] of FP64 accuracy in fixed point, row-major with
 // no padding; uexp: Nc column exponents of U from gemm_fix_prepare.
-bool gemm_fix_supported(long long Nc, int K);
+bool gemm_fix_supported(int K);
 cudaError_t gemm_fix_prepare(cudaStream_t s, int K, long long Nc, const double* U, int* uexp);
 cudaError_t gemm_fix(cudaStream_t s, int M, long long Nc, int K, const double* X, const double* U, const int* uexp, double* C);
 enum OverlapOutput { OVL_THETA = 0, OVL_TRIAL = 1, OVL_INVERSE = 2 };
