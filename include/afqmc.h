@@ -154,7 +154,7 @@ typedef struct {
                            4 warps' shares of Theta (N x (n_up + n_dn) complex) and one matrix (N x n_up) in
                            220 KB of shared memory, and the refresh N^2 + 8 N n_up doubles in 200 KB (with
                            10 + 10 electrons N <= 124; not 120 orbitals with 24 + 24).  Where the digit
-                           products are faster (above 8 orbitals, see afqmc_fp64_digits), the
+                           products are faster (above 5 orbitals, see afqmc_fp64_digits), the
                            measurement runs those and the space stays unread.  0 (default): off */
     int64_t wait_polls; /* tensor-core kernels: polls of an mbarrier before a main wait (a copy landing,
                            MMAs completing, an epilogue freeing a buffer) gives up; the block then sets

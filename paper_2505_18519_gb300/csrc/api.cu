@@ -232,12 +232,13 @@ extern "C" void afqmc_config_default(afqmc_config* c) {
 // rcache = 1: whether the measurement reads cached half-rotated matrices.  The digit-product
 // contraction, which has nothing to cache, is faster than reading them: 50 orbitals, 128 x 32
 // pairs 5.2 ms against 54 with 10 + 10 electrons, 256 x 32 pairs 1.5 against 15 with 1 + 1; 120
-// orbitals, 64 x 32 pairs with 2 + 2 1.6 against 35; 16 orbitals, 512 x 16 pairs 0.70 against 1.96.  Only the
-// smallest systems' contractions are too short for its launches (8 orbitals, 64 x 16
-// pairs, 32 matrices: 0.156 ms against 0.136 with 4 + 4 electrons, 0.151 against 0.130 with 1 + 1).
+// orbitals, 64 x 32 pairs with 2 + 2 1.6 against 35.  Whole steps (us, digits against cache), 4 x 1, 64 x 16 and 512 x 16
+// pairs: 8 orbitals, 3 + 2 electrons 277 / 293, 387 / 386, 1389 / 1637; 6 and 2 + 2 246 / 256, 342 / 323, 1160 / 1281; 4
+// and 2 + 2 230 / 209, 306 / 268, 1003 / 990; 2 and 1 + 1 209 / 176, 267 / 227, 840 / 752: up to 5 orbitals a
+// contraction is too short for its launches.
 // By the system's sizes alone: blocks of walkers run the arithmetic of the whole.
 static bool cache_read(const afqmc_config* c) {
-    return c->rcache && (c->N <= 8 || !contract_fp64d_supported(c->N, c->n_up, c->n_dn, c->n_chol, c->n_walkers, c->n_paths));
+    return c->rcache && (c->N <= 5 || !contract_fp64d_supported(c->N, c->n_up, c->n_dn, c->n_chol, c->n_walkers, c->n_paths));
 }
 
 // The tensor-core contraction's pairs with the largest error get recomputed in

@@ -50,7 +50,8 @@ def _blocks(spec, W, blocks, P, steps=2, **kw):
     (ai.SystemSpec(50, 10, 10, 250, 50, True, 90), 128, [64, 64], 4, {}),             # field planes of 256 and 128 rows
     (ai.SystemSpec(50, 10, 10, 60, 50, True, 91), 40, [3, 37], 16, {}),               # S of 640, 48 and 592 rows
     (ai.SystemSpec(8, 4, 4, 32, 8, False, 92), 700, [1, 699], 16, {}),                # the smallest system
-    (ai.SystemSpec(8, 2, 2, 32, 8, False, 93), 600, [10, 590], 16, dict(rcache=True)),  # the cached form's
+    (ai.SystemSpec(8, 2, 2, 32, 8, False, 93), 600, [10, 590], 16, dict(rcache=True)),  # ... with the cache allowed
+    (ai.SystemSpec(5, 2, 2, 20, 5, False, 97), 900, [10, 890], 16, dict(rcache=True)),  # the cache read
 ])
 def test_walker_blocks_of_the_fp64_path(spec, W, blocks, P, kw):
     _blocks(spec, W, blocks, P, **kw)
