@@ -1180,11 +1180,20 @@ cudaError_t fd_run(cudaStream_t st, const Dims& d, const FdShape& s, const FdWor
             FdZArgs a;
             a.n = f.n; a.G1 = s.G1; a.N8 = s.N8; a.KC = s.KC; a.ksteps = s.zsteps; a.NT = f.NT; a.nbuf = f.nbuf; a.ngrp = f.ngrp; a.GB = f.GB;
             a.NCT = f.NCT; a.P = d.P; a.PB = f.PB; a.MT = f.MT; a.S = f.S; a.T = f.T;
-            // about eight blocks per SM, of FD_RUN column tiles at least
+            // column tiles of a block: up to eight blocks per SM (tensor memory holds one at a time), of FD_RUN tiles at
+            // least, so that the waves take the least time (a block's start: a tile); a list's blocks are not known here
             const long long wm = wb * f.MT;
-            const long long runs = std::max(1LL, std::min<long long>((f.NCT + FD_RUN - 1) / FD_RUN, (8LL * sms + wm - 1) / wm));
-            a.RUN = (int)((f.NCT + runs - 1) / runs);
-            a.NRUN = (f.NCT + a.RUN - 1) / a.RUN;
+            const int most = (int)std::max(1LL, std::min<long long>((f.NCT + FD_RUN - 1) / FD_RUN, (8LL * sms + wm - 1) / wm));
+            long long best = 0;
+            for (int runs = list.count ? most : 1; runs <= most; ++runs) {
+                const int run = (f.NCT + runs - 1) / runs, n = (f.NCT + run - 1) / run;
+                const long long cost = (wm * n + sms - 1) / sms * (run + 1);
+                if (best == 0 || cost < best) {
+                    best = cost;
+                    a.RUN = run;
+                    a.NRUN = n;
+                }
+            }
             a.Bimg = w.aimg[q]; a.bexp = w.bexp[q]; a.bsh = w.bsh[q]; a.bad = w.bad; a.xexp = w.xexp;
             a.Y = w.y[q]; a.ymax = w.ymax + (size_t)q * s.G1;
             a.vpart = w.vpart[q]; a.xpart = w.xpart[q]; a.status = status;
