@@ -303,14 +303,15 @@ __global__ void __launch_bounds__(256) fd_phi_image_kernel(int N, int nt, int KC
     constexpr int D = Dg64<BITS>::D;
     __shared__ unsigned long long smax[4][64];
     __shared__ int se[64];
-    const long long C0 = (long long)blockIdx.x * 64, cols = wb * nt;
+    const int C0 = blockIdx.x * 64, cols = (int)wb * nt;               // fd_shape keeps them in 32 bits
     const int tid = threadIdx.x;
     {
         const int q = tid & 63, part = tid >> 6;
-        const long long C = C0 + q, w = C / nt;
+        const int C = C0 + q;
         unsigned long long m = 0;
         if (C < cols) {
-            const double2* ph = phi + (w0 + w) * (long long)N * nt + C % nt;
+            const double2* ph = phi + (w0 + C / nt) * (long long)N * nt + C % nt;
+#pragma unroll 4
             for (int i = part; i < N; i += 4) {
                 const double2 v = ph[(long long)i * nt];
                 m = max(m, max(fd_abs_bits(v.x), fd_abs_bits(v.y)));
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(256) fd_phi_image_kernel(int N, int nt, int KC
         const bool inf = m >= FD_INF_BITS;
         const int e = inf ? DG64_NAN : dg64_exp<BITS>(__longlong_as_double((long long)m));
         se[tid] = e;
-        const long long C = C0 + tid;
+        const int C = C0 + tid;
         if (C < cols) {
             cexp[C] = inf ? 0 : e;
             if (inf) bad[C / nt] = 1;
@@ -335,7 +336,7 @@ __global__ void __launch_bounds__(256) fd_phi_image_kernel(int N, int nt, int KC
     for (int e = tid; e < KCX * 128 * 8; e += 256) {
         const int r = e & 127, u = (e >> 7) & 7, c = e >> 10;
         long long F[8];
-        const long long C = C0 + (r >> 1);
+        const int C = C0 + (r >> 1);
         const bool ok = C < cols;
         const int pe = ok ? se[r >> 1] : 0;
         const double2* ph = phi + (w0 + C / nt) * (long long)N * nt + C % nt;
@@ -504,7 +505,7 @@ __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt
     extern __shared__ double2 sB[];                                    // column q (pair q / n, a = q % n) at q NS
     __shared__ unsigned long long smax[64];
     __shared__ double sl1[64];
-    __shared__ int se[64], sce[64];
+    __shared__ int se[64], sce[64], scol[64];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long wl = blockIdx.x / MT;
     const int m = blockIdx.x % MT;
@@ -547,30 +548,31 @@ __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt
         }
     }
     __syncthreads();
-    if (tid < np) {
-        bool bad = false;
+    if (tid < np * n)      // the column's exponent in the walker's units; zero columns above, non-finite ones below all
+        scol[tid] = smax[tid] == 0 ? INT_MAX
+                    : smax[tid] >= FD_INF_BITS ? DG64_NAN
+                    : dg64_exp<BITS>(__longlong_as_double((long long)smax[tid])) + sce[tid % n];
+    __syncthreads();
+    if (tid < np * n) {
+        const int p = tid / n;
         int e = INT_MAX;
-        for (int a = 0; a < n; ++a) {
-            const unsigned long long m = smax[tid * n + a];
-            bad |= m >= FD_INF_BITS;
-            if (m > 0 && m < FD_INF_BITS) e = min(e, dg64_exp<BITS>(__longlong_as_double((long long)m)) + sce[a]);
-        }
+        for (int a = 0; a < n; ++a) e = min(e, scol[p * n + a]);
         if (e == INT_MAX) e = 0;
-        if (bad) e = DG64_NAN;
-        se[tid] = e;
-        int sh = 0;
-        if (!bad) {
-            // |Z'| <= b0 2^54 before the shift, b0 the largest sum of a column's integers over 2^(TOT - 1)
-            double b0 = 0.0;
-            for (int a = 0; a < n; ++a) {
-                const double m = __longlong_as_double((long long)smax[tid * n + a]);
-                if (m > 0.0)
-                    b0 = fmax(b0, fmin(sl1[tid * n + a] / m, 2.0 * N) * ldexp(m, e - sce[a] - (Dg64<BITS>::TOT - 1)));
-            }
-            if (b0 > 0.0) sh = max(0, ilogb(b0 * (1.0 + 1e-9)) + 1 + 54 - zbits);
-        }
-        bexp[lp0 + tid] = e;
-        bsh[lp0 + tid] = sh;
+        // the column's integers added up, over 2^(TOT - 1)
+        const double m = __longlong_as_double((long long)smax[tid]);
+        double b0 = 0.0;
+        if (e != DG64_NAN && m > 0.0)
+            b0 = fmin(sl1[tid] / m, 2.0 * N) * ldexp(m, e - sce[tid % n] - (Dg64<BITS>::TOT - 1));
+        sl1[tid] = b0;
+        if (tid == p * n) se[p] = e;
+    }
+    __syncthreads();
+    if (tid < np) {
+        // |Z'| <= b0 2^54 before the shift, b0 the largest of the pair's columns
+        double b0 = 0.0;
+        for (int a = 0; a < n; ++a) b0 = fmax(b0, sl1[tid * n + a]);
+        bexp[lp0 + tid] = se[tid];
+        bsh[lp0 + tid] = b0 > 0.0 ? max(0, ilogb(b0 * (1.0 + 1e-9)) + 1 + 54 - zbits) : 0;
     }
     __syncthreads();
     uint8_t* base = out + (size_t)blockIdx.x * KC * D * FD_ADIG;
