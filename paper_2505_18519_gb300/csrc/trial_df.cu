@@ -289,13 +289,14 @@ __global__ void __launch_bounds__(256) chebyshev_expm_df_list_kernel(int N, int 
 // the other pipes' work beside them), and every
 // quantity of the recurrence is bounded: t = (S - c) / rho has norm about 1 and the
 // columns of V_k = T_k(t) Phi0 do not outgrow those of Phi0.  So t is held in units of
-// 2^-54, column a of V in units of 2^(b_a - 58) with 2^b_a >= 1.25 of its norm, and the
+// 2^-58, column a of V in units of 2^(b_a - 58) with 2^b_a >= 1.25 of its norm, and the
 // coefficients in units of 2^-58 of a power of two above their sum, each value as
 // h 2^28 + l (|l| <= 2^27).  A product is h h' 2^56 + (h l' + l h') 2^28, three integer
-// multiply-adds (the dropped l l' are below a rounding of an FP64 sum of the same length: 2^-58
-// of the column's bound per term, of either sign), and
+// multiply-adds (the dropped l l': 2^-62 of the column's bound per term, of either sign), and
 //     V_k = 2 t V_(k-1) - V_(k-2)
-// takes no FP64 arithmetic at all.  Rounding: 2^-59 of the column's bound per term.
+// takes no FP64 arithmetic at all.  Rounding: 2^-59 of the column's bound per term, and of t at 2^-59, the same in
+// every term: rounded at 2^-55 it was what the result's error came from at 120 orbitals (8.7e-16 of the norm, now 3.4e-16,
+// against FP64's 4.9e-16).
 //
 // What bounds it: that pipe, 3 C multiply-adds per thread and column of S beside the shared-memory
 // reads of S and of C entries of V.  A thread owns one row and C columns of V (consecutive threads
@@ -307,8 +308,9 @@ __global__ void __launch_bounds__(256) chebyshev_expm_df_list_kernel(int N, int 
 // The interval's estimate may miss part of the spectrum.  V is checked after every step, in 64 bits: an
 // entry beyond its column's bound (FX_LIMIT, one unit) or a norm above its limit ends the attempt.  Until then no
 // step overflows: Gershgorin's bound lies within FX_GROW half-widths, so the rows of t have
-// absolute sums of at most FX_GROW, and |2 t V_(k-1) - V_(k-2)| <= 13 units < 2^62; the sums of
-// t's low halves stay below 2^27 2^30 sqrt(N) ||V||, with the norm's limit (below 63^2 / N) less than 2^63.
+// absolute sums of at most FX_GROW: the sums of the high halves stay below 6 2^60, |2 t V_(k-1) - V_(k-2)| below 13
+// units (2^62), and the sums of the cross products below 6 2^57 + 2^27 2^30 sqrt(N) ||V||, with the norm's limit
+// (57^2 / N) less than 2^63.  An entry of t beyond 2, which would not fit, ends the attempt too.
 // Problems outside that, and non-finite or extreme values, take the FP64 recurrence.
 struct ChebShared {
     double coef[CHEB_DF_MAX + 2];
@@ -328,6 +330,7 @@ __device__ __noinline__ void cheb_fp64_problem(ChebShared& sh, long long prob, i
 
 constexpr double FX_GROW = 6.0;
 constexpr long long FX_LIMIT = 1ll << 58;   // largest entry of V: its column's bound
+constexpr long long FX_TMAX = (1ll << 59) - (1ll << 28);   // of t: 2, its high part 32 bits
 
 __device__ __forceinline__ int2 fx_split(long long v) {
     const int l = ((int)v << 4) >> 4;
@@ -378,8 +381,8 @@ __global__ void __launch_bounds__(512) chebyshev_expm_fix_kernel(int N, int nu, 
         const float f = ldexpf((float)Phi0[e], -colb[e % nu]);
         ps = fmaf(f, f, ps);
     }
-    // 1.25 of the norm of Phi0, columns scaled (0.8 at most each: the second limit is above that norm by itself)
-    const float grow_limit = fminf(1.5625f * block_sum_f(ps, sh.sc.red8) + 1e-6f, 3969.f / (float)N);
+    // 1.25 of the norm of Phi0, columns scaled (0.8 at most each, 0.5 for normalised ones: the second limit is above it)
+    const float grow_limit = fminf(1.5625f * block_sum_f(ps, sh.sc.red8) + 1e-6f, 3249.f / (float)N);
 
     for (int attempt = 0; attempt < 2; ++attempt) {
         const double c = attempt == 0 ? sh.sc.est_c : sh.sc.gers_c, rho = attempt == 0 ? sh.sc.est_rho : sh.sc.gers_rho;
@@ -390,13 +393,15 @@ __global__ void __launch_bounds__(512) chebyshev_expm_fix_kernel(int N, int nu, 
             sh.nterms = cheb_coefs(c, rho, 1e-18, sh.coef, status);
             cexp = ilogb(exp(c + rho)) + 1;
         }
-        const double ir = 1.0 / rho;
+        const double ir = 0x1p58 / rho;                        // the unit's power of two: exact
+        bool big = false;
         for (int e = tid; e < N * N; e += nth) {
             const int i = e / N, j = e - i * N;
-            const double t = (i == j ? Sg[e] - c : Sg[e]) * ir;
-            T[(size_t)j * N + i] = fx_split(__double2ll_rn(t * 0x1p54));
+            const long long t = __double2ll_rn((i == j ? Sg[e] - c : Sg[e]) * ir);
+            big |= t > FX_TMAX || t < -FX_TMAX;
+            T[(size_t)j * N + i] = fx_split(t);
         }
-        __syncthreads();
+        if (__syncthreads_or(big)) continue;                   // outside Gershgorin's interval only: once
         const int m = sh.nterms, ce = cexp;
         int2* ci = reinterpret_cast<int2*>(sh.coefd);
         const double cu = ldexp(1.0, 58 - ce);
@@ -454,10 +459,10 @@ __global__ void __launch_bounds__(512) chebyshev_expm_fix_kernel(int N, int nu, 
                     const int o = i * nup + cg * C + q;
                     long long v;
                     if (k == 1) {
-                        v = h[q] * 4 + ((x[q] + (1 << 25)) >> 26);
+                        v = (h[q] + ((x[q] + (1 << 27)) >> 28) + 2) >> 2;
                     } else {
                         const int2 b = Vp[o];
-                        v = h[q] * 8 + ((x[q] + (1 << 24)) >> 25) - ((long long)b.x * (1 << 28) + b.y);
+                        v = ((h[q] + ((x[q] + (1 << 27)) >> 28) + 1) >> 1) - ((long long)b.x * (1 << 28) + b.y);
                     }
                     const int2 w = fx_split(v);
                     Vd[o] = w;
