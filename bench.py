@@ -359,15 +359,49 @@ def hbm_peak():
     return (peak, "measured copy") if peak else (6800.0, "fallback copy")
 
 
+def tensor_peak():
+    """Measured sustained BF16 rate of this GPU type (TFLOP/s; FP16 has the same nominal rate) and where it came from."""
+    path = os.path.join(ROOT, "MEASURED_PEAKS.json")
+    peak = json.load(open(path)).get("bf16_tflops_sustained") if os.path.exists(path) else None
+    if peak is None:
+        return 1700.0, "fallback sustained bf16 (fp16 nominal ratio 1)"
+    return peak, "measured bf16 sustained (fp16 nominal ratio 1)"
+
+
+def running_kernel(lib, cfg):
+    """The contraction kernel that a configuration's measurements run."""
+    return "contract_fp64d_kernel" if lib.fp64_digits(cfg) else lib.contract_kernel(cfg)
+
+
+def digit_flops(spec, W, P):
+    """FP16 operations of the FP64 contraction as integer digit products: Y = X phi (real times complex) per walker,
+    Z = B^T Y (complex) per pair, 36 products of 8-bit digits up to 64 orbitals (45 of 7-bit ones above) each."""
+    products = 36 if 2 * ((spec.N + 7) // 8 * 8) <= 128 else 45
+    y = 2 * spec.N ** 2 * (spec.n_up + spec.n_dn)
+    z = 4 * spec.N * (spec.n_up ** 2 + spec.n_dn ** 2)
+    return 2.0 * products * (spec.n_chol + 1) * W * (y + P * z)
+
+
+def fp64_roofline(lib, cfg, spec, W, P, cms):
+    """The FP64 contraction against what bounds it: executed digit products on the tensor cores, or the per-pair
+    operation count on the FP64 pipe."""
+    flops, (fpeak, fsource) = contract_flops_per_pair(spec) * W * P, fp64_peak()
+    out = {"kernel": running_kernel(lib, cfg), "ms_per_launch": cms, "unit": "TFLOP/s", "traffic": None,
+           "achieved_per_pair_count": flops / (cms / 1e3) / 1e12, "fp64_pipe": fpeak, "fp64_pipe_source": fsource}
+    if not lib.fp64_digits(cfg):
+        return dict(out, bound="alu", achieved=flops / (cms / 1e3) / 1e12, peak=fpeak, peak_source=fsource,
+                    frac=flops / (cms / 1e3) / 1e12 / fpeak, flops_per_launch=flops)
+    executed, (peak, source) = digit_flops(spec, W, P), tensor_peak()
+    return dict(out, bound="tensor", achieved=executed / (cms / 1e3) / 1e12, peak=peak, peak_source=source,
+                frac=executed / (cms / 1e3) / 1e12 / peak, flops_per_launch=executed,
+                note="achieved and frac: executed digit products of both GEMMs over the whole contraction (digits, "
+                     "epilogues and sums included); achieved_per_pair_count: the per-pair FP64 operations it stands for")
+
+
 def tensor_roofline(spec, W, P, prof, kernel):
     """Algorithmic FLOP rate of the tensor-core contraction against the
     measured sustained BF16 peak (FP16 has the same nominal rate)."""
-    peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
-        os.path.join(ROOT, "MEASURED_PEAKS.json")) else {}
-    peak = peaks.get("bf16_tflops_sustained")
-    source = "measured bf16 sustained (fp16 nominal ratio 1)"
-    if peak is None:
-        peak, source = 1700.0, "fallback sustained bf16 (fp16 nominal ratio 1)"
+    peak, source = tensor_peak()
     # the contraction of one step: for the walker-side form, the Y-image kernel and
     # the pair kernel (plus, for the per-pair form, the refinement's launches)
     steps = max(1, prof["steps"])
@@ -435,20 +469,12 @@ def run_variants(args, lib, s, spec, run, seed, rank, world, dev, ew64, hist64, 
         hist64 = ctx.history(warmup + steps)
         ctx.close()
         cms = prof["ms"]["contract"] / max(1, prof["steps"])
-        flops_pp = contract_flops_per_pair(spec) * W * P
-        peak, psrc = fp64_peak()
         out["fp64_medium"] = {
             "precision": "fp64", "what": workload_desc(spec, run, MEDIUM) + "; FP64 (rcache = 1), "
             "20 burn-in sweeps",
             "value": W * P * world * steps / (ms / 1e3), "unit": UNIT, "ms_per_step": ms / steps,
             "gpu_launches": launches, "clocks": clocks,
-            "roofline": {"bound": "tensor" if lib.fp64_digits(cfg) else "alu",
-                         "kernel": "contract_fp64d_kernel" if lib.fp64_digits(cfg) else lib.contract_kernel(cfg),
-                         "ms_per_launch": cms,
-                         "achieved_per_pair_count": flops_pp / (cms / 1e3) / 1e12, "peak": peak, "peak_source": psrc,
-                         "unit": "TFLOP/s", "frac_per_pair_count": flops_pp / (cms / 1e3) / 1e12 / peak,
-                         "note": "per-pair algorithmic count against the FP64 pipe's rate; the products run on the "
-                                 "tensor cores as integer digits, or from the cache with fewer FP64 operations"},
+            "roofline": fp64_roofline(lib, cfg, spec, W, P, cms),
             "phases_ms_per_step": {k: round(v / max(1, prof["steps"]), 3) for k, v in prof["ms"].items()}}
 
     if only in (None, "mixed"):
@@ -676,8 +702,7 @@ def run_variants(args, lib, s, spec, run, seed, rank, world, dev, ew64, hist64, 
 
     if only in (None, "largest"):
         # the largest system (N = 200, 40 + 40 electrons, 1000 Cholesky vectors) in FP64 on a
-        # bounded sample: 19 walkers x 16 paths = 304 pairs, two full waves of the per-pair
-        # kernel (one block per SM), 1 warm-up and 2 timed steps
+        # bounded sample: 19 walkers x 16 paths, 1 warm-up and 2 timed steps
         spec4, run4 = ai.CONFIGS["largest_n200"]
         sy = ai.make_system(spec4)
         W4, P4, st4 = 19, run4.n_paths, 2
@@ -688,21 +713,16 @@ def run_variants(args, lib, s, spec, run, seed, rank, world, dev, ew64, hist64, 
         ctx.profile(True)
         ms, clocks, launches = _timed(ctx.step, lambda: torch.cuda.synchronize(dev), ctx.stream, st4, world, local)
         prof = ctx.profile_read()
-        kernel = lib.contract_kernel(c)
         ctx.close()
         cms = prof["ms"]["contract"] / max(1, prof["launches"]["contract"])
-        flops = contract_flops_per_pair(spec4) * W4 * P4
-        achieved = flops / (cms / 1e3) / 1e12
         out["largest_fp64_sample"] = {
             "precision": "fp64", "what": f"system of the largest workload (N = {spec4.N}, {spec4.n_up} + {spec4.n_dn} "
-            f"electrons, n_chol = {spec4.n_chol}, K = {spec4.K}), {W4} walkers x {P4} paths (304 pairs = 2 x 152 "
-            f"blocks of the per-pair kernel, Theta streamed in row slabs), 1 warm-up and {st4} timed steps",
+            f"electrons, n_chol = {spec4.n_chol}, K = {spec4.K}), {W4} walkers x {P4} paths, 1 warm-up "
+            f"and {st4} timed steps",
             "value": W4 * P4 * world * st4 / (ms / 1e3), "unit": UNIT, "ms_per_step": ms / st4,
             "full_workload_step_s_extrapolated": ms / st4 / 1e3 * (run4.n_walkers * run4.n_paths) / (W4 * P4),
             "gpu_launches": launches, "clocks": clocks,
-            "roofline": {"bound": "alu", "kernel": kernel, "achieved": achieved, "peak": fp64_peak()[0],
-                         "peak_source": fp64_peak()[1], "unit": "TFLOP/s", "frac": achieved / fp64_peak()[0],
-                         "traffic": None, "flops_per_launch": flops, "ms_per_launch": cms},
+            "roofline": fp64_roofline(lib, c, spec4, W4, P4, cms),
             "phases_ms_per_step": {k: round(v / max(1, prof["steps"]), 3) for k, v in prof["ms"].items()}}
 
     if only in (None, "largest_mixed"):
@@ -791,7 +811,7 @@ def run_variants(args, lib, s, spec, run, seed, rank, world, dev, ew64, hist64, 
             ms, clocks, launches = _timed(ctx.step, lambda: torch.cuda.synchronize(dev), ctx.stream, k, world, local)
             refined = ctx.stats()["refined_pairs"]
             res[key] = dict(ew=ew, ms=ms / k, clocks=clocks, refined0=refined0,
-                            refined_per_step=(refined - refined0) / (k + 1), kernel=lib.contract_kernel(c))
+                            refined_per_step=(refined - refined0) / (k + 1), kernel=running_kernel(lib, c))
             ctx.close()
         d = {"what": f"system of the mixed-precision workload (N = {spec2.N}, {spec2.n_up} + {spec2.n_dn} electrons, "
                      f"n_chol = {spec2.n_chol}, K = {spec2.K}), {W2} walkers x {P2} paths after 20 burn-in sweeps; "
@@ -850,7 +870,7 @@ def fp64_sample_leg(lib, s, spec, run, seed, rank, W, dev, state0, ew_mixed, loc
     ctx.step(1)
     ms, clocks, _ = _timed(ctx.step, lambda: torch.cuda.synchronize(dev), ctx.stream, 2, world, local)
     ctx.close()
-    return {"precision": "fp64", "kernel": lib.contract_kernel(cfg),
+    return {"precision": "fp64", "kernel": running_kernel(lib, cfg),
             "what": f"the plain FP64 path on the first {Ws} walkers (x{P} paths) of the same workload, from the "
                     "mixed run's initial state; 1 untimed and 2 timed steps",
             "ms_per_step_sample": ms / 2, "value_sample": Ws * P * world * 2 / (ms / 1e3),
