@@ -714,7 +714,7 @@ def run_variants(args, lib, s, spec, run, seed, rank, world, dev, ew64, hist64, 
         ms, clocks, launches = _timed(ctx.step, lambda: torch.cuda.synchronize(dev), ctx.stream, st4, world, local)
         prof = ctx.profile_read()
         ctx.close()
-        cms = prof["ms"]["contract"] / max(1, prof["launches"]["contract"])
+        cms = prof["ms"]["contract"] / max(1, prof["steps"])
         out["largest_fp64_sample"] = {
             "precision": "fp64", "what": f"system of the largest workload (N = {spec4.N}, {spec4.n_up} + {spec4.n_dn} "
             f"electrons, n_chol = {spec4.n_chol}, K = {spec4.K}), {W4} walkers x {P4} paths, 1 warm-up "

@@ -85,26 +85,23 @@ struct RefineUnits {
     }
 };
 
-// Runs per listed pair: of the numbers that fill one to six waves of `blocks` blocks with n pairs (up to 64, eight units a
-// run: shorter ones lose more to their start than they gain beside other systems' kernels),
-// the one whose waves take the least time (in units).  With 16 for
+// Runs per listed pair (up to 64, eight units each: shorter ones lose more to their start than they gain beside other
+// systems' kernels): the number whose waves of `blocks` blocks take the least time with n pairs, a run's start as half a
+// unit.  Whole warps call it, two numbers a lane.  With 16 for
 // every n, four and eight pairs of 95 and 120 orbitals left three quarters and half of the blocks
 // idle: those two 6.3 -> 2.6 ms; the 18 to 22 pairs a step of 64 x 64 pairs of 120 orbitals
 // (16 runs of 20 pairs: two waves, the second nearly empty) 5.7 -> 4.1.
-__device__ __forceinline__ int split_count(long long n, long long blocks, int units) {
-    if (n <= 0 || n > REFINE_SPLIT) return 1;
-    const long long most = max(min(units, 16), min(64, units / 8));
-    long long best = 1, time = (n + blocks - 1) / blocks * units;
-    for (int k = 1; k <= 6; ++k) {
-        const long long g = min(k * blocks / n, most);
-        if (g < 1) continue;
-        const long long t = (n * g + blocks - 1) / blocks * ((units + g - 1) / g);
-        if (t < time) {
-            best = g;
-            time = t;
-        }
+__device__ __forceinline__ int split_count(long long n_list, int blocks, int units) {
+    if (n_list <= 0 || n_list > REFINE_SPLIT) return 1;
+    const int n = (int)n_list, most = max(min(units, 16), min(64, units / 8));
+    unsigned best = 0xffffffffu;                               // time, then the number
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int g = (threadIdx.x & 31) + 32 * q + 1;
+        const int waves = (n * g + blocks - 1) / blocks, time = waves * (2 * ((units + g - 1) / g) + 1);
+        if (g <= most) best = min(best, (unsigned)time << 7 | (unsigned)g);
     }
-    return (int)best;
+    return (int)(__reduce_min_sync(0xffffffffu, best) & 127u);
 }
 
 template <bool SLAB, bool DF, int OWN>
@@ -346,7 +343,7 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
 
 // E_L of the listed pairs from their units' sums: a warp per pair, a lane per group, the groups in order.
 __global__ void refine_sum_kernel(const int* __restrict__ items, const int* __restrict__ n_items,
-                                  const double2* __restrict__ epart, long long blocks, RefineUnits ru, double2* __restrict__ epair) {
+                                  const double2* __restrict__ epart, int blocks, RefineUnits ru, double2* __restrict__ epair) {
     const long long n = *n_items;
     if (split_count(n, blocks, ru.units) == 1) return;      // summed already
     const int lane = threadIdx.x & 31, u0 = ru.group * lane, u1 = min(ru.units, u0 + ru.group);
@@ -633,7 +630,7 @@ static cudaError_t launch_fp64_shape(cudaStream_t s, const Dims& d, int JB, size
                                                                            epart);
     count_launches(1);
     if (epart) {
-        refine_sum_kernel<<<64, 256, 0, s>>>(items, n_items, epart, blocks, RefineUnits(d.G + 1), epair);
+        refine_sum_kernel<<<64, 256, 0, s>>>(items, n_items, epart, (int)blocks, RefineUnits(d.G + 1), epair);
         count_launches(1);
     }
     return cudaGetLastError();
