@@ -365,7 +365,8 @@ int64_t afqmc_launch_count(void);
  * FP64 the value names the FP64 arithmetic's kernel of these sizes
  * (0, 3, 4 or 6); where afqmc_fp64_digits says so, contract_fp64d_kernel runs in its
  * place: the walker-side form B_p^T (X_g phi_w) on the tensor cores, every product
- * as exact sums of integer digits, no less accurate than FP64 sums. */
+ * as exact sums of integer digits, no less accurate than FP64 sums (the entries of one h or L_g
+ * share an exponent: what lies below 2^-62 of its largest entry is dropped). */
 int afqmc_contract_kernel(const afqmc_config* cfg);
 /* 1 if the FP64 contraction of `cfg` runs on the tensor cores as integer digit
  * products (N <= 224 and up to about 60 electrons per spin, 48 above 64 orbitals;

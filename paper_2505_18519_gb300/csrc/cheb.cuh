@@ -80,7 +80,7 @@ struct ChebScratch {
 
 // Both intervals of the symmetric N x N matrix S held in shared memory as FP32
 // values S32[(i N + j) stride] (stride 2 reads the high parts of double-float
-// pairs).  256 or 512 threads; ends with a barrier, after which every thread
+// pairs).  128, 256 or 512 threads; ends with a barrier, after which every thread
 // may read the results in sc.
 __device__ __forceinline__ void cheb_interval(int N, const float* S32, int stride, ChebScratch& sc) {
     const int tid = threadIdx.x, nth = blockDim.x;

@@ -32,7 +32,7 @@
 // way in (the A digits of a tile of pairs, 0.25 MB at 50 orbitals, pass once per column
 // tile); then the epilogue's 64-bit integer arithmetic, about 30 instructions per entry.
 // Measured on one GB300, whole contraction against the FP64 kernels it replaces:
-// 50 orbitals, 512 x 32 pairs 19.4 ms against 265 (contract_fp64z_kernel, 0.98 of the FP64
+// 50 orbitals, 512 x 32 pairs 18.4 ms against 265 (contract_fp64z_kernel, 0.98 of the FP64
 // pipe); 120 orbitals, 8 x 64 pairs 18 ms against 458 (contract_fp64_kernel); 37 orbitals,
 // 24 x 9 pairs 0.18 ms against 1.07; 8 orbitals, 64 x 16 pairs 0.15 ms against 0.40: faster
 // at every size it takes, so it takes all of those (fd_shape).  With a list of pairs (the mixed path's
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(FDY_THREADS, 1)
 // largest N) and forms exponents and digits from there: read from global memory column by
 // column, the loads' latency bound it, and the
 // FP64 pipe by the maxima's comparisons, integer ones now (48 blocks of 200 orbitals and 40 electrons 110 us,
-// staged 75; 64 blocks of 8 and 4 20 us staged, now 16).
+// staged 75, with a thread per column for the exponents 67; 64 blocks of 8 and 4 20, 16 and 17).
 constexpr int FDB_T = 512;
 template <int BITS>
 __global__ void __launch_bounds__(FDB_T) fd_b_image_kernel(int N, int N8, int nt, int col0, int n, int P, int PB, int MT,

@@ -1,7 +1,7 @@
 // C = X U for the FP64 path's sums over hidden variables and auxiliary fields
 // (S_p = sum_k x_pk U_k, the field planes sum_g y_wg L_g) in fixed point: 32-bit
-// integer multiply-adds with 64-bit sums, which issue at eight times the rate
-// of FP64 ones here (16 against 2 per clock and SM), three to a product.
+// integer multiply-adds with 64-bit sums, which issue at some eight times the rate
+// of FP64 ones here (15 against 2 per clock and SM measured), three to a product.
 //
 // A row of X and a column of U (one entry of every matrix) each share an exponent, so an
 // element keeps the digits that matter to its own sum.  Values become
