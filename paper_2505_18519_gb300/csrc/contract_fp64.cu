@@ -73,27 +73,27 @@ __host__ __device__ __forceinline__ Fp64Layout fp64_layout(int N, int nu, int nd
 // OWN: M entries owned per thread (n_up^2 + n_dn^2 <= OWN * CT); the double-float
 // mode with OWN = 8 fits two blocks per SM (slab layout, at most 128 registers;
 // the FP64 instances keep the same 128-register budget).
-// The split double-float refinement: the matrices of a listed pair make units (one matrix each up to 512), the
+// The split double-float refinement: the matrices of a listed pair make units (one matrix each up to 1024), the
 // units up to 32 groups; a unit's terms, the units of a group and the groups are added in order, and a run (one block)
 // takes whole units, so that E_L does not depend on how many other pairs are listed.
 struct RefineUnits {
     int mats, units, group;     // matrices a unit, units, units a group
     __host__ __device__ explicit RefineUnits(int G1) {
-        mats = (G1 + 511) / 512;
+        mats = (G1 + 1023) / 1024;
         units = (G1 + mats - 1) / mats;
         group = (units + 31) / 32;
     }
 };
 
-// Runs per listed pair (up to 64, eight units each: shorter ones lose more to their start than they gain beside other
+// Runs per listed pair (up to 64, eight matrices each: shorter ones lose more to their start than they gain beside other
 // systems' kernels): the number whose waves of `blocks` blocks take the least time with n pairs, a run's start as half a
 // unit.  Whole warps call it, two numbers a lane.  With 16 for
 // every n, four and eight pairs of 95 and 120 orbitals left three quarters and half of the blocks
 // idle: those two 6.3 -> 2.6 ms; the 18 to 22 pairs a step of 64 x 64 pairs of 120 orbitals
 // (16 runs of 20 pairs: two waves, the second nearly empty) 5.7 -> 4.1.
-__device__ __forceinline__ int split_count(long long n_list, int blocks, int units) {
+__device__ __forceinline__ int split_count(long long n_list, int blocks, RefineUnits ru) {
     if (n_list <= 0 || n_list > REFINE_SPLIT) return 1;
-    const int n = (int)n_list, most = max(min(units, 16), min(64, units / 8));
+    const int n = (int)n_list, units = ru.units, most = max(min(units, 16), min(64, units * ru.mats / 8));
     unsigned best = 0xffffffffu;                               // time, then the number
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
     // item each, so that a few listed pairs still fill the GPU
     const long long n_list = items ? (long long)*n_items : (long long)gridDim.x;
     const RefineUnits ru(G + 1);
-    const int gs = DF && epart ? split_count(n_list, gridDim.x, ru.units) : 1;
+    const int gs = DF && epart ? split_count(n_list, gridDim.x, ru) : 1;
     const long long n_work = n_list * gs;
     for (long long item = blockIdx.x; item < n_work; item += gridDim.x) {
     const long long pair = items ? (long long)items[item / gs] : item;
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(CT, (DF && OWN > 8) ? 1 : 2) contract_fp64_ker
 __global__ void refine_sum_kernel(const int* __restrict__ items, const int* __restrict__ n_items,
                                   const double2* __restrict__ epart, int blocks, RefineUnits ru, double2* __restrict__ epair) {
     const long long n = *n_items;
-    if (split_count(n, blocks, ru.units) == 1) return;      // summed already
+    if (split_count(n, blocks, ru) == 1) return;      // summed already
     const int lane = threadIdx.x & 31, u0 = ru.group * lane, u1 = min(ru.units, u0 + ru.group);
     const long long warps = (long long)gridDim.x * blockDim.x / 32;
     for (long long it = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32; it < n; it += warps) {
