@@ -854,6 +854,8 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
         const int2* R0 = Mg + (size_t)(mine ? pl * n : 0) * ldc + (mine ? gl * n : 0);
         const int2* I0 = R0 + (size_t)64 * ldc;
         const int px = mine ? min(FD_XTRA, sbsh[pl]) : 0, prx = px > 0 ? 1 << (px - 1) : 0;
+        // the stored 2^(x - 1) of a thread's diagonal entries, taken off their sum: a low half may be at the end of 32 bits
+        const long long bias = mine && sub < n ? (long long)prx * ((n - sub + T - 1) / T) : 0;
         for (int t = t0 + grp; t < t1; t += A.ngrp) {
             const int tt = t - t0;
             const uint32_t tbuf = nbuf == 2 && (tt & 1) ? (uint32_t)fd_cols(D, NT) : 0u;
@@ -898,8 +900,8 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
                     if (u < n) {
                         th += xr.x;
                         uh += xi.x;
-                        tl += (long long)xr.y - prx;      // a low half may be at the end of 32 bits
-                        ul += (long long)xi.y - prx;
+                        tl += xr.y;
+                        ul += xi.y;
                     }
                     xr.y >>= px; xi.y >>= px; yr.y >>= px; yi.y >>= px;
                     if (u >= n) {
@@ -919,8 +921,8 @@ __global__ void __launch_bounds__(FDZ_THREADS, 1) contract_fp64d_kernel(const __
             FdRed s;
             s.th = th;
             s.uh = uh;
-            s.tl = tl;
-            s.ul = ul;
+            s.tl = tl - bias;
+            s.ul = ul - bias;
             fd_join(hr, mr, lr, s.rh, s.rl);
             fd_join(hm, mm, lm, s.ih, s.il);
             for (int o = min(T, 32) >> 1; o > 0; o >>= 1) {
