@@ -15,8 +15,8 @@
 // What bounds it: that pipe (15 multiply-adds per clock and SM), 3 R^2 of them a thread and k for
 // 2 R shared-memory reads; few rows, whose tiles of 64 x 64 leave SMs idle, take smaller ones (the sums are
 // integers: the same for every tile).  Against the FP64 GEMM (0.8 of the FP64 pipe) on one GB300:
-// S of 16384 paths, 50 orbitals and variables 4.41 -> 1.41 ms, of 4096 1.11 -> 0.37; the planes of
-// 512 walkers, 250 fields 1.30 -> 0.43.
+// S of 16384 paths, 50 orbitals and variables 4.42 -> 1.27 ms, of 4096 1.11 -> 0.33; the planes of
+// 512 walkers, 250 fields 1.30 -> 0.37.
 #include <algorithm>
 
 #include "digits64.cuh"
@@ -60,6 +60,19 @@ __global__ void __launch_bounds__(256) gemm_fix_kernel(int M, long long Nc, int 
     __shared__ int xe[T], ue[T];
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
     const long long row0 = (long long)blockIdx.y * T, col0 = (long long)blockIdx.x * T;
+    // a k tile's values, one R-th of X's and U's each; small tiles load the next one ahead, the first beside the exponents
+    double xv[R], uv[R];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const int e = tid + q * 256;
+            const int r = e / GF_K, kk = e % GF_K;              // X tile: T rows x 16 k
+            const int kb = e / T, c = e % T;                    // U tile: 16 k x T columns
+            xv[q] = row0 + r < M && k0 + kk < K ? X[(row0 + r) * K + k0 + kk] : 0.0;
+            uv[q] = col0 + c < Nc && k0 + kb < K ? U[(long long)(k0 + kb) * Nc + col0 + c] : 0.0;
+        }
+    };
+    if (R < 4) load(0);
     {   // exponents of the tile's rows: TPR threads a row
         const long long r = row0 + tid / TPR;
         double m = 0.0;
@@ -81,17 +94,15 @@ __global__ void __launch_bounds__(256) gemm_fix_kernel(int M, long long Nc, int 
     __syncthreads();
     long long h[R][R] = {}, x[R][R] = {};
     for (int k0 = 0; k0 < K; k0 += GF_K) {
+        if (R == 4) load(k0);
 #pragma unroll
         for (int q = 0; q < R; ++q) {
             const int e = tid + q * 256;
-            const int r = e / GF_K, kk = e % GF_K;              // X tile: T rows x 16 k
-            const long long gr = row0 + r;
-            Xs[kk][r] = gr < M && k0 + kk < K ? gf_split(X[gr * K + k0 + kk], 28 + bx - xe[r]) : make_int2(0, 0);
-            const int kb = e / T, c = e % T;              // U tile: 16 k x T columns
-            const long long gc = col0 + c;
-            Us[kb][c] = gc < Nc && k0 + kb < K ? gf_split(U[(long long)(k0 + kb) * Nc + gc], 28 + bu - ue[c]) : make_int2(0, 0);
+            Xs[e % GF_K][e / GF_K] = gf_split(xv[q], 28 + bx - xe[e / GF_K]);
+            Us[e / T][e % T] = gf_split(uv[q], 28 + bu - ue[e % T]);
         }
         __syncthreads();
+        if (R < 4 && k0 + GF_K < K) load(k0 + GF_K);
 #pragma unroll
         for (int kk = 0; kk < GF_K; ++kk) {
             int2 a[R], b[R];
