@@ -148,8 +148,8 @@ __device__ __forceinline__ void fd_pipe_init(FdPipe& p, int S, int bfull_count, 
 // without a divergent exit.  Issued like that the pattern of MMAs runs at 90 % (NT =
 // 32) to 97 % (NT = 64) of the tensor peak; each MMA takes max(N / 2, 32 + N / 4)
 // clocks (A and B from shared memory).  After a timeout the waits return at once and
-// the rest of the loop runs on whatever shared memory holds (the block's results are
-// void then).
+// nothing is issued or handed back any more (the block's results are void then): a slot
+// whose copy has not landed must not go back to its producer, whose barrier would take an arrival too many.
 template <int BITS, int NT>
 __device__ __forceinline__ bool fd_mma_loop_nt(FdPipe& p, uint32_t taddr, const uint8_t* bslots, uint32_t bslot_bytes,
                                                const uint8_t* ring, int S, int tiles, int KC, int ksteps, int nbuf,
@@ -181,7 +181,7 @@ __device__ __forceinline__ bool fd_mma_loop_nt(FdPipe& p, uint32_t taddr, const 
                 constexpr int cap = MB;
                 const int n1 = D - i < cap ? D - i : cap, n2 = D - i - n1;
                 __syncwarp();
-                if (tc::elect_one()) {
+                if (tc::elect_one() && ok) {
 #pragma unroll
                     for (int s = 0; s < 4; ++s) {
                         if (s < ks) {

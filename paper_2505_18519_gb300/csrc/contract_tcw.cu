@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(TCW_THREADS, 1)
                     const uint64_t pa = abase + (uint64_t)((uint32_t)c * (CS >> 4));
                     const uint64_t pb = bbase + (uint64_t)((uint32_t)st * (RX >> 4));
                     __syncwarp();
-                    if (tc::elect_one()) {
+                    if (tc::elect_one() && ok) {   // a slot whose copy has not landed is not handed back
 #pragma unroll
                         for (int s = 0; s < 4; ++s) {
                             if (s >= ks) break;
@@ -706,13 +706,13 @@ __device__ __forceinline__ void tcw_z_block(const TcwZArgs& A, long long bid, ui
         // ---- MMA issue: one lane's instructions, but the whole warp runs the loop without a
         // divergent exit, so that the operands stay in the uniform registers the MMA takes them
         // from (in a branch of one lane each MMA's operands were moved there first).  After a
-        // timeout the waits return at once; the block's results are void then.
+        // timeout the waits return at once and nothing is issued or handed back; the block's results are void then.
         const uint32_t idesc = F16 ? tc::idesc_f16_f32(128, NT) : tc::idesc_bf16_f32(128, NT);
         const uint64_t abase = tc::desc_sw128(tc::smem_u32(a_res ? Ares : ring));
         const uint64_t bbase = tc::desc_sw128(tc::smem_u32(ring + (a_res ? 0 : CH)));
         const uint32_t sstep = stage_bytes >> 4, bstep = bpart >> 4;   // descriptors count 16-byte units
         bool ok = !a_res || wait_or_fail(&a_bar, 0, lim, &fail);
-        int st = 0;
+        int st = 0, committed = 0;   // units handed back (of the issuing lane)
         uint32_t ph = 0;
         for (int t = 0; t < NTILES; ++t) {
             const int b = t & 1;
@@ -726,7 +726,7 @@ __device__ __forceinline__ void tcw_z_block(const TcwZArgs& A, long long bid, ui
                 const uint64_t pb = bbase + (uint64_t)((uint32_t)st * sstep);
                 const uint32_t firstc = c == 0 ? 0u : 1u;
                 __syncwarp();
-                if (tc::elect_one()) {
+                if (tc::elect_one() && ok) {   // a slot whose copy has not landed is not handed back
 #pragma unroll
                     for (int s = 0; s < 4; ++s) {
                         if (s >= ks) break;
@@ -755,6 +755,7 @@ __device__ __forceinline__ void tcw_z_block(const TcwZArgs& A, long long bid, ui
                         }
                     }
                     tc::mma_commit(&empty_bar[st]);
+                    ++committed;
                     if (c == KC - 1) tc::mma_commit(&dfull[b]);
                 }
                 __syncwarp();
@@ -768,7 +769,8 @@ __device__ __forceinline__ void tcw_z_block(const TcwZArgs& A, long long bid, ui
         tc::mbar_wait(&drain_bar, 0, 1u << 22);
         // the ring's last hand-backs, which no producer wait consumed, have arrived
         // (the barriers may be initialised again for the block's next piece of work)
-        for (int v = max(0, n_units - S); v < n_units; ++v)
+        committed = (int)__reduce_add_sync(0xffffffffu, (unsigned)committed);
+        for (int v = max(0, committed - S); v < committed; ++v)
             tc::mbar_wait(&empty_bar[v % S], (uint32_t)((v / S) & 1), 1u << 22);
         __syncwarp();
     } else {

@@ -185,11 +185,11 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
         __syncwarp();
     } else if (warp == 1) {
         // ---- MMA issue: one lane's instructions, the loop warp-uniform without a divergent exit, so
-        // that the operands stay in uniform registers; after a timeout the waits return at once
-        // (the block's results are void then)
+        // that the operands stay in uniform registers; after a timeout the waits return at once and
+        // nothing is issued or handed back (the block's results are void then)
         const uint64_t bbase = tc::desc_sw128(tc::smem_u32(BD)), rbase = tc::desc_sw128(tc::smem_u32(ring));
         bool ok = true;
-        int st = 0;
+        int st = 0, committed = 0;   // units handed back (of the issuing lane)
         uint32_t ph = 0;
         for (int t = 0; t < NTILE; ++t) {
             const int b = t & 1;
@@ -206,12 +206,13 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
                     const uint64_t pa = rbase + (uint64_t)((uint32_t)st * (SP_TILE >> 4));
                     const uint64_t pb = bbase + (uint64_t)((uint32_t)kb * (SP_BKB >> 4));
                     __syncwarp();
-                    if (tc::elect_one()) {
+                    if (tc::elect_one() && ok) {   // a slot whose copy has not landed is not handed back
 #pragma unroll
                         for (int s = 0; s < 4; ++s)
                             tc::mma_f16(dbase + (uint32_t)(i * SP_NB), pa + 2 * s, pb + 2 * s, idesc,
                                         (i == 0 && kb == 0 && s == 0) ? 0u : 1u);
                         tc::mma_commit(&empty_bar[st]);
+                        ++committed;
                         if (i == DG_DIG - 1 && kb == KBLK - 1) tc::mma_commit(&dfull[b]);
                     }
                     __syncwarp();
@@ -224,8 +225,8 @@ __global__ void __launch_bounds__(SP_THREADS, 1)
         if (tc::elect_one()) tc::mma_commit(&drain_bar);         // every issued MMA completes before the block leaves
         __syncwarp();
         tc::mbar_wait(&drain_bar, 0, 1u << 22);
-        const int units = NTILE * DG_DIG * KBLK;
-        for (int u = max(0, units - SP_STAGES); u < units; ++u)
+        committed = (int)__reduce_add_sync(0xffffffffu, (unsigned)committed);
+        for (int u = max(0, committed - SP_STAGES); u < committed; ++u)
             tc::mbar_wait(&empty_bar[u % SP_STAGES], (uint32_t)((u / SP_STAGES) & 1), 1u << 22);
         __syncwarp();
     } else {
